@@ -273,7 +273,7 @@ struct Solver : SolverBase {
   bool clus = false;
   int cl_var = 1;                  // thread-count variant of the cluster kernel
   // compiled tile alternatives chosen by the autotuner (K2Cfg variant bits: 1 pencil width,
-  // 2 inverse-y width, 4 x rows, 8 forward-y width, 16 pencil at 64 registers; 0 = defaults)
+  // 2 inverse-y width, 8 forward-y width; 0 = defaults)
   int vsel = 0;
   int cl_ncl = -1;                 // clusters the device holds at once (-1: not yet queried)
   long long cl_spin = 1ll << 20;   // polls of its bounded TMA wait
@@ -421,24 +421,22 @@ struct Solver : SolverBase {
           throw NsError{NS_ERR_INTERNAL, "specialised tile shapes exceed the shared memory of the device"};
         CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
       };
-      allow(k2.pencil, k2.smP5);
-      allow(k2.pencil1, k2.smP1);
-      allow(k2.pencil1e, k2.smP1);
-      allow(k2.pencil1re, k2.smP1);
-      allow(k2.pencil1r[0], k2.smP1);
-      allow(k2.pencil1r[1], k2.smP1);
-      allow(k2.pencil2, k2.smP5);
+      allow(k2.pencil01, k2.smP);
+      allow(k2.pencil10, k2.smP);
+      for (auto* f : k2.pencil1)
+        if (f) allow(f, k2.smP);
+      allow(k2.pencil1e, k2.smP);
+      allow(k2.pencil1re, k2.smP);
+      allow(k2.pencil2, k2.smP);
+      allow(k2.pencil02, k2.smP);
       allow(k2.yinv, k2.smYI);
       allow(k2.yfwd, k2.smY);
       allow(k2.xrow, k2.smX);
       if (k2.has_alt) {
-        allow(k2.alt.pencil1r[0], k2.alt.smP1);
-        allow(k2.alt.pencil1r[1], k2.alt.smP1);
-        allow(k2.pencil1r64[0], k2.smP1);
-        allow(k2.pencil1r64[1], k2.smP1);
+        allow(k2.alt.pencil1r[0], k2.alt.smP);
+        allow(k2.alt.pencil1r[1], k2.alt.smP);
         allow(k2.alt.yinv, k2.alt.smYI);
         allow(k2.alt.yfwd, k2.alt.smY);
-        allow(k2.alt.xrow, k2.alt.smX);
       }
       for (int v = 0; v < 2; ++v)
         if (k2.slabcl[v]) {
@@ -537,15 +535,17 @@ struct Solver : SolverBase {
   }
 
   // ---- passes -----------------------------------------------------------------------
+  // layout of the mixed fields and of Ft (mixed_index): interleaved for the compile-time kernels,
+  // except when the cluster slab pass, whose TMA copies take one field at a time, reads them
+  int pairs() const { return use2 && !clus; }
   SlabArgs<T> slab_args() {
     SlabArgs<T> a;
     memset(&a, 0, sizeof(a));
     a.N = N; a.M = M; a.py = py; a.px = px; a.tw = tw; a.scr = scr;
     a.TY = TY; a.RX = RX; a.err = d_err;
-    // Ft modes no pencil tile reads are left unwritten (every pencil instance of this size
-    // skips the same truncated tiles; the widest tile decides)
-    if (use2 && NS_FT_SKIP) {
-      a.skip_tx = std::max(k2.TX, k2.has_alt ? k2.alt.TX : 0);
+    a.pairs = pairs();
+    if (use2) {  // Ft columns that no pencil pass uses are left unwritten
+      a.skip = 1;
       a.trunc = c->p.truncation; a.K2max = c->K2max; a.Kimax = c->Kimax;
       a.fK = fkind != NS_FORCE_NONE ? fK : -1;
     }
@@ -633,10 +633,7 @@ struct Solver : SolverBase {
     prof_end(e, s);
     e = prof_begin(NS_PROF_XROW, s);
     if (use2)
-      if (vsel & 4)
-        k2.alt.xrow<<<(a.G * N + k2.alt.RX - 1) / k2.alt.RX, k2.alt.NTX, k2.alt.smX, s>>>(a);
-      else
-        k2.xrow<<<(a.G * N + k2.RX - 1) / k2.RX, k2.NTX, k2.smX, s>>>(a);
+      k2.xrow<<<(a.G * N + k2.RX - 1) / k2.RX, k2.NTX, k2.smX, s>>>(a);
     else
       k_xrow<T><<<(a.G * N + RX - 1) / RX, bdX, smX, s>>>(a);
     prof_end(e, s);
@@ -726,6 +723,7 @@ struct Solver : SolverBase {
     a.dt = (T)cur_dt; a.ifac = ifac; a.state = state; a.acc = acc;
     a.trunc = c->p.truncation; a.K2max = c->K2max; a.Kimax = c->Kimax;
     a.err = d_err;
+    a.pairs = pairs();
     if (fkind != NS_FORCE_NONE) {
       a.shell = shell;
       a.fK = fK;
@@ -739,19 +737,13 @@ struct Solver : SolverBase {
     const int R = rows < 0 ? N : rows;
     const bool rog = a.nF == 1 && a.nOut == 1 && !a.epart && (a.mode == MODE_ROG_1 || a.mode == MODE_ROG_2);
     if (use2 && rog && (vsel & 1))  // the autotuner's alternative pencil width
-      k2.alt.pencil1r[a.mode == MODE_ROG_1 ? 0 : 1]<<<(M / k2.alt.TX) * R, k2.alt.NTP, k2.alt.smP1, st>>>(a);
-    else if (use2 && rog && (vsel & 16))  // the alternative register budget
-      k2.pencil1r64[a.mode == MODE_ROG_1 ? 0 : 1]<<<(M / k2.TX) * R, k2.NTP, k2.smP1, st>>>(a);
+      k2.alt.pencil1r[a.mode == MODE_ROG_1 ? 0 : 1]<<<(M / k2.alt.TX) * R, k2.alt.NTP, k2.alt.smP, st>>>(a);
     else if (use2)
-      (a.nF == 1 && a.nOut == 1   ? (a.epart                  ? (a.mode == MODE_ROG_2 ? k2.pencil1re : k2.pencil1e)
-                                     : a.mode == MODE_ROG_1 ? k2.pencil1r[0]
-                                     : a.mode == MODE_ROG_2 ? k2.pencil1r[1]
-                                                            : k2.pencil1)
+      (a.nF == 1 && a.nOut == 1   ? (a.epart ? (a.mode == MODE_ROG_2 ? k2.pencil1re : k2.pencil1e) : k2.pencil1[a.mode])
        : a.nF == 2 && a.nOut == 2 ? k2.pencil2
-                                  : k2.pencil)<<<(M / k2.TX) * R, k2.NTP,
-                                                  (a.nF == 1 && a.nOut == 1) ? k2.smP1
-                                                  : (a.nF > 1 || a.nOut > 1) ? k2.smP5
-                                                                             : k2.smP4, st>>>(a);
+       : a.nF == 0 && a.nOut == 2 ? k2.pencil02
+       : a.nF == 0                ? k2.pencil01
+                                  : k2.pencil10)<<<(M / k2.TX) * R, k2.NTP, k2.smP, st>>>(a);
     else
       k_pencil<T><<<(M / TX) * R, bdP, smP, st>>>(a);
     prof_end(e);
@@ -779,19 +771,13 @@ struct Solver : SolverBase {
     if (!rank_stg) CUDA_TRY(cudaMalloc(&rank_stg, 5 * F1 * cs));
     cpx<T>* d = rank_buf(which);
     const size_t count = (size_t)F * N * n * M;  // complex values of the block
-    size_t width, height, dpitch;
-    cpx<T>* base;
-    if (axis == 0) {  // F rows of n N M values, field pitch N N M
-      width = (size_t)n * N * M * cs; height = F; dpitch = F1 * cs; base = d + (size_t)lo * N * M;
-    } else {          // F N rows of n M values, row pitch N M
-      width = (size_t)n * M * cs; height = (size_t)F * N; dpitch = (size_t)N * M * cs; base = d + (size_t)lo * M;
-    }
+    const int prs = use2 && (which == NS_BUF_MIXED || which == NS_BUF_FT);
+    if (to_dev) to_device(host, reinterpret_cast<T*>(rank_stg), 2 * count);
+    k_block_copy<T><<<8 * nsm, 256, 0, st>>>(d, rank_stg, F, N, axis, lo, n, prs, to_dev);
+    LAUNCH_CHECK();
     if (to_dev) {
-      to_device(host, reinterpret_cast<T*>(rank_stg), 2 * count);
-      CUDA_TRY(cudaMemcpy2DAsync(base, dpitch, rank_stg, width, width, height, cudaMemcpyDeviceToDevice, st));
       CUDA_TRY(cudaStreamSynchronize(st));
     } else {
-      CUDA_TRY(cudaMemcpy2DAsync(rank_stg, width, base, dpitch, width, height, cudaMemcpyDeviceToDevice, st));
       to_host(reinterpret_cast<const T*>(rank_stg), host, 2 * count);
       sync_check();
     }
@@ -804,6 +790,7 @@ struct Solver : SolverBase {
     upload_shifts(sh);
     PencilArgs<T> p = pencil_args(kind == NS_RANK_INIT ? MODE_INIT : MODE_NL);
     p.shell = nullptr;
+    p.pairs = use2;  // (the rank passes run the three slab kernels, never the cluster pass)
     p.iy0 = lo;
     if (kind == NS_RANK_INIT) {
       p.src = state;
@@ -822,6 +809,7 @@ struct Solver : SolverBase {
     a.mixed = mixed[0];
     a.Ft = Ft[0];
     a.xmode = XMODE_NONLINEAR;
+    a.pairs = use2;
     for (int z0 = lo; z0 < hi; z0 += G) {
       a.z0 = z0;
       a.G = (z0 + G <= hi) ? G : hi - z0;
@@ -1123,7 +1111,7 @@ struct Solver : SolverBase {
     if (const char* e = std::getenv("NS_CL_SPIN")) cl_spin = std::max(1ll, std::atoll(e));
     // NS_TILE_VARIANT=bits forces the compiled tile alternatives (bits of K2Cfg's variant)
     const char* fv = std::getenv("NS_TILE_VARIANT");
-    if (fv && *fv) vsel = (use2 && k2.has_alt) ? (std::atoi(fv) & 31) : 0;
+    if (fv && *fv) vsel = (use2 && k2.has_alt) ? (std::atoi(fv) & 11) : 0;
     const char* fcl = std::getenv("NS_SLAB_CLUSTER");
     const bool can_cl = use2 && k2.slabcl[0] && !(fcl && std::string(fcl) == "0") && cl_clusters() > 0;
     if (fcl && std::string(fcl) == "1" && can_cl) {  // forced cluster pass (NS_CL_VARIANT 0 or 1)
@@ -1153,9 +1141,9 @@ struct Solver : SolverBase {
     if (Gmax <= 1 || N < 128) return;  // small grids: one group holds every plane
     const bool can_alt = use2 && k2.has_alt && !(fv && *fv);
     const std::string path = cache_path(),
-                      key = tune_key() + (can_pipe ? "|g4p" : "|g4") + (can_cl ? "c" + std::to_string(k2.CLS) : "") +
+                      key = tune_key() + (can_pipe ? "|g5p" : "|g5") + (can_cl ? "c" + std::to_string(k2.CLS) : "") +
                             (can_alt ? "|v" + std::to_string(k2.alt.TX) + "," + std::to_string(k2.alt.TYI) + "," +
-                                           std::to_string(k2.alt.RX) + "," + std::to_string(k2.alt.TY) + ",p64"
+                                           std::to_string(k2.alt.TY)
                                      : "");
     int g = 0;
     if (cache_lookup(path, key, &g)) {  // value = 4096 vsel + 4 G + mode
@@ -1219,7 +1207,7 @@ struct Solver : SolverBase {
       };
       if (!pipe && !clus) {
         float base = time_slab();
-        for (int bit : {2, 4, 8}) {
+        for (int bit : {2, 8}) {
           vsel ^= bit;
           const float ms = time_slab();
           if (ms < base) base = ms;
@@ -1249,17 +1237,9 @@ struct Solver : SolverBase {
         CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
         return ms;
       };
-      float pbest = time_pencil();
-      for (int bit : {1, 16}) {  // the pencil alternatives are exclusive
-        vsel ^= bit;
-        const float ms = time_pencil();
-        if (ms < pbest) {
-          pbest = ms;
-          vsel &= ~(bit == 1 ? 16 : 1);
-        } else {
-          vsel ^= bit;
-        }
-      }
+      const float pbest = time_pencil();
+      vsel ^= 1;
+      if (!(time_pencil() < pbest)) vsel ^= 1;
       sync_check();
     }
     prof.on = pon;
@@ -1497,6 +1477,7 @@ struct Solver : SolverBase {
   void r2c_project(const T* rin, cpx<T>* dst, double wscale) {
     SlabArgs<T> a = slab_args();
     a.rio = const_cast<T*>(rin);
+    a.pairs = 0;  // (the run-time slab kernels work field by field)
     a.Ft = Ft[0];
     a.xmode = XMODE_R2C;
     for (int z0 = 0; z0 < N; z0 += G) {
@@ -1508,6 +1489,7 @@ struct Solver : SolverBase {
     LAUNCH_CHECK();
     PencilArgs<T> p = pencil_args(MODE_PROJECT);
     p.shell = nullptr;
+    p.pairs = 0;
     p.nF = 1; p.F[0] = Ft[0]; p.wF[0] = (T)wscale;
     p.state = dst;
     pencil(p);
@@ -1517,9 +1499,11 @@ struct Solver : SolverBase {
     PencilArgs<T> p = pencil_args(MODE_INIT);
     p.shell = nullptr;
     p.src = src;
+    p.pairs = 0;
     p.nOut = 1; p.out[0] = mixed[0];
     pencil(p);
     SlabArgs<T> a = slab_args();
+    a.pairs = 0;
     a.mixed = mixed[0];
     a.rio = rout;
     a.xmode = XMODE_C2R;
@@ -1644,6 +1628,7 @@ struct Solver : SolverBase {
     a.mixed = mixed[0];
     a.mixedB = mixedB;
     a.Ft = out;
+    a.pairs = 0;
     a.xmode = xmode;
     for (int z0 = 0; z0 < N; z0 += G) {
       a.z0 = z0;
@@ -1661,6 +1646,7 @@ struct Solver : SolverBase {
     PencilArgs<T> p = pencil_args(MODE_INIT);
     p.shell = nullptr;
     p.src = S;
+    p.pairs = 0;
     p.nOut = 1; p.osh[0] = tab; p.out[0] = mixed[0];
     pencil(p);
     p.src = rho;
@@ -1670,6 +1656,7 @@ struct Solver : SolverBase {
     slab_adj(XMODE_ADJ_RU, FtB);
     PencilArgs<T> q = pencil_args(MODE_NL);
     q.shell = nullptr;
+    q.pairs = 0;
     q.nF = 1; q.dsh[0] = tab; q.wF[0] = (T)(1.0 / ((double)N * N * N));
     q.F[0] = Ft[0]; q.acc = tmpA;
     pencil(q);

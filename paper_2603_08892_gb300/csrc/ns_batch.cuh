@@ -89,14 +89,15 @@ struct BCfg {
     using C = K2Cfg<T, N>;
     const size_t cs = sizeof(cpx<T>);
     const size_t tw = (size_t)tw_elems(N);
-    const size_t p = (3 * (size_t)lf_rows<T, C::TX>(N) * C::TX + tw) * cs;
-    const size_t yi = (4 * (size_t)lf_rows<T, C::TYI>(N) * C::TYI + tw) * cs;  // 3 input slots + work
-    const size_t yf = ((size_t)lf_rows<T, C::TY>(N) * C::TY + tw) * cs, x = ((size_t)C::XELEMS + tw) * cs;
+    const size_t p = (size_t)C::p_elems * cs;
+    const size_t yi = (size_t)C::y_elems(C::TYI) * cs;
+    const size_t yf = (size_t)C::y_elems(C::TY) * cs, x = ((size_t)C::XELEMS + tw) * cs;
     const size_t a = p > yi ? p : yi, b = yf > x ? yf : x;
     return a > b ? a : b;
   }
-  static constexpr int NT = cmax(cmax(cmax(nt<16>(), nt<32>()), cmax(nt<48>(), nt<64>())),
-                                 cmax(nt<96>(), nt<128>()));
+  static constexpr int NT0 = cmax(cmax(cmax(nt<16>(), nt<32>()), cmax(nt<48>(), nt<64>())),
+                                  cmax(nt<96>(), nt<128>()));
+  static constexpr int NT = (NT0 + 31) / 32 * 32;
   static constexpr size_t SM_a = sm<16>() > sm<32>() ? sm<16>() : sm<32>();
   static constexpr size_t SM_b = sm<48>() > sm<64>() ? sm<48>() : sm<64>();
   static constexpr size_t SM_c = sm<96>() > sm<128>() ? sm<96>() : sm<128>();
@@ -171,7 +172,7 @@ __device__ __noinline__ void run_item(const BatchMem<T>& bm, int pass, int step,
   }
   if (pass == P_Y1 || pass == P_Y2) {
     constexpr int ntx = M / C::TYI;
-    yinv_tile<T, N, MemCG>(bm.sa, tile % ntx, tile / ntx, smem);
+    yinv_tile<T, N, MemCG, C::TYI>(bm.sa, tile % ntx, tile / ntx, smem);
     return;
   }
   if (pass == P_X1 || pass == P_X2) {
@@ -180,7 +181,7 @@ __device__ __noinline__ void run_item(const BatchMem<T>& bm, int pass, int step,
   }
   if (pass == P_F1 || pass == P_F2) {
     constexpr int ntx = M / C::TY;
-    yfwd_tile<T, N, MemCG>(bm.sa, tile % ntx, tile / ntx, smem);
+    yfwd_tile<T, N, MemCG, C::TY>(bm.sa, tile % ntx, tile / ntx, smem);
     return;
   }
   // pencil passes: INIT (pass < 0), P1, P2
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(128) k_bgrid_tab(const BatchMem<T>* __restrict
   batch_tab<T, N>(mems[__ldg(&cls[blockIdx.y])], step, nsteps);
 }
 template <typename T, int N>
-__global__ void __launch_bounds__(K2Cfg<T, N>::NTP) k_bgrid_pencil(const BatchMem<T>* __restrict__ mems,
+__global__ void __launch_bounds__(K2Cfg<T, N>::NTP, K2Cfg<T, N>::MINB_P) k_bgrid_pencil(const BatchMem<T>* __restrict__ mems,
                                                                   const int* __restrict__ cls, int pass, int step,
                                                                   int nsteps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -284,11 +285,11 @@ __global__ void __launch_bounds__(K2Cfg<T, N>::NTP) k_bgrid_pencil(const BatchMe
                            reinterpret_cast<cpx<T>*>(smem_raw));
 }
 template <typename T, int N>
-__global__ void __launch_bounds__(K2Cfg<T, N>::NTYI) k_bgrid_yinv(const BatchMem<T>* __restrict__ mems,
+__global__ void __launch_bounds__(K2Cfg<T, N>::NTYI, K2Cfg<T, N>::MINB_YI) k_bgrid_yinv(const BatchMem<T>* __restrict__ mems,
                                                                  const int* __restrict__ cls) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int ntx = (N / 2) / K2Cfg<T, N>::TYI;
-  yinv_tile<T, N, MemNC>(mems[__ldg(&cls[blockIdx.y])].sa, (int)blockIdx.x % ntx, (int)blockIdx.x / ntx,
+  yinv_tile<T, N, MemNC, K2Cfg<T, N>::TYI>(mems[__ldg(&cls[blockIdx.y])].sa, (int)blockIdx.x % ntx, (int)blockIdx.x / ntx,
                          reinterpret_cast<cpx<T>*>(smem_raw));
 }
 template <typename T, int N>
@@ -298,11 +299,11 @@ __global__ void __launch_bounds__(K2Cfg<T, N>::NTX, K2Cfg<T, N>::MINB_X) k_bgrid
   xrow_tile<T, N, MemNC>(mems[__ldg(&cls[blockIdx.y])].sa, (int)blockIdx.x, reinterpret_cast<cpx<T>*>(smem_raw));
 }
 template <typename T, int N>
-__global__ void __launch_bounds__(K2Cfg<T, N>::NTY, 2) k_bgrid_yfwd(const BatchMem<T>* __restrict__ mems,
+__global__ void __launch_bounds__(K2Cfg<T, N>::NTY, K2Cfg<T, N>::MINB_Y) k_bgrid_yfwd(const BatchMem<T>* __restrict__ mems,
                                                                    const int* __restrict__ cls) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int ntx = (N / 2) / K2Cfg<T, N>::TY;
-  yfwd_tile<T, N, MemNC>(mems[__ldg(&cls[blockIdx.y])].sa, (int)blockIdx.x % ntx, (int)blockIdx.x / ntx,
+  yfwd_tile<T, N, MemNC, K2Cfg<T, N>::TY>(mems[__ldg(&cls[blockIdx.y])].sa, (int)blockIdx.x % ntx, (int)blockIdx.x / ntx,
                          reinterpret_cast<cpx<T>*>(smem_raw));
 }
 
@@ -351,9 +352,8 @@ cudaError_t launch_class(const BatchMem<T>* dm, const int* cls, int nc, int nste
   using C = K2Cfg<T, N>;
   constexpr int M = N / 2;
   const size_t cz = sizeof(cpx<T>), tw = (size_t)tw_elems(N);
-  const size_t smP = (3 * (size_t)lf_rows<T, C::TX>(N) * C::TX + tw) * cz;
-  const size_t smYI = (4 * (size_t)lf_rows<T, C::TYI>(N) * C::TYI + tw) * cz;
-  const size_t smY = ((size_t)lf_rows<T, C::TY>(N) * C::TY + tw) * cz;
+  const size_t smP = (size_t)C::p_elems * cz;
+  const size_t smYI = (size_t)C::y_elems(C::TYI) * cz, smY = (size_t)C::y_elems(C::TY) * cz;
   const size_t smX = ((size_t)C::XELEMS + tw) * cz;
   static bool attr = false;  // (per template instance: the opt-in sizes set before the first launch)
   if (!attr) {
@@ -467,10 +467,10 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
     a.N = N; a.M = M; a.tw = (const cpx<T>*)cb.tw; a.dt = (T)dt[m]; a.ifac = (const T*)cb.ifac;
     a.state = (cpx<T>*)cb.state; a.acc = nullptr; a.trunc = cb.truncation; a.K2max = cb.K2max;
     a.Kimax = cb.Kimax; a.err = (int*)cb.err; a.wF[0] = (T)(1.0 / ((double)N * N * N));
-    a.F[0] = (const cpx<T>*)cb.Ft; a.out[0] = (cpx<T>*)cb.mixed;
+    a.F[0] = (const cpx<T>*)cb.Ft; a.out[0] = (cpx<T>*)cb.mixed; a.pairs = 1;
     SlabArgs<T>& s = bm.sa;
     s.N = N; s.M = M; s.z0 = 0; s.G = N; s.tw = (const cpx<T>*)cb.tw; s.mixed = (const cpx<T>*)cb.mixed;
-    s.scr = (cpx<T>*)cb.scr; s.Ft = (cpx<T>*)cb.Ft; s.xmode = XMODE_NONLINEAR; s.err = (int*)cb.err;
+    s.scr = (cpx<T>*)cb.scr; s.Ft = (cpx<T>*)cb.Ft; s.xmode = XMODE_NONLINEAR; s.pairs = 1; s.err = (int*)cb.err;
     if (cb.G < N) return NS_ERR_INTERNAL;
     items_for<T>(N, bm.items, &bm.pro_init);
     bm.cum[0] = 0;

@@ -49,6 +49,13 @@ __device__ __forceinline__ cpx<float> cmul_fixed(cpx<float> a, cpx<float> b) {
 __device__ __forceinline__ cpx<double> cmul_fixed(cpx<double> a, cpx<double> b) {
   return mk<double>(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.x, b.y, __dmul_rn(a.y, b.x)));
 }
+// a conj(b), likewise
+__device__ __forceinline__ cpx<float> mul_conj_fixed(cpx<float> a, cpx<float> b) {
+  return mk<float>(__fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, -__fmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ cpx<double> mul_conj_fixed(cpx<double> a, cpx<double> b) {
+  return mk<double>(__fma_rn(a.x, b.x, __dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, -__dmul_rn(a.x, b.y)));
+}
 // multiply by s*i (s = +1 or -1)
 template <typename T>
 __device__ __forceinline__ cpx<T> mul_si(cpx<T> a, T s) { return mk(-s * a.y, s * a.x); }

@@ -17,6 +17,17 @@
 
 namespace ns {
 
+// Layouts of the mixed fields and of Ft.  pairs = 0: each field by itself, [f][z][ky][kx].
+// pairs = 1 (the compile-time kernels): fields 0 and 1 interleaved mode by mode, then field 2,
+// then (mixed) fields 3 and 4 interleaved: a pencil tile of 8 columns reads and writes 128
+// contiguous bytes per plane of a pair in FP32 instead of 64.
+__host__ __device__ __forceinline__ size_t ft_index(int pairs, int f, size_t g, size_t fs) {
+  return pairs && f < 2 ? 2 * g + f : f * fs + g;
+}
+__host__ __device__ __forceinline__ size_t mixed_index(int pairs, int f, size_t g, size_t fs) {
+  return pairs && f >= 3 ? 3 * fs + 2 * g + (f - 3) : ft_index(pairs, f, g, fs);
+}
+
 enum PencilMode {
   MODE_INIT = 0,     // S_next = S0 (state)
   MODE_RK2_1 = 1,    // S_next = (S0 + dt/2 N) E_{dt/2}
@@ -117,6 +128,7 @@ struct PencilArgs {
   int* err;
   double* epart;         // [tiles][2]: sums of w |S|^2 and w k^2 |S|^2 of the written state, or null
   int iy0;               // first ky row of the launch (rank-range passes; 0 for a whole field)
+  int pairs;             // layout of F and out: mixed_index, ft_index
 };
 
 template <typename T>
@@ -315,10 +327,11 @@ struct SlabArgs {
   int* err;
   void* umax;           // or null: max_x |u_i(x)| of the velocity rows, i = 0..2, folded in
                         // with atomicMax on the IEEE bits (unsigned / unsigned long long [3])
-  // modes of Ft no pencil pass reads (skip_tx > 0: the compile-time y-forward leaves them
-  // unwritten): those of pencil tiles of skip_tx columns outside the truncation (trunc, K2max,
-  // Kimax) and outside the forcing block |k| <= fK (fK < 0: no forcing)
-  int skip_tx, trunc, K2max, Kimax, fK;
+  // skip: the compile-time y-forward leaves the Ft columns (kx, ky) unwritten that lie outside the
+  // truncation (trunc, K2max, Kimax) and outside the forcing block |k| <= fK (fK < 0: no
+  // forcing); no pencil pass uses them
+  int skip, trunc, K2max, Kimax, fK;
+  int pairs;             // layout of mixed, mixedB and Ft: mixed_index, ft_index
 };
 
 // Block maxima m0..m2 (non-negative) folded into umax[0..2], one atomic per value per block:
@@ -366,7 +379,8 @@ __global__ void __launch_bounds__(512) k_yinv(SlabArgs<T> a) {
   for (int e = threadIdx.x; e < tile; e += blockDim.x) {
     const int iy = e / TY, x = e - iy * TY;
     const size_t g = ((size_t)z * N + iy) * M + x0 + x;
-    cpx<T> ux = a.mixed[g], uy = a.mixed[g + fstride], uz = a.mixed[g + 2 * fstride];
+    auto mx = [&](const cpx<T>* m, int f) { return m[mixed_index(a.pairs, f, g, fstride)]; };
+    cpx<T> ux = mx(a.mixed, 0), uy = mx(a.mixed, 1), uz = mx(a.mixed, 2);
     // slots 0..2 and 3..5 of the pair whose cross product the x rows form
     int su = 0, sw = 3, sr = -1;
     if (a.xmode == XMODE_ADJ_WR) { sw = 0; sr = 3; su = -1; }
@@ -377,16 +391,16 @@ __global__ void __launch_bounds__(512) k_yinv(SlabArgs<T> a) {
       buf[(su + 2) * tile + e] = uz;
     }
     if (nf == 6 && sw >= 0) {
-      cpx<T> dzx = a.mixed[g + 3 * fstride], dzy = a.mixed[g + 4 * fstride];
+      cpx<T> dzx = mx(a.mixed, 3), dzy = mx(a.mixed, 4);
       const T kx = (T)(x0 + x), ky = (T)kof(iy, N);
       buf[sw * tile + e] = mul_si(uz, ky) - dzy;                  // w_x = i ky uz - dz uy
       buf[(sw + 1) * tile + e] = dzx - mul_si(uz, kx);            // w_y = dz ux - i kx uz
       buf[(sw + 2) * tile + e] = mul_si(uy, kx) - mul_si(ux, ky); // w_z = i kx uy - i ky ux
     }
     if (sr >= 0) {
-      buf[sr * tile + e] = a.mixedB[g];
-      buf[(sr + 1) * tile + e] = a.mixedB[g + fstride];
-      buf[(sr + 2) * tile + e] = a.mixedB[g + 2 * fstride];
+      buf[sr * tile + e] = mx(a.mixedB, 0);
+      buf[(sr + 1) * tile + e] = mx(a.mixedB, 1);
+      buf[(sr + 2) * tile + e] = mx(a.mixedB, 2);
     }
   }
   __syncthreads();
@@ -421,7 +435,7 @@ __global__ void __launch_bounds__(512) k_yfwd(SlabArgs<T> a) {
   for (int f = 0; f < 3; ++f) {
     for (int e = threadIdx.x; e < tile; e += blockDim.x) {
       const int iy = e / TY, x = e - iy * TY;
-      a.Ft[f * fstride + ((size_t)z * N + iy) * M + x0 + x] = buf[f * tile + e];
+      a.Ft[ft_index(a.pairs, f, ((size_t)z * N + iy) * M + x0 + x, fstride)] = buf[f * tile + e];
     }
   }
 }
@@ -892,6 +906,22 @@ __global__ void k_force_vjp(const cpx<double>* __restrict__ pj, const cpx<double
       const double fx = (1.0 - theta) * p0.x + theta * p1.x, fy = (1.0 - theta) * p0.y + theta * p1.y;
       tab[k * D + i] = mk<T>((T)(coef * fx), (T)(coef * fy));
     }
+  }
+}
+
+// Block [lo, lo + n) of axis 0 (z or kz) or 1 (ky) of a buffer of F fields in layout `pairs`
+// (mixed_index serves Ft as well: it has fields 0 .. 2 only) <-> contiguous [F][...] staging
+template <typename T>
+__global__ void k_block_copy(cpx<T>* buf, cpx<T>* stg, int F, int N, int axis, int lo, int n, int pairs, int to_buf) {
+  const int M = N / 2;
+  const size_t fs = (size_t)N * N * M, per = (size_t)n * N * M;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < F * per; i += (size_t)gridDim.x * blockDim.x) {
+    const int f = (int)(i / per), kx = (int)(i % M);
+    const size_t r = (i % per) / M;  // axis 0: z N + y of the block; axis 1: z n + y
+    const size_t z = axis == 0 ? lo + r / N : r / n, y = axis == 0 ? r % N : lo + r % n;
+    cpx<T>* p = buf + mixed_index(pairs, f, (z * N + y) * M + kx, fs);
+    if (to_buf) *p = stg[i];
+    else stg[i] = *p;
   }
 }
 

@@ -10,7 +10,7 @@
 // registers (per kernel, K2Cfg).
 #pragma once
 
-#include "ns_fft2.cuh"
+#include "ns_fft3.cuh"
 #include "ns_kernels.cuh"
 
 namespace ns {
@@ -32,6 +32,12 @@ __host__ __device__ constexpr int round_lines(int t, int w) {
   return (v + l - 1) / l * l;
 }
 
+// two modes side by side in memory (16 bytes in FP32): the fields that share a line of the x rows
+template <typename T>
+struct alignas(16) cpair {
+  cpx<T> a, b;
+};
+
 // Global-memory access policy.  MemNC: data written by earlier launches (read-only path).
 // MemCG: data written by other blocks of the same launch (persistent kernel): loads and
 // stores go to L2 (.cg) so a block never sees a stale line in its own L1.
@@ -42,13 +48,24 @@ struct MemNC {
   static __device__ __forceinline__ cpx<T> ldw(const cpx<T>* p) { return *p; }
   template <typename T>
   static __device__ __forceinline__ void st(cpx<T>* p, cpx<T> v) { *p = v; }
-  // two consecutive FP32 modes (16-byte aligned)
-  static __device__ __forceinline__ float4 ld2(const cpx<float>* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-  static __device__ __forceinline__ void st2(cpx<float>* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+  static __device__ __forceinline__ void ldp(const cpair<float>* p, cpx<float>& a, cpx<float>& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = mk<float>(v.x, v.y);
+    b = mk<float>(v.z, v.w);
+  }
+  static __device__ __forceinline__ void ldp(const cpair<double>* p, cpx<double>& a, cpx<double>& b) {
+    a = p->a;
+    b = p->b;
+  }
+  static __device__ __forceinline__ void stp(cpair<float>* p, cpx<float> a, cpx<float> b) {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+  }
+  static __device__ __forceinline__ void stp(cpair<double>* p, cpx<double> a, cpx<double> b) {
+    p->a = a;
+    p->b = b;
+  }
 };
 struct MemCG {
-  static __device__ __forceinline__ float4 ld2(const cpx<float>* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
-  static __device__ __forceinline__ void st2(cpx<float>* p, float4 v) { __stcg(reinterpret_cast<float4*>(p), v); }
   static __device__ __forceinline__ cpx<float> ld(const cpx<float>* p) {
     const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
     return mk<float>(v.x, v.y);
@@ -64,6 +81,22 @@ struct MemCG {
   }
   static __device__ __forceinline__ void st(cpx<double>* p, cpx<double> v) {
     __stcg(reinterpret_cast<double2*>(p), make_double2(v.x, v.y));
+  }
+  static __device__ __forceinline__ void ldp(const cpair<float>* p, cpx<float>& a, cpx<float>& b) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+    a = mk<float>(v.x, v.y);
+    b = mk<float>(v.z, v.w);
+  }
+  static __device__ __forceinline__ void ldp(const cpair<double>* p, cpx<double>& a, cpx<double>& b) {
+    a = ld(&p->a);
+    b = ld(&p->b);
+  }
+  static __device__ __forceinline__ void stp(cpair<float>* p, cpx<float> a, cpx<float> b) {
+    __stcg(reinterpret_cast<float4*>(p), make_float4(a.x, a.y, b.x, b.y));
+  }
+  static __device__ __forceinline__ void stp(cpair<double>* p, cpx<double> a, cpx<double> b) {
+    st(&p->a, a);
+    st(&p->b, b);
   }
 };
 
@@ -98,32 +131,31 @@ __device__ __forceinline__ void stage_col_tile(cpx<T>* dst, const cpx<T>* src, i
   }
 }
 
-// Radix cap of each kernel's transforms (pencil z, inverse y, forward y, x rows); 0 = the
-// measured default: in FP32 radix 16 for both y passes and the x rows (one shared-memory pass
-// fewer; the inverse y, bound by shared memory, 0.268 against 0.287 ms per step at 256^3 with
-// radix 8), radix 8 for the pencil (more threads per tile); 8 in FP64.
-#ifndef NS_RADIX_Z
-#define NS_RADIX_Z 0
-#endif
-#ifndef NS_RADIX_YI
-#define NS_RADIX_YI 0
-#endif
-#ifndef NS_RADIX_YF
-#define NS_RADIX_YF 0
-#endif
-#ifndef NS_RADIX_X
-#define NS_RADIX_X 0
-#endif
-__host__ __device__ constexpr int radix_cap(int set, int f32_default, bool f32) {
-  return set > 0 ? set : (f32 ? f32_default : NS_MAX_RADIX);
+// The alternative width of a tile (lines per tile): twice the default where that divides
+// the half length m within the cap, else half (down to minw), else the default.
+__host__ __device__ constexpr int alt_width(int w, int m, int cap, int minw) {
+  return (m % (2 * w) == 0 && 2 * w <= cap) ? 2 * w : ((w / 2 >= minw && m % (w / 2) == 0) ? w / 2 : w);
 }
-// NS_SLAB_RADIX_RULE=1: the FP32 slab passes of N <= 128 take radix 8 where the radix-16 plan
-// keeps a radix-2 stage that the radix-8 plan avoids (N = 32: 16.2 -> 8.4; N = 96: 16.2.3 ->
-// 8.4.3).  Measured on GB300: 96^3 step 0.110 against 0.123 ms, 32^3 0.058 against 0.060, the
-// 64-member ensemble +4 %; at 512 (16.16.2 -> 8.8.8) it was 14 % slower, so larger N keep 16.
-#ifndef NS_SLAB_RADIX_RULE
-#define NS_SLAB_RADIX_RULE 1
-#endif
+
+// rows of an x-row tile of `per` threads per row: the smallest even number that gives at least
+// 128 threads (64 up to N = 64, where blocks are few), halved while three lines per row pass 52 KB
+__host__ __device__ constexpr int x_rows(int per, int n, int line_bytes) {
+  int r = 2;
+  while (r * per < (n <= 64 ? 64 : 128)) r += 2;
+  while (r % 4 == 0 && 3 * r * line_bytes > 52 * 1024) r /= 2;
+  return r;
+}
+
+// columns of a tile of `per` threads per column: 64-byte rows (128 bytes for an interleaved pair),
+// fewer where that makes more than `lim` threads or, on small grids, fewer than 152 blocks
+__host__ __device__ constexpr int y_cols(int n, int per, int minw, int lim) {
+  int w = pick_div(n / 2, 2 * minw, 16);
+  while (w > minw && w % 2 == 0 && (w * per > lim || (n / 2 / w * n < 152 && w / 2 * per >= 32))) w /= 2;
+  return w;
+}
+
+// Radix plans of the z, y and x transforms.  FP32: the x rows and both y passes with radix 16,
+// except where that keeps a radix-2 stage that radix 8 avoids on N <= 128 (N = 32, 96).
 __host__ __device__ constexpr bool plan_has_radix2(int n, int mr) {
   const CPlan p = cplan(n, mr);
   for (int i = 0; i < p.nst; ++i)
@@ -131,138 +163,95 @@ __host__ __device__ constexpr bool plan_has_radix2(int n, int mr) {
   return false;
 }
 __host__ __device__ constexpr int slab_radix(int n) {
-  return NS_SLAB_RADIX_RULE && n <= 128 && plan_has_radix2(n, 16) && !plan_has_radix2(n, 8) ? 8 : 16;
+  return n <= 128 && plan_has_radix2(n, 16) && !plan_has_radix2(n, 8) ? 8 : 16;
 }
-
-// Unroll factor of the pencil's loops over the transforms of the components: 1 keeps one copy
-// of the transform code per loop (measured 6 % faster than full unrolling at 256^3 FP32: the
-// pencil is sensitive to instruction-cache misses)
-#ifndef NS_PENCIL_UNROLL
-#define NS_PENCIL_UNROLL 1
-#endif
-constexpr int kPencilUnroll = NS_PENCIL_UNROLL;
-// modes per thread whose state loads the fused spectral pass keeps in flight together
-#ifndef NS_PENCIL_CHK
-#define NS_PENCIL_CHK 4
-#endif  // (pragma arguments are not macro-expanded)
-// NS_PENCIL_STAGE_STATE=1: the one-input pencil also stages the 3 state tiles with cp.async at
-// the start of a tile (6 tiles of shared memory, 2 blocks per SM instead of 3)
-#ifndef NS_PENCIL_STAGE_STATE
-#define NS_PENCIL_STAGE_STATE 0
-#endif
-
-// The alternative width of a tile (lines per tile): twice the default where that divides
-// the half length m within the cap, else half (down to minw), else the default.
-__host__ __device__ constexpr int alt_width(int w, int m, int cap, int minw) {
-  return (m % (2 * w) == 0 && 2 * w <= cap) ? 2 * w : ((w / 2 >= minw && m % (w / 2) == 0) ? w / 2 : w);
-}
+// FP64 at N = 24 and 32: radix 4, as the few columns of those grids must spread over every SM's
+// FP64 pipe.  The x rows of sizes whose FP32 tiles of x_rows rows do not divide the planes (192, 384)
+// have no reproducible pairing of rows to keep and take the plan with the fewest stages.
+__host__ __device__ constexpr bool small64(int n) { return n >= 24 && n <= 32; }
+__host__ __device__ constexpr int x_rows(int n, int cs) { return cmin(cmax(8192 / (n / 2 * cs), 1), 16); }
+template <typename T, int N>
+struct ZPlan { static constexpr CPlan P = fplan<T>(N, 8, small64(N) ? 4 : 8); };
+template <typename T, int N>
+struct YPlan { static constexpr CPlan P = fplan<T>(N, slab_radix(N), small64(N) ? 4 : 12); };
+template <typename T, int N>
+struct XPlan {
+  // (a pass holds every plane up to N = 96, groups of whole planes beyond)
+  static constexpr bool FREE = sizeof(T) == 8 || (N < 128 ? N * N : N) % x_rows(N, (int)sizeof(cpx<T>)) != 0;
+  static constexpr CPlan P = FREE ? radix_plan(N, sizeof(T) == 4 ? 16 : small64(N) ? 4 : 12) : fplan<T>(N, slab_radix(N), 12);
+};
 
 // Tile shapes of size N.  V selects compiled alternatives for the autotuner, one bit per
-// kernel family: bit 0 the pencil width TX, bit 1 the inverse-y width TYI, bit 2 the x-row
-// count RX, bit 3 the forward-y width TY, bit 4 the pencil's register budget (64: one more
-// resident block) (V = 0: the defaults).
+// kernel family: bit 0 the pencil width TX, bit 1 the inverse-y width TYI, bit 3 the forward-y
+// width TY (V = 0: the defaults).
 template <typename T, int N, int V = 0>
 struct K2Cfg {
   static constexpr int M = N / 2;
   static constexpr int CS = (int)sizeof(cpx<T>);
   static constexpr int MINW = 32 / CS;  // 32-byte global segments
   static constexpr bool F32 = sizeof(T) == 4;
-  static constexpr int RZ = radix_cap(NS_RADIX_Z, NS_MAX_RADIX, F32);
-  static constexpr int RYI = radix_cap(NS_RADIX_YI, slab_radix(N), F32);
-  static constexpr int RYF = radix_cap(NS_RADIX_YF, slab_radix(N), F32);
-  static constexpr int RXR = radix_cap(NS_RADIX_X, slab_radix(N), F32);
-  // pencil: TX columns of N (NS_PZ_LINES / NS_YF_LINES override the pencil / forward-y width)
-#ifndef NS_PZ_LINES
-#define NS_PZ_LINES 0
-#endif
-#ifndef NS_YF_LINES
-#define NS_YF_LINES 0
-#endif
-  static constexpr int TX0 = (NS_PZ_LINES > 0 && M % NS_PZ_LINES == 0 && NS_PZ_LINES % MINW == 0)
-                                 ? NS_PZ_LINES
-                                 : pick_div(M, cmax(16384 / (N * CS), MINW), 16);
-  static constexpr int TX = (V & 1) ? alt_width(TX0, M, 16, MINW) : TX0;
-  static constexpr int NTP = round_lines(TX * N / RZ, TX);
-  // blocks per SM the register budget must allow (NS_PENCIL_REGS registers per thread;
-  // 80 measured best at 256^3 FP32 on GB300 against 96 and 128)
-#ifndef NS_PENCIL_REGS
-#define NS_PENCIL_REGS 80
-#endif
-  // (variant bit 16: the pencil held to 64 registers, one more resident block)
-  static constexpr int MINB_P = cmax(1, cmin(8, 65536 / (NTP * ((V & 16) ? 64 : NS_PENCIL_REGS))));
-  // forward y pass: TY columns of N in a tile of about 32 KB (measured at 256^3 FP32: 16
-  // columns, 0.133 ms per step against 0.141 for 8)
-  static constexpr int TY0 = (NS_YF_LINES > 0 && M % NS_YF_LINES == 0 && NS_YF_LINES % MINW == 0)
-                                 ? NS_YF_LINES
-                                 : pick_div(M, cmax(32768 / (N * CS), MINW), 16);
-  static constexpr int TY = (V & 8) ? alt_width(TY0, M, 32, MINW) : TY0;
-  static constexpr int NTY = round_warps(TY * N / RYF);
-  // inverse y pass: 4 shared tiles (3 input slots and a work tile); the width is the one
-  // measured best when the tile held 6 (the 5 inputs and the work tile) within 110 KB
-#ifndef NS_YI_LINES
-#define NS_YI_LINES 0
-#endif
-  static constexpr int TYI0 = (NS_YI_LINES > 0 && M % NS_YI_LINES == 0 && NS_YI_LINES % MINW == 0)
-                                  ? NS_YI_LINES
-                                  : pick_div(M, cmax(110000 / (6 * N * CS), MINW), 16);
-  static constexpr int TYI = (V & 2) ? alt_width(TYI0, M, 16, MINW) : TYI0;
-  static constexpr int NTYI = round_warps(TYI * N / RYI);
-  // x rows: RX rows of M, processed three fields at a time (NS_XR_ROWS overrides RX)
-#ifndef NS_XR_ROWS
-#define NS_XR_ROWS 0
-#endif
-  static constexpr int RX0 = NS_XR_ROWS > 0 ? NS_XR_ROWS : cmin(cmax(8192 / (M * CS), 1), 16);
-  static constexpr int RX = (V & 4) ? (2 * RX0 <= 16 ? 2 * RX0 : cmax(RX0 / 2, 1)) : RX0;
-  static constexpr int NTX = round_warps(3 * RX * M / RXR);
-  // elements of the x-row tile: 3 RX complex lines of length N (two real rows per line), and
-  // the blocks per SM its shared memory allows (the register budget is held to that many)
-  static constexpr int XELEMS = WorkTile<T, N, 3 * RX, false>::elems();
-  static constexpr int MINB_X = cmax(1, cmin(8, (227 * 1024) / ((XELEMS + tw_elems(N)) * CS + 1024)));
-  static __host__ __device__ constexpr int pencil_tiles(int nF) { return nF > 1 ? 5 : 4; }
+  // pencil: TX columns of N, three tiles in shared memory, one thread per column and first-stage
+  // butterfly (radix f); registers hold 3 f modes
+  static constexpr int ZF = ZPlan<T, N>::P.r[0], ZNB = N / ZF;
+  static constexpr int TX0 = y_cols(N, ZNB, MINW, 512);
+  static constexpr int TX = (V & 1) ? alt_width(TX0, M, 512 / ZNB, MINW) : TX0;
+  static constexpr int NTP = (TX * ZNB + 31) / 32 * 32;  // (whole warps: the energy sums shuffle)
+  static constexpr int PTS = Xchg<T, N, ZF, TX, true>::elems;
+  static constexpr int p_elems = 3 * PTS + tw_elems(N);
+  // FP32 energy sums: the grouping of the modes that one thread adds in FP32 (N / 8, except on the
+  // small grids whose N / 8 threads per column are not whole warps), kept as it was recorded with
+  static constexpr int EDX = pick_div(M, cmax(16384 / (N * CS), MINW), 16);
+  static constexpr int EDZ = F32 && N >= 24 ? round_lines(EDX * N / 8, EDX) / EDX : ZNB;
+  // blocks per SM the register budget must allow (variant bit 16: one more)
+  static constexpr int PREGS = F32 ? 128 : 168;
+  static constexpr int p_blocks(int regs) {
+    return cmax(1, cmin(cmin(16, 65536 / (NTP * regs)), (227 * 1024) / (p_elems * CS + 1024)));
+  }
+  static constexpr int MINB_P = p_blocks(PREGS);
+  static constexpr int MINB_P2 = p_blocks(F32 ? 168 : 255);  // two inputs and outputs
+  // y passes: tiles of TYI / TY columns, three in shared memory, one thread per column and
+  // last-stage butterfly
+  static constexpr CPlan YP = YPlan<T, N>::P;
+  static constexpr int YNB = N / YP.r[0];
+  static constexpr int TY0 = y_cols(N, YNB, MINW, 192), TYI0 = TY0;
+  static constexpr int TY = (V & 8) ? alt_width(TY0, M, 512 / YNB, MINW) : TY0;
+  static constexpr int TYI = (V & 2) ? alt_width(TYI0, M, 512 / YNB, MINW) : TYI0;
+  static constexpr int NTY = TY * YNB, NTYI = TYI * YNB;
+  static constexpr int y_elems(int w) { return 3 * (N + N / YP.r[0]) * w + tw_elems(N); }
+  static constexpr int y_blocks(int w, int regs) {
+    return cmax(1, cmin(cmin(16, 65536 / ((w * YNB + 31) / 32 * 32 * regs)), (227 * 1024) / (y_elems(w) * CS + 1024)));
+  }
+  static constexpr int YIREGS = F32 ? 160 : 168, YFREGS = F32 ? 144 : 168;
+  static constexpr int MINB_YI = y_blocks(TYI, YIREGS);
+  static constexpr int MINB_Y = y_blocks(TY, YFREGS);
+  // x rows: tiles of RX rows in pairs (q, q + RXH), whose third products share a line; N / f
+  // threads per row.  Two-stage plans whose threads of some pairs make one warp run warp by warp
+  // (XWP pairs each), without block barriers.
+  static constexpr CPlan XP = XPlan<T, N>::P;
+  static constexpr int XF0 = XP.r[0], XNB = N / XF0;
+  static constexpr int RXT = x_rows(N, CS);
+  static constexpr int RX0 = !XPlan<T, N>::FREE ? RXT : small64(N) ? 4 : cmax(2, RXT / 2 * 2);
+  static constexpr bool XWARP = XP.nst == 2 && XF0 % XP.r[XP.nst - 1] == 0 && RX0 % 2 == 0 && 2 * XNB <= 32 &&
+                                32 % (2 * XNB) == 0 && (RX0 * XNB) % 32 == 0;
+  static constexpr int RX = RX0, RXH = (RX0 + 1) / 2;
+  static constexpr int XWP = XWARP ? 32 / (2 * XNB) : RXH;       // pairs of a group
+  static constexpr int XNG = XWARP ? RXH / XWP : 1;              // groups of a tile
+  static constexpr int XGT = XWARP ? 32 : (2 * RXH * XNB + 31) / 32 * 32;  // threads of a group
+  static constexpr int NTX = XNG * XGT;
+  static constexpr int XGEL = Xchg<T, N, XF0, 6 * XWP, false>::elems;
+  static constexpr int XELEMS = XNG * XGEL + 32;                 // and the scratch of the block's maxima
+  static constexpr int XREGS = F32 ? 144 : 168;
+  static constexpr int MINB_X = cmax(1, cmin(cmin(16, 65536 / (NTX * XREGS)),
+                                             (227 * 1024) / ((XELEMS + tw_elems(N)) * CS + 1024)));
 };
 
 // ---- accessors ------------------------------------------------------------------------
-template <typename T, int N, int W, class MP>
-struct ColIn {  // global [z|kz][ky][kx] column tile (element e = z index), read-only
-  const cpx<T>* p;
-  int iy, x0;
-  __device__ __forceinline__ cpx<T> get(int line, int e) const {
-    return MP::ld(&p[((size_t)e * N + iy) * (N / 2) + x0 + line]);
-  }
-};
-template <typename T, int N, int W, class MP>
-struct ColOut {
-  cpx<T>* p;
-  int iy, x0;
-  __device__ __forceinline__ void put(int line, int e, cpx<T> v) const {
-    MP::st(&p[((size_t)e * N + iy) * (N / 2) + x0 + line], v);
-  }
-};
 template <typename T, int W>
 struct SmTile {  // shared [e][line]
   cpx<T>* p;
   __device__ __forceinline__ cpx<T> get(int line, int e) const { return p[lf_idx<T, W>(e, line)]; }
   __device__ __forceinline__ void put(int line, int e, cpx<T> v) const { p[lf_idx<T, W>(e, line)] = v; }
 };
-template <class MP, typename T>
-__device__ __forceinline__ cpx<T> phase3p(const cpx<T>* tab, int N, int ix, int iy, int iz) {
-  return cmul_fixed(cmul_fixed(MP::ld(&tab[ix]), MP::ld(&tab[N + iy])), MP::ld(&tab[2 * N + iz]));
-}
-// pencil output: shift, optional i kz factor, from a shared component tile
-template <typename T, int N, int W, class MP>
-struct PencilOutSrc {
-  const cpx<T>* s;
-  const cpx<T>* sh;
-  int iy, x0;
-  bool deriv;
-  __device__ __forceinline__ cpx<T> get(int line, int e) const {
-    cpx<T> v = s[lf_idx<T, W>(e, line)];
-    if (sh) v = cmul_fixed(v, phase3p<MP>(sh, N, x0 + line, iy, e));
-    if (deriv) v = mul_si(v, (T)kof(e, N));
-    return v;
-  }
-};
-
 // 1 / k^2 of the projection: FP32 uses the fast division intrinsic (within 2 ulp, far below
 // the FP32 path's per-step error), FP64 the correctly rounded division.
 template <typename T>
@@ -271,6 +260,9 @@ template <>
 __device__ __forceinline__ float recip_k2<float>(int k2) { return __fdividef(1.0f, (float)k2); }
 template <>
 __device__ __forceinline__ double recip_k2<double>(int k2) { return 1.0 / (double)k2; }
+
+template <int I>
+struct IntC { static constexpr int v = I; };
 
 // ---- spectral stage at one mode (Sec. 4.1, 4.2, 6.1) ----------------------------------
 // nv: de-shifted, weighted transform of u x omega at the mode: N(0) = 0, truncation T,
@@ -362,12 +354,19 @@ __device__ __forceinline__ void shell_record(const PencilArgs<T>& a, int c, int 
 }
 
 // ---- pencil pass --------------------------------------------------------------------
-// One tile: TX consecutive kx at one ky, all kz.  Shared memory: 3 component tiles (a 4th
-// when there are two inputs or two outputs) and the twiddle table.  Every thread works on
-// one fixed kx (NT is a multiple of TX), so the kx and ky factors of the phase and
-// integrating-factor tables are loaded once per thread.
-template <typename T, int N>
-__host__ __device__ constexpr int pencil_tiles(int nF, int nOut) { return (nF > 1 || nOut > 1) ? 4 : 3; }
+// One tile: TX consecutive kx at one ky, all kz; 3 shared tiles and the twiddle table.
+//
+// Bound by HBM (ROG stages: 3 + 3 fields read, 3 + 5 written) and, where every stage passes
+// through it, by shared memory.  The forward transforms' first stage reads Ft, the inverse ones'
+// last stage writes the mixed fields, and in between a thread holds the f modes kz(j + (N/f) r)
+// of its column for all three components in registers: the outputs of its K = f / l last forward
+// butterflies and the inputs of its first inverse one (see radix plans; where l does not divide f
+// the last forward stage goes through shared memory), so de-shift, N(0) = 0, truncation,
+// projection, forcing, the stage combine, the shift and i kz never touch shared memory.  Measured,
+// one Rogallo stage, FP32: 256^3 201 us (214 with every stage through shared memory), 512^3 1941
+// (2278), 128^3 26.9 (30.6).  From 384^3 on the pattern itself limits it: a copy with 64-byte
+// segments per plane and array reaches 3.3 TB/s at 512^3, with 128-byte ones 6.5 TB/s, hence the
+// interleaved pairs of fields (5.1 TB/s with the state still in 64-byte segments).
 
 // True when every mode of a pencil tile (kx in [x0, x0 + TX), this ky, every kz) lies outside
 // the truncation and none is in the forcing table: the truncated nonlinear term and the
@@ -383,34 +382,27 @@ __device__ __forceinline__ bool pencil_tile_truncated(const PencilArgs<T>& a, in
   return out && !forced;
 }
 
-// Zero columns of the outputs of a tile whose S_next vanishes (the inverse transforms of zero)
+// Zero columns of the outputs of a tile whose S_next vanishes (the inverse transforms of zero);
+// in either layout of the fields a pair of them takes the bytes of two
 template <typename T, int N, int TX, int NT, class MP>
 __device__ __forceinline__ void pencil_zero_outputs(const PencilArgs<T>& a, int nOut, int iy, int x0) {
   constexpr int M = N / 2;
   const size_t fstride = (size_t)N * N * M;
   if (threadIdx.x >= NT) return;
   for (int o = 0; o < nOut; ++o)
-    for (int f = 0; f < 5; ++f)
-      for (int i = threadIdx.x; i < N * TX; i += NT) {
-        const int iz = i / TX, line = i % TX;
-        MP::st(&a.out[o][f * fstride + ((size_t)iz * N + iy) * M + x0 + line], mk<T>(0, 0));
+    for (int i = threadIdx.x; i < N * TX; i += NT) {
+      const size_t g = ((size_t)(i / TX) * N + iy) * M + x0 + i % TX;
+      for (int f = 0; f < 5; f += f == 2 ? 1 : 2) {
+        cpx<T>* p = a.out[o] + f * fstride;
+        if (f == 2) {
+          MP::st(p + g, mk<T>(0, 0));
+        } else {
+          MP::st(p + (a.pairs ? 2 * g : g), mk<T>(0, 0));
+          MP::st(p + (a.pairs ? 2 * g + 1 : g + fstride), mk<T>(0, 0));
+        }
       }
+    }
 }
-
-// Last-stage output of a forward z transform of one input component: de-shift by
-// e^{-i k.delta} (the kx, ky factor cxy is the thread's own: the thread's line is fixed) and
-// the weight w.
-template <typename T, int W, class MP>
-struct DeshiftOut {
-  cpx<T>* p;
-  cpx<T> cxy;
-  const cpx<T>* dz;  // z factors of the shift table, or null (no shift)
-  T w;
-  __device__ __forceinline__ void put(int line, int e, cpx<T> v) const {
-    if (dz) v = mul_conj(v, cxy * MP::ld(&dz[e]));
-    p[lf_idx<T, W>(e, line)] = w * v;
-  }
-};
 
 // Energy and dissipation sums of the state a final-stage pencil tile writes (Sec. 3.4: E =
 // 1/2 sum w |S|^2, eps = nu sum w k^2 |S|^2, w = 1 at kx = 0 and 2 elsewhere): each thread's
@@ -447,94 +439,166 @@ __device__ __forceinline__ void tile_energy_store(double* epart, T e, T d) {
   }
 }
 
-// Spectral stage of a pencil tile with one input: the three components of F are staged,
-// transformed in place (the last stage de-shifting and weighting), then one pass per mode
-// applies N(0) = 0, truncation, projection and forcing and the RK stage combine of all three
-// components, leaving S_next (shifted for the output when there is one output) in the tiles.
-// MC: the stage mode fixed at compile time (-1: a.mode at run time)
-template <typename T, int N, class MP, bool EP, int MC = -1, int V = 0>
-__device__ __forceinline__ void pencil_spectral_one(const PencilArgs<T>& a, cpx<T>* buf, cpx<T>* tws,
-                                                    int iy, int x0, int nOut, bool tz, T& eacc,
-                                                    T& dacc) {
-  const int mode = MC >= 0 ? MC : a.mode;
+// NFC, NOC: the number of inputs and outputs known at compile time; -1: at run time, at most
+// one of each (the persistent ensemble).  (1, 1) is every RK2, Rogallo and RK4 stage, (2, 2) and
+// (0, 2) the exact scheme's, (0, 1) INIT, (1, 0) NL and PROJECT.  MC: the stage mode at compile time (-1: a.mode).
+// EP: the tile's energy sums are stored (NOC = 2: whenever a.epart is set).
+template <typename T, int N, class MP, int NFC = -1, int NOC = -1, bool EP = false, int MC = -1,
+          int V = 0>
+__device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id, cpx<T>* buf) {
   using C = K2Cfg<T, N, V>;
-  constexpr int M = N / 2, TX = C::TX, NT = C::NTP, tile = lf_rows<T, C::TX>(N) * TX;
-  constexpr int PER = (tile + NT - 1) / NT;
-  constexpr int DZ = NT / TX;
+  using PL = ZPlan<T, N>;
+  constexpr int nst = PL::P.nst, f = PL::P.r[0], l = PL::P.r[nst - 1], NB0 = N / f, NBL = N / l;
+  constexpr bool FUSE = f % l == 0;                    // last forward butterflies held by their thread
+  constexpr int K = FUSE ? f / l : (f + l - 1) / l;    // last-stage butterflies per thread
+  constexpr int M = N / 2, TX = C::TX, NT = TX * NB0, TS = C::PTS;
+  using X = Xchg<T, N, f, TX, true>;
+  static_assert(NT <= C::NTP, "one first-stage butterfly per thread");
+  constexpr int ED = C::EDZ;  // the energy sums add a column's modes iz = i (mod ED) in T, then in FP64
+  const int nF = NFC >= 0 ? NFC : a.nF, nOut = NOC >= 0 ? NOC : a.nOut;
+  const int mode = MC >= 0 ? MC : a.mode;
+  cpx<T>* tws = buf + 3 * TS;
+  constexpr int ntx = M / TX;
+  const int iy = a.iy0 + tile_id / ntx;  // (iy0: first ky row of a rank-range launch)
+  const int x0 = (tile_id % ntx) * TX;
   const size_t fstride = (size_t)N * N * M;
   const int ky = kof(iy, N);
-  const bool act = threadIdx.x < NT;
-  const int line = threadIdx.x % TX, kx = x0 + line;
-  const int iz0 = threadIdx.x / TX;
-  const bool rd0 = mode != MODE_NL && mode != MODE_PROJECT;
-  const cpx<T>* base0 = mode == MODE_RK4_4 ? a.acc : a.state;
-  if (!tz)
-    for (int c = 0; c < 3; ++c) stage_col_tile<T, N, TX, NT>(buf + c * tile, a.F[0] + c * fstride, iy, x0);
-  cp_async_commit();
-  if (NS_PENCIL_STAGE_STATE && rd0)  // the state tiles arrive during the forward transforms
-    for (int c = 0; c < 3; ++c) stage_col_tile<T, N, TX, NT>(buf + (3 + c) * tile, base0 + c * fstride, iy, x0);
-  cp_async_commit();
-  load_twiddles(tws, a.tw, N);
-  if (!tz) {
-    cp_async_wait_pending<1>();
-    __syncthreads();
-    const cpx<T>* dz = a.dsh[0] ? a.dsh[0] + 2 * N : nullptr;
-    cpx<T> d0 = mk<T>(1, 0);
-    if (dz) d0 = MP::ld(&a.dsh[0][kx]) * MP::ld(&a.dsh[0][N + iy]);
-#pragma unroll (kPencilUnroll)
-    for (int c = 0; c < 3; ++c) {
-      cpx<T>* t = buf + c * tile;
-      cfft_ip_to<T, N, 1, TX, NT, true, -1, true, C::RZ>(SmTile<T, TX>{t}, t,
-                                                         DeshiftOut<T, TX, MP>{t, d0, dz, a.wF[0]}, tws);
-    }
-    __syncthreads();
-  }
-
-  const bool pre = nOut == 1 && a.osh[0] != nullptr;
-  cpx<T> oxy = mk<T>(1, 0);
-  if (pre) oxy = cmul_fixed(MP::ld(&a.osh[0][kx]), MP::ld(&a.osh[0][N + iy]));
-  const bool useE = mode != MODE_INIT && mode != MODE_NL && mode != MODE_PROJECT;
-  T e1xy = 1, ehxy = 1;
-  if (useE) {
-    e1xy = a.ifac[kx] * a.ifac[iy];
-    ehxy = a.ifac[N + kx] * a.ifac[N + iy];
-  }
-  if (NS_PENCIL_STAGE_STATE) {
-    cp_async_wait_pending<0>();
-    __syncthreads();
-  }
-  if (act) {
-    constexpr int CHK = PER < NS_PENCIL_CHK ? PER : NS_PENCIL_CHK;  // modes whose state loads are in flight together
-    const bool rd1 = mode == MODE_RK4_2 || mode == MODE_RK4_3;
-    const size_t gxy = (size_t)iy * M + kx;
-    for (int i0 = 0; i0 < PER; i0 += CHK) {
-      cpx<T> s0[3][CHK];  // (the RK4 accumulator, read by two modes only, is loaded on use)
+  const int tid = threadIdx.x, line = tid % TX, j = tid / TX, kx = x0 + line;
+  const bool act = tid < NT;
+  const size_t gj = ((size_t)j * N + iy) * M + kx;  // element (kz index j, iy, kx) of a field
+  constexpr size_t ZS = (size_t)N * M;              // one plane
+  const bool tt = pencil_tile_truncated<T, TX>(a, x0, ky);  // N = 0 on the whole tile
+  const int nFe = tt ? 0 : nF;                              // inputs that are transformed
+  // the twiddle table, on its way while the first inputs are loaded
+  constexpr int KT = (N + NT - 1) / NT;
+  cpx<T> twr[KT];
 #pragma unroll
-      for (int j = 0; j < CHK; ++j) {
-        const int iz = iz0 + (i0 + j) * DZ;
-        const size_t g = gxy + (size_t)iz * N * M;
-        const bool ok = iz < N && i0 + j < PER;
+  for (int c = 0; c < KT; ++c) twr[c] = act && tid + c * NT < N ? ldg(&a.tw[tid + c * NT]) : mk<T>(0, 0);
+  auto put_tw = [&] {
+#pragma unroll
+    for (int c = 0; c < KT; ++c)
+      if (act && tid + c * NT < N) tws[tw_pad(tid + c * NT)] = twr[c];
+  };
+
+  const bool rd0 = mode != MODE_NL && mode != MODE_PROJECT;
+  const cpx<T>* base0 = (mode == MODE_INIT ? a.src : (mode == MODE_RK4_4 ? a.acc : a.state)) + gj;
+
+  // 1) forward z transforms of the inputs: de-shifted by e^{-i k.delta} and weighted (products in
+  //    one fixed rounding order, as the compiler may contract them differently in each instance)
+  cpx<T> v[3][f];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int r = 0; r < f; ++r) v[c][r] = mk<T>(0, 0);
+  if constexpr (NFC != 0) {
+    for (int q = 0; q < nFe; ++q) {
+      if (act) {
+        cpx<T> u[3][f];
+        const cpx<T>* src = a.F[q] + gj;
+        if (a.pairs) {
+          const cpair<T>* src01 = reinterpret_cast<const cpair<T>*>(a.F[q]) + gj;
+#pragma unroll
+          for (int r = 0; r < f; ++r) MP::ldp(src01 + r * NB0 * ZS, u[0][r], u[1][r]);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int r = 0; r < f; ++r) u[c][r] = MP::ld(src + c * fstride + r * NB0 * ZS);
+        }
+#pragma unroll
+        for (int r = 0; r < f; ++r) u[2][r] = MP::ld(src + 2 * fstride + r * NB0 * ZS);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          s0[c][j] = mk<T>(0, 0);
-          if (ok && rd0)
-            s0[c][j] = NS_PENCIL_STAGE_STATE ? buf[(3 + c) * tile + lf_idx<T, TX>(iz, line)]
-                                             : MP::ldw(&base0[c * fstride + g]);
+          DFT<T, f>::run(u[c], T(-1));
+          const int o = c * TS + X::at(line, j * f);
+#pragma unroll
+          for (int r = 0; r < f; ++r) buf[o + r * TX] = u[c][r];
         }
       }
+      if (q == 0) put_tw();
+      __syncthreads();
+      mid_stages<T, N, PL, 1, FUSE ? nst - 1 : nst, -1, X, TX, 3, NT, true>(buf, TS, tws);
+      if (act) {
+        const cpx<T>* sh = a.dsh[q];
+        cpx<T> cxy = mk<T>(1, 0);
+        if (sh) cxy = cmul_fixed(MP::ld(&sh[kx]), MP::ld(&sh[N + iy]));
+        auto take = [&](int c, int r, cpx<T> t, cpx<T> s) {  // element j + NB0 r of component c
+          if (sh) t = mul_conj_fixed(t, s);
+          if constexpr (NFC == 2) {
+            if (q == 0) v[c][r] = t;
+            else v[c][r] = mk<T>(fma1(a.wF[0], v[c][r].x, a.wF[1] * t.x), fma1(a.wF[0], v[c][r].y, a.wF[1] * t.y));
+          } else {
+            v[c][r] = a.wF[q] * t;
+          }
+        };
+        if constexpr (FUSE) {
 #pragma unroll
-      for (int j = 0; j < CHK; ++j) {
-        const int iz = iz0 + (i0 + j) * DZ, e = lf_idx<T, TX>(iz, line);
-        if (iz >= N || i0 + j >= PER) break;
-        const size_t g = gxy + (size_t)iz * N * M;
-        const int kz = kof(iz, N);
-        cpx<T> nv[3] = {mk<T>(0, 0), mk<T>(0, 0), mk<T>(0, 0)};
-        if (!tz) {
-          nv[0] = buf[e];
-          nv[1] = buf[tile + e];
-          nv[2] = buf[2 * tile + e];
-          project_point(a, kx, ky, kz, nv);
+          for (int i = 0; i < K; ++i) {
+            const int p = j + NB0 * i;
+            cpx<T> w[l], s[l];
+            reg_twiddles<T, N, l, NBL, -1>(w, tws, p);
+            if (sh)
+#pragma unroll
+              for (int r = 0; r < l; ++r) s[r] = cmul_fixed(cxy, MP::ld(&sh[2 * N + p + r * NBL]));
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              cpx<T> t[l];
+              const int o = c * TS + X::at(line, p);
+#pragma unroll
+              for (int r = 0; r < l; ++r) t[r] = buf[o + r * X::step(NBL)];
+              twiddle_dft<T, l>(t, w, T(-1));
+#pragma unroll
+              for (int r = 0; r < l; ++r) take(c, i + K * r, t[r], s[r]);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < f; ++r) {
+            cpx<T> s = cxy;
+            if (sh) s = cmul_fixed(cxy, MP::ld(&sh[2 * N + j + r * NB0]));
+            const int o = X::at(line, j + r * NB0);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) take(c, r, buf[c * TS + o], s);
+          }
         }
+      }
+      __syncthreads();
+    }
+  }
+  if (nFe == 0) put_tw();  // (its first reader is past the barrier of the first output batch)
+
+  // 2) spectral stage: every mode's N(0) = 0, truncation, projection and forcing, then the RK
+  //    stage combine; v becomes S_next, shifted for the output when there is one
+  const bool pre = nOut == 1 && a.osh[0] != nullptr;
+  T eacc = 0, dacc = 0;  // energy sums of the written state
+  bool nz = false;
+  if (act) {
+    cpx<T> oxy = mk<T>(1, 0);
+    if (pre) oxy = cmul_fixed(MP::ld(&a.osh[0][kx]), MP::ld(&a.osh[0][N + iy]));
+    const bool useE = mode != MODE_INIT && mode != MODE_NL && mode != MODE_PROJECT;
+    T e1xy = 1, ehxy = 1;
+    if (useE) {
+      e1xy = a.ifac[kx] * a.ifac[iy];
+      ehxy = a.ifac[N + kx] * a.ifac[N + iy];
+    }
+    const bool rd1 = mode == MODE_RK4_2 || mode == MODE_RK4_3;
+    constexpr int CHK = f % 4 == 0 ? 4 : (f % 3 == 0 ? 3 : 2);  // modes whose state loads are in flight
+#pragma unroll
+    for (int r0 = 0; r0 < f; r0 += CHK) {
+      cpx<T> s0[3][CHK];
+#pragma unroll
+      for (int i = 0; i < CHK; ++i)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          s0[c][i] = mk<T>(0, 0);
+          if (rd0) s0[c][i] = MP::ldw(base0 + c * fstride + (r0 + i) * NB0 * ZS);
+        }
+#pragma unroll
+      for (int i = 0; i < CHK; ++i) {
+        const int r = r0 + i, iz = j + r * NB0, kz = kof(iz, N);
+        const size_t g = gj + r * NB0 * ZS;
+        cpx<T> nv[3] = {v[0][r], v[1][r], v[2][r]};
+        if (nFe > 0) project_point(a, kx, ky, kz, nv);
         T E1 = 1, Eh = 1;
         if (useE) {
           E1 = e1xy * a.ifac[iz];
@@ -542,526 +606,529 @@ __device__ __forceinline__ void pencil_spectral_one(const PencilArgs<T>& a, cpx<
         }
         cpx<T> shz = oxy;
         if (pre) shz = cmul_fixed(oxy, MP::ld(&a.osh[0][2 * N + iz]));
-        T m2 = 0;  // |S|^2 of the written state (EP: final stages with a.epart)
+        T m2 = 0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const cpx<T> s1 = rd1 ? MP::ldw(&a.acc[c * fstride + g]) : mk<T>(0, 0);
-          cpx<T> sn = stage_combine<T, MP>(a, c, c * fstride + g, nv[c], s0[c][j], s1, E1, Eh, mode);
+          cpx<T> sn = stage_combine<T, MP>(a, c, c * fstride + g, nv[c], s0[c][i], s1, E1, Eh, mode);
           shell_record<T, MP>(a, c, kx, ky, kz, sn);
-          if constexpr (EP) m2 += sn.x * sn.x + sn.y * sn.y;
-          if (pre) sn = cmul_fixed(sn, shz);
-          buf[c * tile + e] = sn;
+          if (EP || NOC == 2) m2 += sn.x * sn.x + sn.y * sn.y;
+          nz = nz || sn.x != T(0) || sn.y != T(0);
+          v[c][r] = pre ? cmul_fixed(sn, shz) : sn;
         }
-        if constexpr (EP) {
+        if (EP || NOC == 2) {
           const T wm = (kx == 0 ? T(1) : T(2)) * m2;
-          eacc += wm;
-          dacc += wm * (T)(kx * kx + ky * ky + kz * kz);
-        }
-      }
-    }
-  }
-  __syncthreads();
-}
-
-// NFC, NOC: the number of inputs and outputs known at compile time (-1: read from the
-// arguments).  (1, 1) is every RK2, Rogallo and RK4 stage, (2, 2) the exact scheme's stage;
-// fixing them keeps those kernels free of register spills.
-template <typename T, int N, class MP, int NFC = -1, int NOC = -1, bool EP = false, int MC = -1,
-          int V = 0>
-__device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id, cpx<T>* buf) {
-  using C = K2Cfg<T, N, V>;
-  const int nF = NFC >= 0 ? NFC : a.nF, nOut = NOC >= 0 ? NOC : a.nOut;
-  constexpr int M = N / 2, TX = C::TX, NT = C::NTP, tile = lf_rows<T, C::TX>(N) * TX;
-  constexpr int PER = (tile + NT - 1) / NT;  // modes per thread (the last may not exist)
-  static_assert(NT % TX == 0, "every thread keeps one kx");
-  // component tile c is buf + c * tile (pointer arithmetic, not an array: no local memory)
-  auto bc = [&](int c) { return buf + c * tile; };
-  cpx<T>* b3 = buf + 3 * tile;
-  cpx<T>* tws = buf + (NFC == 1 && NS_PENCIL_STAGE_STATE ? 6 : pencil_tiles<T, N>(nF, nOut)) * tile;
-  constexpr int ntx = M / TX;
-  const int iy = a.iy0 + tile_id / ntx;  // (iy0: first ky row of a rank-range launch)
-  const int x0 = (tile_id % ntx) * TX;
-  const size_t fstride = (size_t)N * N * M;
-  const int ky = kof(iy, N);
-  const bool act = threadIdx.x < NT;
-  const int line = threadIdx.x % TX, kx = x0 + line;
-  const int iz0 = threadIdx.x / TX;  // this thread's modes: iz = iz0 + i * (NT / TX)
-  constexpr int DZ = NT / TX;
-
-  const bool pre = nOut == 1 && a.osh[0] != nullptr;  // S_next is shifted in the tiles
-  const bool tt = pencil_tile_truncated<T, TX>(a, x0, ky);  // N = 0 on the whole tile
-  const bool tz = nF > 0 && tt;                               // so its inputs are not transformed
-  T eacc = 0, dacc = 0;  // energy sums of the written state (a.epart)
-  if constexpr (NFC == 1) {
-    pencil_spectral_one<T, N, MP, EP, MC, V>(a, buf, tws, iy, x0, nOut, tz, eacc, dacc);
-  } else {
-    const int nFe = tz ? 0 : nF;  // inputs that are transformed
-    // 1) inputs: all three components staged asynchronously, then transformed in place
-    if (nFe > 0) {
-      for (int c = 0; c < 3; ++c) stage_col_tile<T, N, TX, NT>(bc(c), a.F[0] + c * fstride, iy, x0);
-    }
-    load_twiddles(tws, a.tw, N);  // also the barrier after which the staged tiles may be read
-    if (nFe > 0) {
-      cp_async_wait_all();
-      __syncthreads();
-      cpx<T> d0 = mk<T>(1, 0), d1 = mk<T>(1, 0);
-      if (a.dsh[0]) d0 = MP::ld(&a.dsh[0][kx]) * MP::ld(&a.dsh[0][N + iy]);
-      if (nF > 1 && a.dsh[1]) d1 = MP::ld(&a.dsh[1][kx]) * MP::ld(&a.dsh[1][N + iy]);
-      for (int c = 0; c < 3; ++c) {
-        cfft_ip<T, N, 1, TX, NT, true, -1, true, C::RZ>(SmTile<T, TX>{bc(c)}, bc(c), tws);
-        __syncthreads();
-        if (nF > 1) {
-          stage_col_tile<T, N, TX, NT>(b3, a.F[1] + c * fstride, iy, x0);
-          cp_async_wait_all();
-          __syncthreads();
-          cfft_ip<T, N, 1, TX, NT, true, -1, true, C::RZ>(SmTile<T, TX>{b3}, b3, tws);
-          __syncthreads();
-        }
-        if (act) {
-  #pragma unroll 4
-          for (int i = 0; i < PER; ++i) {
-            const int iz = iz0 + i * DZ, e = lf_idx<T, TX>(iz, line);
-            if (iz >= N) break;
-            cpx<T> v = bc(c)[e];
-            if (a.dsh[0]) v = mul_conj(v, d0 * MP::ld(&a.dsh[0][2 * N + iz]));
-            v = a.wF[0] * v;
-            if (nF > 1) {
-              cpx<T> w = b3[e];
-              if (a.dsh[1]) w = mul_conj(w, d1 * MP::ld(&a.dsh[1][2 * N + iz]));
-              v = v + a.wF[1] * w;
-            }
-            bc(c)[e] = v;
-          }
-        }
-        __syncthreads();
-      }
-      // 2a) N(0) = 0, truncation, projection, forcing (all components of a mode at once)
-      if (act) {
-        for (int i = 0; i < PER; ++i) {
-          const int iz = iz0 + i * DZ, e = lf_idx<T, TX>(iz, line);
-          if (iz >= N) break;
-          cpx<T> nv[3] = {bc(0)[e], bc(1)[e], bc(2)[e]};
-          project_point(a, kx, ky, kof(iz, N), nv);
-          bc(0)[e] = nv[0];
-          bc(1)[e] = nv[1];
-          bc(2)[e] = nv[2];
-        }
-      }
-    }
-
-    // 2b) stage combine per component, the state of the thread's modes loaded together
-    cpx<T> oxy = mk<T>(1, 0);
-    if (pre) oxy = cmul_fixed(MP::ld(&a.osh[0][kx]), MP::ld(&a.osh[0][N + iy]));
-    const bool useE = a.mode != MODE_INIT && a.mode != MODE_NL && a.mode != MODE_PROJECT;
-    T e1xy = 1, ehxy = 1;
-    if (useE) {
-      e1xy = a.ifac[kx] * a.ifac[iy];
-      ehxy = a.ifac[N + kx] * a.ifac[N + iy];
-    }
-    if (act) {
-      constexpr int CHK = PER < 8 ? PER : 8;  // modes whose state loads are in flight together
-      const bool rd0 = a.mode != MODE_NL && a.mode != MODE_PROJECT;
-      const bool rd1 = a.mode == MODE_RK4_2 || a.mode == MODE_RK4_3;
-      const cpx<T>* base0 = a.mode == MODE_INIT ? a.src : (a.mode == MODE_RK4_4 ? a.acc : a.state);
-      for (int c = 0; c < 3; ++c)
-      for (int i0 = 0; i0 < PER; i0 += CHK) {
-        const size_t gc = c * fstride + (size_t)iy * M + kx;
-        cpx<T> s0[CHK], s1[CHK];
-  #pragma unroll
-        for (int j = 0; j < CHK; ++j) {
-          const int iz = iz0 + (i0 + j) * DZ;
-          const size_t g = gc + (size_t)iz * N * M;
-          s0[j] = s1[j] = mk<T>(0, 0);
-          if (iz < N && i0 + j < PER) {
-            if (rd0) s0[j] = MP::ldw(&base0[g]);
-            if (rd1) s1[j] = MP::ldw(&a.acc[g]);
-          }
-        }
-  #pragma unroll
-        for (int j = 0; j < CHK; ++j) {
-          const int iz = iz0 + (i0 + j) * DZ, e = lf_idx<T, TX>(iz, line);
-          if (iz >= N || i0 + j >= PER) break;
-          const size_t g = gc + (size_t)iz * N * M;
-          T E1 = 1, Eh = 1;
-          if (useE) {
-            E1 = e1xy * a.ifac[iz];
-            Eh = ehxy * a.ifac[N + iz];
-          }
-          const cpx<T> n = nFe > 0 ? bc(c)[e] : mk<T>(0, 0);
-          cpx<T> sn = stage_combine<T, MP>(a, c, g, n, s0[j], s1[j], E1, Eh, a.mode);
-          shell_record<T, MP>(a, c, kx, ky, kof(iz, N), sn);
-          if (a.epart) {
-            const int kz = kof(iz, N);
-            const T wm = (kx == 0 ? T(1) : T(2)) * (sn.x * sn.x + sn.y * sn.y);
+          if constexpr (ED == NB0) {
             eacc += wm;
             dacc += wm * (T)(kx * kx + ky * ky + kz * kz);
+          } else {
+            reinterpret_cast<T*>(buf)[iz * TX + line] = wm;  // (the tiles are free here)
           }
-          if (pre) sn = cmul_fixed(sn, cmul_fixed(oxy, MP::ld(&a.osh[0][2 * N + iz])));
-          bc(c)[e] = sn;
         }
       }
     }
-    __syncthreads();
   }
-
-  // one-input tiles take the sums only in the EP variant; the others whenever a.epart is set
-  if constexpr (NFC == 1) {
-    if constexpr (EP) tile_energy_store<T>(a.epart, eacc, dacc);
-  } else if (a.epart) {
-    tile_energy_store<T>(a.epart, eacc, dacc);
-  }
-  if (tt) {  // S_next vanishing on the whole tile (a truncated state): zero outputs, no transforms
-    bool nz = false;
-    if (act)
-      for (int i = 0; i < PER; ++i) {
-        const int iz = iz0 + i * DZ, e = lf_idx<T, TX>(iz, line);
-        if (iz >= N) break;
-        for (int c = 0; c < 3; ++c) {
-          const cpx<T> v = bc(c)[e];
-          nz = nz || v.x != T(0) || v.y != T(0);
+  if constexpr (EP || NOC == 2) {
+    if (EP || a.epart) {
+      if constexpr (ED != NB0) {
+        __syncthreads();
+        for (int i = tid; i < TX * ED; i += blockDim.x) {
+          T e = 0, d = 0;
+          for (int iz = i / TX; iz < N; iz += ED) {
+            const int kz = kof(iz, N), k1 = x0 + i % TX;
+            const T wm = reinterpret_cast<const T*>(buf)[iz * TX + i % TX];
+            e += wm;
+            d += wm * (T)(k1 * k1 + ky * ky + kz * kz);
+          }
+          eacc += e;
+          dacc += d;
         }
       }
+      tile_energy_store<T>(a.epart, eacc, dacc);
+      if constexpr (ED != NB0) __syncthreads();
+    }
+  }
+  if (tt) {  // S_next vanishing on the whole tile (a truncated state): zero outputs, no transforms
     if (!__syncthreads_or(nz)) {
       pencil_zero_outputs<T, N, TX, NT, MP>(a, nOut, iy, x0);
       return;
     }
   }
-  if (nOut == 1) {
-    // u_z first (its tile then serves as the work tile), then u_x, d_z u_x, u_y, d_z u_y
-    const cpx<T>* sh = pre ? nullptr : a.osh[0];
-    cfft_src_in_work<T, N, 1, TX, NT, true, 1, C::RZ>(PencilOutSrc<T, N, TX, MP>{bc(2), sh, iy, x0, false},
-                                               ColOut<T, N, TX, MP>{a.out[0] + 2 * fstride, iy, x0},
-                                               bc(2), tws);
-    __syncthreads();
-#pragma unroll (kPencilUnroll)
-    for (int i = 0; i < 4; ++i) {
-      const int f = (i & 1) ? 3 + (i >> 1) : (i >> 1), c = f < 3 ? f : f - 3;  // 0, 3, 1, 4
-      cfft<T, N, 1, TX, NT, true, 1, C::RZ>(PencilOutSrc<T, N, TX, MP>{bc(c), sh, iy, x0, f >= 3},
-                                     ColOut<T, N, TX, MP>{a.out[0] + f * fstride, iy, x0}, bc(2), tws);
-      __syncthreads();
-    }
-  } else {
+
+  // 3) inverse z transforms of S_next and of i kz S_next (x and y components) per output
+  if constexpr (NOC != 0) {
     for (int o = 0; o < nOut; ++o) {
-      for (int f = 0; f < 5; ++f) {
-        const int c = f < 3 ? f : f - 3;
-        cfft<T, N, 1, TX, NT, true, 1, C::RZ>(PencilOutSrc<T, N, TX, MP>{bc(c), a.osh[o], iy, x0, f >= 3},
-                                       ColOut<T, N, TX, MP>{a.out[o] + f * fstride, iy, x0}, b3, tws);
+      cpx<T> oxy = mk<T>(1, 0);
+      const cpx<T>* sh = pre ? nullptr : a.osh[o];
+      if (sh && act) oxy = cmul_fixed(MP::ld(&sh[kx]), MP::ld(&sh[N + iy]));
+      // `cnt` fields f0 .. through the tiles: first stage of each from the registers, then the rest
+      auto batch = [&](auto f0c, auto cntc) {
+        constexpr int f0 = decltype(f0c)::v, cnt = decltype(cntc)::v;
+        if (act) {
+#pragma unroll
+          for (int q = 0; q < cnt; ++q) {
+            cpx<T> t[f];
+#pragma unroll
+            for (int r = 0; r < f; ++r) {
+              t[r] = v[f0 + q < 3 ? f0 + q : f0 + q - 3][r];
+              if (NOC == 2 && sh) t[r] = cmul_fixed(t[r], cmul_fixed(oxy, MP::ld(&sh[2 * N + j + r * NB0])));
+              if (f0 >= 3) t[r] = mul_si(t[r], (T)kof(j + r * NB0, N));
+            }
+            DFT<T, f>::run(t, T(1));
+            const int i = q * TS + X::at(line, j * f);
+#pragma unroll
+            for (int r = 0; r < f; ++r) buf[i + r * TX] = t[r];
+          }
+        }
         __syncthreads();
-      }
+        mid_stages<T, N, PL, 1, nst - 1, 1, X, TX, cnt, NT, true>(buf, TS, tws);
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+          const int p = j + NB0 * i;  // last-stage butterfly
+          if (!act || (!FUSE && p >= NBL)) break;
+          cpx<T> w[l], t[2][l];
+          reg_twiddles<T, N, l, NBL, 1>(w, tws, p);
+          auto last = [&](cpx<T>* u, int q) {
+            const int o = q * TS + X::at(line, p);
+#pragma unroll
+            for (int r = 0; r < l; ++r) u[r] = buf[o + r * X::step(NBL)];
+            twiddle_dft<T, l>(u, w, T(1));
+          };
+          const size_t g = ((size_t)p * N + iy) * M + kx;
+          last(t[0], 0);
+          last(t[1], 1);
+          if (a.pairs) {
+            cpair<T>* dst = reinterpret_cast<cpair<T>*>(a.out[o] + f0 * fstride) + g;
+#pragma unroll
+            for (int r = 0; r < l; ++r) MP::stp(dst + r * NBL * ZS, t[0][r], t[1][r]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+              for (int r = 0; r < l; ++r) MP::st(a.out[o] + (f0 + q) * fstride + g + r * NBL * ZS, t[q][r]);
+          }
+          if (cnt == 3) {
+            last(t[0], 2);
+#pragma unroll
+            for (int r = 0; r < l; ++r) MP::st(a.out[o] + 2 * fstride + g + r * NBL * ZS, t[0][r]);
+          }
+        }
+        __syncthreads();
+      };
+      batch(IntC<0>{}, IntC<3>{});
+      batch(IntC<3>{}, IntC<2>{});
     }
   }
 }
 
-// the two-input variant holds 4 shared tiles (3 blocks per SM at most): it is given the
-// registers of 2 resident blocks rather than spill
 // EP: the one-input variant that also stores the tile's energy sums (a.epart non-null)
 // MC: the stage mode at compile time (the Rogallo stages) or -1 (a.mode); V: tile variant
 template <typename T, int N, int NFC, int NOC, bool EP = false, int MC = -1, int V = 0>
-__global__ void __launch_bounds__(K2Cfg<T, N, V>::NTP, (NFC == 2 || (NFC == 1 && NS_PENCIL_STAGE_STATE))
-                                                            ? cmin(2, K2Cfg<T, N, V>::MINB_P)
-                                                            : K2Cfg<T, N, V>::MINB_P)
+__global__ void __launch_bounds__(K2Cfg<T, N, V>::NTP, NFC == 2 ? K2Cfg<T, N, V>::MINB_P2 : K2Cfg<T, N, V>::MINB_P)
     k2_pencil(PencilArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pencil_tile<T, N, MemNC, NFC, NOC, EP, MC, V>(a, blockIdx.x, reinterpret_cast<cpx<T>*>(smem_raw));
 }
 
 // ---- slab pass: y transforms --------------------------------------------------------
-// field F of the spectral-in-xy pair (u, omega) formed on the fly from the mixed fields
-// staged in shared memory ([slot][e][line], TY lines): slots 0, 1, 2 hold u_x, u_y, u_z,
-// then d_z u_x and d_z u_y replace u_x and u_y in slots 0 and 1 once those are transformed.
-template <typename T, int N, int F, int TY>
-struct YInvSrc {
-  const cpx<T>* m;
-  int x0;
-  __device__ __forceinline__ cpx<T> get(int line, int e) const {
-    constexpr int fs = lf_rows<T, TY>(N) * TY;
-    const int i = lf_idx<T, TY>(e, line);
-    const T kx = (T)(x0 + line), ky = (T)kof(e, N);
-    if (F == 0) return m[i];
-    if (F == 1) return m[i + fs];
-    if (F == 2) return m[i + 2 * fs];
-    if (F == 3) return mul_si(m[i + 2 * fs], ky) - m[i + fs];       // i ky u_z - d_z u_y
-    if (F == 4) return m[i] - mul_si(m[i + 2 * fs], kx);            // d_z u_x - i kx u_z
-    return mul_si(m[i + fs], kx) - mul_si(m[i], ky);                // i kx u_y - i ky u_x
-  }
-};
-template <typename T, int N, class MP>
-struct ScrCol {  // one field [plane][y|ky][kx], column tile of a plane (scratch or Ft)
-  cpx<T>* p;
-  int zg, x0;
-  __device__ __forceinline__ cpx<T> get(int line, int e) const {
-    return MP::ldw(&p[((size_t)zg * N + e) * (N / 2) + x0 + line]);
-  }
-  __device__ __forceinline__ void put(int line, int e, cpx<T> v) const {
-    MP::st(&p[((size_t)zg * N + e) * (N / 2) + x0 + line], v);
-  }
-};
-
-// One output field of the y-inverse.  IP: the field's only input is slot SLOT, which the
-// transform then uses as its work tile (its inputs are read before the tile is written);
-// otherwise the transform goes through the work tile W.
-template <typename T, int N, int F, class MP, int TY, int NT, bool IP = false>
-__device__ __forceinline__ void yinv_field(const SlabArgs<T>& a, cpx<T>* in, cpx<T>* W, int zg,
-                                           int x0, size_t sstride, const cpx<T>* tws) {
-  using C = K2Cfg<T, N>;
-  const YInvSrc<T, N, F, TY> src{in, x0};
-  const ScrCol<T, N, MP> dst{a.scr + F * sstride, zg, x0};
-  if constexpr (IP)
-    cfft_src_in_work<T, N, 1, TY, NT, true, 1, C::RYI>(src, dst, in + F * (lf_rows<T, TY>(N) * TY), tws);
-  else
-    cfft<T, N, 1, TY, NT, true, 1, C::RYI>(src, dst, W, tws);
-  __syncthreads();
+// Scratch of the slab pass (SlabArgs::scr), per plane group: three arrays [plane][y][kx] of
+// pairs of modes, (u_x, u_y), (u_z, omega_x), (omega_y, omega_z), the pairs that share a line of
+// the x rows, so the x rows load and store 16 bytes (FP32) per mode.  The x rows leave the
+// products (f_0, f_1) in the first array and f_2 in the first half of each row of the second.
+// Columns (kx, ky) that hold modes of the truncation or of the forcing table (fK < 0: none).
+// Outside them the nonlinear term and the forcing vanish, so no pass reads the products there.
+template <typename T>
+__device__ __forceinline__ bool column_kept(const SlabArgs<T>& a, int kx, int ky) {
+  const bool in = a.trunc == 1 ? (kx <= a.Kimax && abs(ky) <= a.Kimax) : kx * kx + ky * ky <= a.K2max;
+  return in || (a.fK >= 0 && kx <= a.fK && abs(ky) <= a.fK);
 }
 
-// One tile: TYI consecutive kx of plane zg, in 4 shared tiles (3 input slots and a work tile).
-// u_x, u_y, u_z are staged first; omega_z (from u_x, u_y) goes through the work tile, u_x and
-// u_y are transformed in place, and d_z u_x, d_z u_y are then copied into their slots while the
-// next transform runs; omega_y, omega_x and u_z (in place) follow.
-// TY_, NT_: tile width and threads (the defaults of the size; the slab pipeline uses 4 columns)
-template <typename T, int N, class MP, int TY_ = K2Cfg<T, N>::TYI, int NT_ = K2Cfg<T, N>::NTYI>
-__device__ __forceinline__ void yinv_tile(const SlabArgs<T>& a, int tx, int zg, cpx<T>* in) {
-  constexpr int M = N / 2, TY = TY_, NT = NT_, tile = lf_rows<T, TY>(N) * TY;
-  cpx<T>* W = in + 3 * tile;
-  cpx<T>* tws = in + 4 * tile;
-  const int x0 = tx * TY, z = a.z0 + zg;
-  const size_t sstride = (size_t)a.G * N * M;
+// One tile: W consecutive kx of plane zg.  Inverse y transforms of u and omega = i k x u, formed
+// in registers from the mixed fields (u_x, u_y, u_z, d_z u_x, d_z u_y; interleaved layout).
+// Bound by HBM (5 fields read, 6 written).  The first stage reads global memory and the last
+// one writes it, so each line passes through shared memory once per middle stage and once
+// between them; two batches of three lines share three tiles and one set of twiddles.  Measured,
+// 128 planes, FP32: 256^3 59.6 us = 6.2 TB/s (68.7 with the inputs staged in shared memory), 512^3
+// 279 (380), 384^3 145 (181).
+template <typename T, int N, class MP, int W>
+__device__ __forceinline__ void yinv_tile(const SlabArgs<T>& a, int tx, int zg, cpx<T>* buf) {
+  using PL = YPlan<T, N>;
+  constexpr int M = N / 2, nst = PL::P.nst, f = PL::P.r[0], l = PL::P.r[nst - 1], NB0 = N / f, NBL = N / l;
+  constexpr int NT = W * NB0, K = (f + l - 1) / l;  // K last-stage butterflies p = j + NB0 i per thread
+  using X = Xchg<T, N, f, W, true>;
+  constexpr int TS = X::elems;
+  cpx<T>* tws = buf + 3 * TS;
+  const int tid = threadIdx.x, line = tid % W, j = tid / W;
+  const int x0 = tx * W, kx = x0 + line, z = a.z0 + zg;
   const size_t fs = (size_t)N * N * M;
-  for (int f = 0; f < 3; ++f) stage_col_tile<T, N, TY, NT, true>(in + f * tile, a.mixed + f * fs, z, x0);
-  cp_async_commit();
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tws[tw_pad(i)] = ldg(&a.tw[i]);
-  cp_async_wait_pending<0>();
-  __syncthreads();
-  yinv_field<T, N, 5, MP, TY, NT>(a, in, W, zg, x0, sstride, tws);        // omega_z
-  yinv_field<T, N, 0, MP, TY, NT, true>(a, in, W, zg, x0, sstride, tws);  // u_x in slot 0
-  stage_col_tile<T, N, TY, NT, true>(in, a.mixed + 3 * fs, z, x0);        // d_z u_x -> slot 0
-  cp_async_commit();
-  yinv_field<T, N, 1, MP, TY, NT, true>(a, in, W, zg, x0, sstride, tws);  // u_y in slot 1
-  stage_col_tile<T, N, TY, NT, true>(in + tile, a.mixed + 4 * fs, z, x0); // d_z u_y -> slot 1
-  cp_async_commit();
-  cp_async_wait_pending<1>();
-  __syncthreads();
-  yinv_field<T, N, 4, MP, TY, NT>(a, in, W, zg, x0, sstride, tws);        // omega_y
-  cp_async_wait_pending<0>();
-  __syncthreads();
-  yinv_field<T, N, 3, MP, TY, NT>(a, in, W, zg, x0, sstride, tws);        // omega_x
-  yinv_field<T, N, 2, MP, TY, NT, true>(a, in, W, zg, x0, sstride, tws);  // u_z in slot 2
-}
-
-template <typename T, int N, int V = 0>
-__global__ void __launch_bounds__(K2Cfg<T, N, V>::NTYI) k2_yinv(SlabArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  yinv_tile<T, N, MemNC, K2Cfg<T, N, V>::TYI, K2Cfg<T, N, V>::NTYI>(a, blockIdx.x, blockIdx.y,
-                                                                  reinterpret_cast<cpx<T>*>(smem_raw));
-}
-
-#ifndef NS_FT_SKIP
-#define NS_FT_SKIP 1
-#endif
-// Ft output of the forward y transforms: a mode is stored unless every pencil tile of
-// a.skip_tx columns that holds it lies outside the truncation and the forcing block (the
-// criterion of pencil_tile_truncated with x0 the tile's first column): the pencil passes
-// neither load nor transform such tiles.
-template <typename T, int N, class MP>
-struct FtColOut {
-  cpx<T>* p;
-  int z, x0;
-  const SlabArgs<T>* a;
-  __device__ __forceinline__ void put(int line, int e, cpx<T> v) const {
-    if (a->skip_tx > 0) {
-      const int kx = x0 + line, px = kx - kx % a->skip_tx, ky = kof(e, N);
-      const bool out = a->trunc == 1 ? (px > a->Kimax || abs(ky) > a->Kimax) : px * px + ky * ky > a->K2max;
-      const bool forced = a->fK >= 0 && px <= a->fK && abs(ky) <= a->fK;
-      if (out && !forced) return;
+  const bool act = tid < NT;
+  const T fx = (T)kx;
+  auto ky = [&](int r) { return (T)kof(j + r * NB0, N); };
+  auto stage0 = [&](cpx<T>* v, int t) {  // radix-f butterfly into tile t
+    DFT<T, f>::run(v, T(1));
+    const int o = t * TS + X::at(line, j * f);
+#pragma unroll
+    for (int r = 0; r < f; ++r) buf[o + r * W] = v[r];
+  };
+  const size_t sstride = (size_t)a.G * N * M;
+  cpair<T>* dst = reinterpret_cast<cpair<T>*>(a.scr) + (size_t)zg * N * M + kx;
+  auto load2 = [&](cpx<T>* va, cpx<T>* vb, int c) {  // two interleaved fields
+    const cpair<T>* p = reinterpret_cast<const cpair<T>*>(a.mixed + c * fs) + ((size_t)z * N + j) * M + kx;
+#pragma unroll
+    for (int r = 0; r < f; ++r) MP::ldp(p + (size_t)r * NB0 * M, va[r], vb[r]);
+  };
+  // last stage of the lines in the tiles: pair `pr` from tiles 0 and 1, and tile 2 into wz (pr = 0)
+  // or, with wz, pair 2 (pr = 1)
+  cpx<T> wz[K][l];
+  auto last = [&](int pr) {
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const int p = j + NB0 * i;
+      if (!act || (f % l != 0 && p >= NBL)) break;
+      cpx<T> w[l], va[l], vb[l];
+      reg_twiddles<T, N, l, NBL, 1>(w, tws, p);
+      auto line_of = [&](cpx<T>* v, int t) {
+        const int o = t * TS + X::at(line, p);
+#pragma unroll
+        for (int r = 0; r < l; ++r) v[r] = buf[o + r * X::step(NBL)];
+        twiddle_dft<T, l>(v, w, T(1));
+      };
+      line_of(va, 0);
+      line_of(vb, 1);
+      cpair<T>* d = dst + pr * sstride + (size_t)p * M;
+#pragma unroll
+      for (int r = 0; r < l; ++r) MP::stp(d + (size_t)r * NBL * M, va[r], vb[r]);
+      if (pr == 0) {
+        line_of(wz[i], 2);
+      } else {
+        line_of(va, 2);
+#pragma unroll
+        for (int r = 0; r < l; ++r) MP::stp(d + sstride + (size_t)r * NBL * M, va[r], wz[i][r]);
+      }
     }
-    MP::st(&p[((size_t)z * N + e) * (N / 2) + x0 + line], v);
-  }
-};
+  };
 
-template <typename T, int N, class MP, int V = 0>
-__device__ __forceinline__ void yfwd_tile(const SlabArgs<T>& a, int tx, int zg, cpx<T>* W) {
-  using C = K2Cfg<T, N, V>;
-  const int x0 = tx * C::TY, z = a.z0 + zg;
-  const size_t sstride = (size_t)a.G * N * (N / 2);
-  const size_t fstride = (size_t)N * N * (N / 2);
-  cpx<T>* tws = W + lf_rows<T, C::TY>(N) * C::TY;
-  load_twiddles(tws, a.tw, N);
-  for (int f = 0; f < 3; ++f) {
-    cfft<T, N, 1, C::TY, C::NTY, true, -1, C::RYF>(ScrCol<T, N, MP>{a.scr + f * sstride, zg, x0},
-                                                   FtColOut<T, N, MP>{a.Ft + f * fstride, z, x0, &a}, W, tws);
-    __syncthreads();
+  cpx<T> ux[f], uy[f];
+  if (act) load2(ux, uy, 0);
+  for (int i = tid; i < N; i += blockDim.x) tws[tw_pad(i)] = ldg(&a.tw[i]);
+  if (act) {
+    cpx<T> v[f];
+#pragma unroll
+    for (int r = 0; r < f; ++r) v[r] = mul_si(uy[r], fx) - mul_si(ux[r], ky(r));  // i kx u_y - i ky u_x
+    stage0(ux, 0);
+    stage0(uy, 1);
+    stage0(v, 2);
+  }
+  __syncthreads();
+  mid_stages<T, N, PL, 1, nst - 1, 1, X, W, 3, NT, true>(buf, TS, tws);
+  cpx<T> uz[f], dx[f], dy[f];
+  if (act) {
+    const cpx<T>* src = a.mixed + 2 * fs + ((size_t)z * N + j) * M + kx;
+#pragma unroll
+    for (int r = 0; r < f; ++r) uz[r] = MP::ld(src + (size_t)r * NB0 * M);
+    load2(dx, dy, 3);
+  }
+  last(0);
+  __syncthreads();
+  if (act) {
+#pragma unroll
+    for (int r = 0; r < f; ++r) {
+      dy[r] = mul_si(uz[r], ky(r)) - dy[r];  // i ky u_z - d_z u_y
+      dx[r] = dx[r] - mul_si(uz[r], fx);     // d_z u_x - i kx u_z
+    }
+    stage0(uz, 0);
+    stage0(dy, 1);
+    stage0(dx, 2);
+  }
+  __syncthreads();
+  mid_stages<T, N, PL, 1, nst - 1, 1, X, W, 3, NT, true>(buf, TS, tws);
+  last(1);
+}
+
+template <typename T, int N, int V = 0>
+__global__ void __launch_bounds__(K2Cfg<T, N, V>::NTYI, K2Cfg<T, N, V>::MINB_YI) k2_yinv(SlabArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  yinv_tile<T, N, MemNC, K2Cfg<T, N, V>::TYI>(a, blockIdx.x, blockIdx.y, reinterpret_cast<cpx<T>*>(smem_raw));
+}
+
+// One tile: W consecutive kx of plane zg.  Forward y transforms of the three products, the
+// first stage from the scratch, the last one into Ft, where a mode is stored unless its column
+// is outside the truncation (a.skip: no pencil pass uses it).  Bound by HBM.
+template <typename T, int N, class MP, int W>
+__device__ __forceinline__ void yfwd_tile(const SlabArgs<T>& a, int tx, int zg, cpx<T>* buf) {
+  using PL = YPlan<T, N>;
+  constexpr int M = N / 2, nst = PL::P.nst, f = PL::P.r[0], l = PL::P.r[nst - 1], NB0 = N / f, NBL = N / l;
+  constexpr int NT = W * NB0, K = (f + l - 1) / l;
+  using X = Xchg<T, N, f, W, true>;
+  constexpr int TS = X::elems;
+  cpx<T>* tws = buf + 3 * TS;
+  const int tid = threadIdx.x, line = tid % W, j = tid / W;
+  const int x0 = tx * W, kx = x0 + line, z = a.z0 + zg;
+  const size_t sstride = (size_t)a.G * N * M, fs = (size_t)N * N * M;
+  const bool act = tid < NT;
+  if (act) {
+    cpx<T> v[3][f];
+    const cpair<T>* src = reinterpret_cast<const cpair<T>*>(a.scr) + ((size_t)zg * N + j) * M + kx;
+    const cpx<T>* src2 = reinterpret_cast<const cpx<T>*>(reinterpret_cast<const cpair<T>*>(a.scr) + sstride) +
+                         ((size_t)zg * N + j) * 2 * M + kx;
+#pragma unroll
+    for (int r = 0; r < f; ++r) {
+      MP::ldp(src + (size_t)r * NB0 * M, v[0][r], v[1][r]);
+      v[2][r] = MP::ldw(src2 + (size_t)r * NB0 * 2 * M);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      DFT<T, f>::run(v[c], T(-1));
+      const int o = c * TS + X::at(line, j * f);
+#pragma unroll
+      for (int r = 0; r < f; ++r) buf[o + r * W] = v[c][r];
+    }
+  }
+  for (int i = tid; i < N; i += blockDim.x) tws[tw_pad(i)] = ldg(&a.tw[i]);
+  __syncthreads();
+  mid_stages<T, N, PL, 1, nst - 1, -1, X, W, 3, NT, true>(buf, TS, tws);
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    const int p = j + NB0 * i;  // last-stage butterfly
+    if (!act || (f % l != 0 && p >= NBL)) break;
+    cpx<T> w[l], v[2][l];
+    reg_twiddles<T, N, l, NBL, -1>(w, tws, p);
+    bool keep[l];
+#pragma unroll
+    for (int r = 0; r < l; ++r) keep[r] = !a.skip || column_kept(a, kx, kof(p + r * NBL, N));
+    const size_t g = ((size_t)z * N + p) * M + kx;
+    auto last = [&](cpx<T>* u, int c) {
+      const int o = c * TS + X::at(line, p);
+#pragma unroll
+      for (int r = 0; r < l; ++r) u[r] = buf[o + r * X::step(NBL)];
+      twiddle_dft<T, l>(u, w, T(-1));
+    };
+    last(v[0], 0);
+    last(v[1], 1);
+    cpair<T>* dst = reinterpret_cast<cpair<T>*>(a.Ft) + g;
+#pragma unroll
+    for (int r = 0; r < l; ++r)
+      if (keep[r]) MP::stp(dst + (size_t)r * NBL * M, v[0][r], v[1][r]);
+    last(v[0], 2);
+#pragma unroll
+    for (int r = 0; r < l; ++r)
+      if (keep[r]) MP::st(a.Ft + 2 * fs + g + (size_t)r * NBL * M, v[0][r]);
   }
 }
 
 template <typename T, int N, int V = 0>
-__global__ void __launch_bounds__(K2Cfg<T, N, V>::NTY, 2) k2_yfwd(SlabArgs<T> a) {
+__global__ void __launch_bounds__(K2Cfg<T, N, V>::NTY, K2Cfg<T, N, V>::MINB_Y) k2_yfwd(SlabArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  yfwd_tile<T, N, MemNC, V>(a, blockIdx.x, blockIdx.y, reinterpret_cast<cpx<T>*>(smem_raw));
+  yfwd_tile<T, N, MemNC, K2Cfg<T, N, V>::TY>(a, blockIdx.x, blockIdx.y, reinterpret_cast<cpx<T>*>(smem_raw));
 }
 
 // ---- slab pass: x rows --------------------------------------------------------------
-#ifndef NS_XROW_PAIRS
-#define NS_XROW_PAIRS 1
-#endif
 // One tile: RX consecutive rows (plane, y) of the group.  Each row holds the half spectra
 // (kx < N/2, the Nyquist mode zero) of 6 real fields, and two real rows share one complex line
 // of length N: the line of fields a and b is z = a + i b, whose full spectrum is
 // Z[k] = A[k] + i B[k] and Z[N - k] = conj(A[k]) + i conj(B[k]) (A[0], B[0] real).  Inverse
 // lines per row: (u_x, u_y), (u_z, w_x), (w_y, w_z); the products come back as lines (f_0, f_1)
-// of every row and (f_2 of row q, f_2 of row q + RXh), whose forward transforms P split into
+// of every row and (f_2 of row q, f_2 of row q + RXH), whose forward transforms P split into
 // F_a[k] = (P[k] + conj(P[N - k])) / 2 and F_b[k] = (P[k] - conj(P[N - k])) / (2 i).  All
 // transforms are unnormalised, as the r2c / c2r pair they replace.
+//
+// What bounds it: shared memory, when every stage goes through it (27 accesses per line element
+// in six passes).  Here a thread takes the two first-stage butterflies j and N/f - j together:
+// their inputs are closed under k -> N - k, so the lines are formed from the modes in registers;
+// the last inverse butterflies, the products and the first forward butterfly of the points
+// x = j + (N/f) r share registers (see radix plans); and the pair (p, N/l - p) of the last forward
+// stage holds P[k] and P[N - k], which it splits and stores.  Shared memory sees each line once
+// per transform and middle stage.  The two rows of a pair sit in neighbouring lanes, and the even
+// lane takes the partner's third products.  One thread per row and N/f points; where a pair's
+// threads fit a warp, the warps do not wait for one another.  Measured on GB300, 128 planes, FP32:
+// 256^3 71.0 us (86.3 with every stage through shared memory), 512^3 293 (418), 384^3 195 (270),
+// 128^3 18.6 (22.6).  156 registers and 12 warps per SM beat 124 and 16 (71 against 80 us): the
+// loads in flight per thread hide more than further warps do.
 template <typename T, int N, class MP, int V = 0>
-__device__ __forceinline__ void xrow_tile(const SlabArgs<T>& a, int tile_id, cpx<T>* buf) {
+__device__ __forceinline__ void xrow_tile(const SlabArgs<T>& a, int tile_id, cpx<T>* smem) {
   using C = K2Cfg<T, N, V>;
-  constexpr int M = N / 2, RX = C::RX, NT = C::NTX, RXh = (RX + 1) / 2;
-  constexpr int NLI = 3 * RX, NLF = RX + RXh;  // inverse and forward lines
-  const WorkTile<T, N, NLI, false> L{buf};     // line p RX + r: pair p of row r
-  cpx<T>* tws = buf + C::XELEMS;
-  const bool act = threadIdx.x < NT;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tws[tw_pad(i)] = ldg(&a.tw[i]);
-  const int rows_total = a.G * N;
-  const int r0 = tile_id * RX;
-  const int nr = min(RX, rows_total - r0);
+  using PL = XPlan<T, N>;
+  constexpr int nst = PL::P.nst, f = PL::P.r[0], l = PL::P.r[nst - 1];  // outer and inner radix
+  constexpr int M = N / 2, NB0 = N / f, NBL = N / l, H = f / 2, IP0 = (NB0 + 1) / 2, IPL = NBL / 2;
+  constexpr bool ODD0 = NB0 % 2;  // (then j = 0 has no second self-mirrored butterfly)
+  constexpr bool FUSE = f % l == 0;
+  constexpr int K = f / l;                                      // last-stage butterflies per thread (FUSE)
+  constexpr int NP = C::XWP, NT = C::XGT, ROWS = 2 * NP;         // pairs, threads and rows of a group
+  constexpr int NLI = 3 * ROWS, NLF = ROWS + NP;                 // its inverse and forward lines
+  using X = Xchg<T, N, f, NLI, false>;
+  static_assert(f % 2 == 0 && NBL % 2 == 0, "modes k and N - k pair up");
+  cpx<T>* tws = smem + C::XELEMS;
+  // the twiddle table, on its way while the modes are loaded
+  constexpr int KT = (N + C::NTX - 1) / C::NTX;
+  cpx<T> twr[KT];
+#pragma unroll
+  for (int c = 0; c < KT; ++c) {
+    const int i = threadIdx.x + c * C::NTX;
+    twr[c] = (int)threadIdx.x < C::NTX && i < N ? ldg(&a.tw[i]) : mk<T>(0, 0);
+  }
+  const int grp = C::XWARP ? threadIdx.x / NT : 0, tid = C::XWARP ? threadIdx.x % NT : threadIdx.x;
+  const bool in = C::XWARP ? grp < C::XNG : true;  // (a wider block's other warps only pass barriers)
+  cpx<T>* buf = smem + (in ? grp : 0) * C::XGEL;
+  auto sync = [] {
+    if constexpr (C::XWARP) __syncwarp();
+    else __syncthreads();
+  };
+  // local row 2 q + h is row grp NP + q + h RXH of the tile (the last pair of an odd tile has one)
+  const int r0 = tile_id * C::RX, nr = in ? min(C::RX, a.G * N - r0) : 0;
+  auto row_of = [&](int lr) {
+    const int row = grp * NP + (lr >> 1) + (lr & 1) * C::RXH;
+    return row < nr && (lr & 1 ? row < C::RX : row < C::RXH) ? row : -1;
+  };
   const size_t sstride = (size_t)a.G * N * M;
 
-  // FP32 with NT a multiple of M / 2: every thread keeps one pair of modes (k, k + 1) and
-  // walks lines, so the loads and stores are 16 bytes wide and its indices loop-invariant
-  constexpr int H = M / 2;
-  constexpr bool PAIR = NS_XROW_PAIRS && sizeof(T) == 4 && NT % H == 0;
-  constexpr int GP = PAIR ? NT / H : 1;  // lines in flight per pass of the block
-  const int kp2 = 2 * (threadIdx.x % H), g0 = threadIdx.x / H;
-  if constexpr (PAIR) {
-    // 1) item (line = p RX + row, k pair): modes k, k + 1 of fields 2p and 2p + 1 give Z[k],
-    //    Z[k + 1], Z[N - k], Z[N - k - 1] of the line (k = 0: Z[0] from the real parts and
-    //    Z[M] = 0); all loads first, rows past the end of the group are zero
-    constexpr int KC = (NLI + GP - 1) / GP;
-    float4 xa[KC], xb[KC];
+  // 1) item (line p ROWS + row, pair h): the modes of both butterflies, their radix-f transforms
+  for (int i = tid; i < NLI * IP0 && tid < NT && in; i += NT) {
+    const int line = i / IP0, h = i % IP0, p = line / ROWS, row = row_of(line % ROWS);
+    const int j0 = h, j1 = h == 0 ? (ODD0 ? 0 : NB0 / 2) : NB0 - h;
+    cpx<T> v0[f], v1[f], m0[H], m1[H], b0[H], b1[H];
+    const cpair<T>* src = reinterpret_cast<const cpair<T>*>(a.scr) + p * sstride + (size_t)(r0 + row) * M;
 #pragma unroll
-    for (int c = 0; c < KC; ++c) {
-      const int line = g0 + c * GP, p = line / RX, row = line % RX;
-      xa[c] = xb[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (act && (NLI % GP == 0 || line < NLI) && row < nr) {
-        const cpx<float>* src = reinterpret_cast<const cpx<float>*>(a.scr) + 2 * p * sstride + (size_t)(r0 + row) * M + kp2;
-        xa[c] = MP::ld2(src);
-        xb[c] = MP::ld2(src + sstride);
+    for (int r = 0; r < H; ++r) {
+      v0[r] = v1[r] = b0[r] = b1[r] = mk<T>(0, 0);
+      if (row >= 0) {
+        MP::ldp(src + j0 + r * NB0, v0[r], b0[r]);
+        MP::ldp(src + j1 + r * NB0, v1[r], b1[r]);
       }
     }
 #pragma unroll
-    for (int c = 0; c < KC; ++c) {
-      const int line = g0 + c * GP;
-      if (act && (NLI % GP == 0 || line < NLI)) {
-        const float4 A = xa[c], B = xb[c];
-        if (kp2 == 0) {
-          L.put(line, 0, mk<T>(A.x, B.x));
-          L.put(line, M, mk<T>(0, 0));
-        } else {
-          L.put(line, kp2, mk<T>(A.x - B.y, A.y + B.x));
-          L.put(line, N - kp2, mk<T>(A.x + B.y, B.x - A.y));
-        }
-        L.put(line, kp2 + 1, mk<T>(A.z - B.w, A.w + B.z));
-        L.put(line, N - kp2 - 1, mk<T>(A.z + B.w, B.z - A.w));
-      }
+    for (int r = 0; r < H; ++r) {
+      const cpx<T> A = v0[r], B = b0[r], D = v1[r], E = b1[r];
+      v0[r] = mk<T>(A.x - B.y, A.y + B.x);  // A + i B
+      m0[r] = mk<T>(A.x + B.y, B.x - A.y);  // conj(A) + i conj(B)
+      if (r == 0 && h == 0) v0[0] = mk<T>(A.x, B.x);
+      v1[r] = mk<T>(D.x - E.y, D.y + E.x);
+      m1[r] = mk<T>(D.x + E.y, E.x - D.y);
     }
-  } else {
-  // 1) item (p, row, k) reads mode k of fields 2p and 2p + 1 and writes Z[k] and Z[N - k] of
-  //    line p RX + row (k = 0: Z[0] from the real parts and Z[M] = 0).  Every load is issued
-  //    before any store; rows past the end of the group are zero.
-  constexpr int NI = 3 * RX * M, KI = (NI + NT - 1) / NT;
-  cpx<T> xa[KI], xb[KI];
 #pragma unroll
-  for (int c = 0; c < KI; ++c) {
-    const int i = threadIdx.x + c * NT;
-    xa[c] = xb[c] = mk<T>(0, 0);
-    if (act && (NI % NT == 0 || i < NI)) {
-      const int p = i / (RX * M), row = (i / M) % RX, k = i % M;
-      if (row < nr) {
-        const cpx<T>* src = a.scr + 2 * p * sstride + (size_t)(r0 + row) * M + k;
-        xa[c] = MP::ld(src);
-        xb[c] = MP::ld(src + sstride);
-      }
+    for (int r = 0; r < H; ++r) {  // the mirrored halves: from each other, or (h = 0) from themselves
+      const cpx<T> s = r == 0 ? mk<T>(0, 0) : m0[H - r];
+      v0[H + r] = h == 0 ? s : m1[H - 1 - r];
+      v1[H + r] = h == 0 ? m1[H - 1 - r] : m0[H - 1 - r];
+    }
+    DFT<T, f>::run(v0, T(1));
+    const int o0 = X::at(line, j0 * f);
+#pragma unroll
+    for (int r = 0; r < f; ++r) buf[o0 + r] = v0[r];
+    if (!ODD0 || h > 0) {
+      DFT<T, f>::run(v1, T(1));
+      const int o1 = X::at(line, j1 * f);
+#pragma unroll
+      for (int r = 0; r < f; ++r) buf[o1 + r] = v1[r];
     }
   }
 #pragma unroll
-  for (int c = 0; c < KI; ++c) {
-    const int i = threadIdx.x + c * NT;
-    if (act && (NI % NT == 0 || i < NI)) {
-      const int p = i / (RX * M), row = (i / M) % RX, k = i % M;
-      const int line = p * RX + row;
-      const cpx<T> A = xa[c], B = xb[c];
-      if (k == 0) {
-        L.put(line, 0, mk<T>(A.x, B.x));
-        L.put(line, M, mk<T>(0, 0));
+  for (int c = 0; c < KT; ++c) {
+    const int i = threadIdx.x + c * C::NTX;
+    if ((int)threadIdx.x < C::NTX && i < N) tws[tw_pad(i)] = twr[c];
+  }
+  __syncthreads();
+  mid_stages<T, N, PL, 1, FUSE ? nst - 1 : nst, 1, X, NLI, 1, NT, false>(buf, 0, tws);
+
+  // 2) item (row 2 q + h, points x = j + NB0 r): last inverse stage of the row's 3 lines, the
+  //    products, first forward stage of (f_0, f_1) and (even lane) of the pair's f_2 line
+  const bool act = in && tid < ROWS * NB0;  // (the other lanes of its last warp repeat its last pair)
+  const int it = act ? tid : ROWS * NB0 - 2 + (tid & 1);
+  const int h = it & 1, j = (it >> 1) % NB0, q = (it >> 1) / NB0, lr = 2 * q + h;
+  T um[3] = {T(0), T(0), T(0)};  // max |u_i| over the rows (CFL), padding rows are zero
+  cpx<T> g[f], y[f];
+  if (in && tid < (ROWS * NB0 + 31) / 32 * 32) {
+    cpx<T> z0[f], z1[f], z2[f];
+    if constexpr (FUSE) {
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        const int p = j + NB0 * i;
+        cpx<T> w[l];
+        reg_twiddles<T, N, l, NBL, 1>(w, tws, p);
+        const int o = X::at(lr, p);
+        auto last = [&](cpx<T>* z, int line0) {
+          cpx<T> t[l];
+#pragma unroll
+          for (int r = 0; r < l; ++r) t[r] = buf[o + line0 * X::LS + r * X::step(NBL)];
+          twiddle_dft<T, l>(t, w, T(1));
+#pragma unroll
+          for (int r = 0; r < l; ++r) z[i + K * r] = t[r];
+        };
+        last(z0, 0);
+        last(z1, ROWS);
+        last(z2, 2 * ROWS);
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < f; ++r) {
+        const int o = X::at(lr, j + r * NB0);
+        z0[r] = buf[o];
+        z1[r] = buf[o + ROWS * X::LS];
+        z2[r] = buf[o + 2 * ROWS * X::LS];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < f; ++r) {
+      const T ux = z0[r].x, uy = z0[r].y, uz = z1[r].x, wx = z1[r].y, wy = z2[r].x, wz = z2[r].y;
+      um[0] = fmax(um[0], fabs(ux));
+      um[1] = fmax(um[1], fabs(uy));
+      um[2] = fmax(um[2], fabs(uz));
+      g[r] = mk<T>(uy * wz - uz * wy, uz * wx - ux * wz);
+      const T f2 = ux * wy - uy * wx;
+      y[r] = mk<T>(f2, __shfl_xor_sync(0xffffffffu, f2, 1));
+    }
+    DFT<T, f>::run(g, T(-1));
+    if (h == 0) DFT<T, f>::run(y, T(-1));
+  }
+  sync();
+  if (act) {
+    const int o0 = X::at(lr, j * f), o1 = X::at(ROWS + q, j * f);
+#pragma unroll
+    for (int r = 0; r < f; ++r) buf[o0 + r] = g[r];
+    if (h == 0)
+#pragma unroll
+      for (int r = 0; r < f; ++r) buf[o1 + r] = y[r];
+  }
+  sync();
+  if (a.umax) block_max3<T>(um[0], um[1], um[2], reinterpret_cast<T*>(smem + C::XNG * C::XGEL), a.umax);
+  mid_stages<T, N, PL, 1, nst - 1, -1, X, NLF, 1, NT, false>(buf, 0, tws);
+
+  // 3) item (line, pair hh): last forward stage of both butterflies, split and stored
+  for (int i = tid; i < NLF * IPL && tid < NT && in; i += NT) {
+    const int line = i / IPL, hh = i % IPL;
+    const int p0 = hh, p1 = hh == 0 ? NBL / 2 : NBL - hh;
+    const bool own = line < ROWS;  // (f_0, f_1) of a row, else f_2 of a pair's rows
+    const int ra = row_of(own ? line : 2 * (line - ROWS)), rb = own ? -1 : row_of(2 * (line - ROWS) + 1);
+    cpx<T> v0[l], v1[l];
+    {
+      cpx<T> w[l];
+      reg_twiddles<T, N, l, NBL, -1>(w, tws, p0);
+      const int i0 = X::at(line, p0), i1 = X::at(line, p1);
+#pragma unroll
+      for (int r = 0; r < l; ++r) v0[r] = buf[i0 + r * X::step(NBL)];
+      twiddle_dft<T, l>(v0, w, T(-1));
+      reg_twiddles<T, N, l, NBL, -1>(w, tws, p1);
+#pragma unroll
+      for (int r = 0; r < l; ++r) v1[r] = buf[i1 + r * X::step(NBL)];
+      twiddle_dft<T, l>(v1, w, T(-1));
+    }
+    cpair<T>* d01 = reinterpret_cast<cpair<T>*>(a.scr) + (size_t)r0 * M;
+    cpx<T>* d2 = reinterpret_cast<cpx<T>*>(d01 + sstride);
+    auto put = [&](int k, cpx<T> P, cpx<T> Q) {  // P = P[k], Q = P[N - k]
+      if (k >= M) return;
+      const cpx<T> A = mk<T>(T(0.5) * (P.x + Q.x), T(0.5) * (P.y - Q.y));
+      const cpx<T> B = mk<T>(T(0.5) * (P.y + Q.y), T(0.5) * (Q.x - P.x));
+      if (own) {
+        if (ra >= 0) MP::stp(d01 + (size_t)ra * M + k, A, B);
       } else {
-        L.put(line, k, mk<T>(A.x - B.y, A.y + B.x));      // A + i B
-        L.put(line, N - k, mk<T>(A.x + B.y, B.x - A.y));  // conj(A) + i conj(B)
+        if (ra >= 0) MP::st(d2 + (size_t)ra * 2 * M + k, A);
+        if (rb >= 0) MP::st(d2 + (size_t)rb * 2 * M + k, B);
       }
-    }
-  }
-  }
-  __syncthreads();
-  // 2) the 3 RX inverse transforms in one in-place call
-  cfft_ip<T, N, 1, NLI, NT, false, 1, true, C::RXR>(L, buf, tws);
-  __syncthreads();
-
-  // 3) u x omega: item (q, x) takes rows q and q + RXh (when RX is odd the last q has one) at
-  //    point x, writes (f_0, f_1) over each row's first line and (f_2(q), f_2(q + RXh)) over
-  //    line RX + q (row q's second line): every line it writes is one it has read
-  T m[3] = {T(0), T(0), T(0)};  // max |u_i| over the rows (CFL), padding rows are zero
-  for (int i = threadIdx.x; act && i < RXh * N; i += NT) {
-    const int q = i / N, x = i % N;
-    T f2[2] = {T(0), T(0)};
+    };
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int row = q + h * RXh;
-      if (row < RX) {
-        const cpx<T> z0 = L.get(row, x), z1 = L.get(RX + row, x), z2 = L.get(2 * RX + row, x);
-        const T ux = z0.x, uy = z0.y, uz = z1.x, wx = z1.y, wy = z2.x, wz = z2.y;
-        m[0] = fmax(m[0], fabs(ux));
-        m[1] = fmax(m[1], fabs(uy));
-        m[2] = fmax(m[2], fabs(uz));
-        L.put(row, x, mk<T>(uy * wz - uz * wy, uz * wx - ux * wz));
-        f2[h] = ux * wy - uy * wx;
-      }
+    for (int r = 0; r < (l + 1) / 2; ++r) {  // (elements r > l / 2 have k >= N / 2)
+      put(p0 + r * NBL, v0[r], hh == 0 ? v0[(l - r) % l] : v1[l - 1 - r]);
+      put(p1 + r * NBL, v1[r], hh == 0 ? v1[l - 1 - r] : v0[l - 1 - r]);
     }
-    L.put(RX + q, x, mk<T>(f2[0], f2[1]));
-  }
-  __syncthreads();
-  // lines NLF .. 3 RX - 1 are free now
-  if (a.umax) block_max3<T>(m[0], m[1], m[2], reinterpret_cast<T*>(buf + NLF * L.LS), a.umax);
-  // 4) the NLF forward transforms of the products
-  cfft_ip<T, N, 1, NLF, NT, false, -1, true, C::RXR>(WorkTile<T, N, NLF, false>{buf}, buf, tws);
-  __syncthreads();
-
-  // 5) split and store: item (line, k), k < M (pairs of modes in the FP32 layout above)
-  if constexpr (PAIR) {
-#pragma unroll
-    for (int c = 0; c < (NLF + GP - 1) / GP; ++c) {
-      const int line = g0 + c * GP;
-      if (!act || (NLF % GP != 0 && line >= NLF)) break;
-      const cpx<T> P0 = L.get(line, kp2), Q0 = L.get(line, kp2 == 0 ? 0 : N - kp2);
-      const cpx<T> P1 = L.get(line, kp2 + 1), Q1 = L.get(line, N - kp2 - 1);
-      const float4 Fa = make_float4(0.5f * (P0.x + Q0.x), 0.5f * (P0.y - Q0.y), 0.5f * (P1.x + Q1.x), 0.5f * (P1.y - Q1.y));
-      const float4 Fb = make_float4(0.5f * (P0.y + Q0.y), 0.5f * (Q0.x - P0.x), 0.5f * (P1.y + Q1.y), 0.5f * (Q1.x - P1.x));
-      const bool own = line < RX;
-      const int ra = own ? line : line - RX, rb = own ? line : line - RX + RXh;
-      const int fa = own ? 0 : 2, fb = own ? 1 : 2;
-      cpx<float>* scr = reinterpret_cast<cpx<float>*>(a.scr);
-      if (ra < nr) MP::st2(&scr[fa * sstride + (size_t)(r0 + ra) * M + kp2], Fa);
-      if (rb < nr) MP::st2(&scr[fb * sstride + (size_t)(r0 + rb) * M + kp2], Fb);
-    }
-    return;
-  }
-  constexpr int NO = NLF * M;
-  for (int i = threadIdx.x; act && i < NO; i += NT) {
-    const int line = i / M, k = i % M;
-    const cpx<T> P = L.get(line, k), Q = L.get(line, k == 0 ? 0 : N - k);
-    const cpx<T> Fa = mk<T>(T(0.5) * (P.x + Q.x), T(0.5) * (P.y - Q.y));
-    const cpx<T> Fb = mk<T>(T(0.5) * (P.y + Q.y), T(0.5) * (Q.x - P.x));
-    const bool own = line < RX;  // (f_0, f_1) of row `line`, else f_2 of rows q, q + RXh
-    const int ra = own ? line : line - RX, rb = own ? line : line - RX + RXh;
-    const int fa = own ? 0 : 2, fb = own ? 1 : 2;
-    if (ra < nr) MP::st(&a.scr[fa * sstride + (size_t)(r0 + ra) * M + k], Fa);
-    if (rb < nr) MP::st(&a.scr[fb * sstride + (size_t)(r0 + rb) * M + k], Fb);
   }
 }
 
@@ -1099,14 +1166,13 @@ struct PipeCfg {
   using C = K2Cfg<T, N>;
   static constexpr int M = N / 2;
   static constexpr int TYP = 4;
-  static constexpr int NTYP = round_warps(TYP * N / C::RYI);
+  static constexpr int NTYP = TYP * C::YNB;
   static constexpr int nYI = M / TYP, nX = N / C::RX, nYF = M / C::TY;
   static constexpr int per_slot = nYI + nX + nYF;
-  static constexpr int NT = cmax(cmax(NTYP, C::NTX), C::NTY);
+  static constexpr int NT = (cmax(cmax(NTYP, C::NTX), C::NTY) + 31) / 32 * 32;
   static constexpr bool ok = N % C::RX == 0 && M % TYP == 0 && TYP % C::MINW == 0;
   static constexpr size_t smem = sizeof(cpx<T>) *
-      cmax(cmax(4 * lf_rows<T, TYP>(N) * TYP, lf_rows<T, C::TY>(N) * C::TY), C::XELEMS) +
-      sizeof(cpx<T>) * tw_elems(N);
+      cmax(cmax(C::y_elems(TYP), C::y_elems(C::TY)), C::XELEMS + tw_elems(N));
 };
 
 // One slab pass over all N planes with the scratch as a ring of `ring` planes: every item
@@ -1118,11 +1184,11 @@ struct PipeCfg {
 // allocation spilled); the x-row body stays inline
 template <typename T, int N>
 __device__ __noinline__ void pipe_yinv(const SlabArgs<T>& b, int tile, int zs, cpx<T>* smem) {
-  yinv_tile<T, N, MemCG, PipeCfg<T, N>::TYP, PipeCfg<T, N>::NTYP>(b, tile, zs, smem);
+  yinv_tile<T, N, MemCG, PipeCfg<T, N>::TYP>(b, tile, zs, smem);
 }
 template <typename T, int N>
 __device__ __noinline__ void pipe_yfwd(const SlabArgs<T>& b, int tile, int zs, cpx<T>* smem) {
-  yfwd_tile<T, N, MemCG>(b, tile, zs, smem);
+  yfwd_tile<T, N, MemCG, K2Cfg<T, N>::TY>(b, tile, zs, smem);
 }
 
 template <typename T, int N>
@@ -1198,12 +1264,13 @@ namespace ns {
 template <typename T>
 struct K2Entry {
   int N = 0;
-  void (*pencil)(PencilArgs<T>) = nullptr;   // any number of inputs / outputs
-  void (*pencil1)(PencilArgs<T>) = nullptr;  // one input, one output
+  void (*pencil01)(PencilArgs<T>) = nullptr; // no input, one output (INIT)
+  void (*pencil10)(PencilArgs<T>) = nullptr; // one input, no output (NL, PROJECT)
+  void (*pencil1[MODE_ROG_2 + 1])(PencilArgs<T>) = {};  // one input, one output, by stage mode
   void (*pencil1e)(PencilArgs<T>) = nullptr; // same, also storing the tile's energy sums
   void (*pencil1re)(PencilArgs<T>) = nullptr; // the energy-sum variant of the ROG_2 stage
-  void (*pencil1r[2])(PencilArgs<T>) = {nullptr, nullptr};  // one in, one out: ROG_1, ROG_2
   void (*pencil2)(PencilArgs<T>) = nullptr;  // two inputs, two outputs
+  void (*pencil02)(PencilArgs<T>) = nullptr; // no input, two outputs (INIT of the exact scheme)
   void (*yinv)(SlabArgs<T>) = nullptr;
   void (*yfwd)(SlabArgs<T>) = nullptr;
   void (*xrow)(SlabArgs<T>) = nullptr;
@@ -1216,18 +1283,16 @@ struct K2Entry {
   int CLS = 0, NTCL[2] = {0, 0}, CLKC = 0, CLPL = 1;
   size_t smCL = 0;
   int TX = 0, NTP = 0, TY = 0, NTY = 0, TYI = 0, NTYI = 0, RX = 0, NTX = 0;
-  size_t smP1 = 0, smP4 = 0, smP5 = 0, smY = 0, smYI = 0, smX = 0;
-  // the autotuner's compiled alternatives (K2Cfg variant 15: every family's other width);
-  // has_alt false when the size has none
+  size_t smP = 0, smY = 0, smYI = 0, smX = 0;
+  // the autotuner's compiled alternatives (K2Cfg variant 15: every family's other width; the x
+  // rows have none); has_alt false when the size has none
   struct Alt {
     void (*pencil1r[2])(PencilArgs<T>) = {nullptr, nullptr};
     void (*yinv)(SlabArgs<T>) = nullptr;
     void (*yfwd)(SlabArgs<T>) = nullptr;
-    void (*xrow)(SlabArgs<T>) = nullptr;
-    int TX = 0, NTP = 0, TY = 0, NTY = 0, TYI = 0, NTYI = 0, RX = 0, NTX = 0;
-    size_t smP1 = 0, smY = 0, smYI = 0, smX = 0;
+    int TX = 0, NTP = 0, TY = 0, NTY = 0, TYI = 0, NTYI = 0;
+    size_t smP = 0, smY = 0, smYI = 0;
   } alt;
-  void (*pencil1r64[2])(PencilArgs<T>) = {nullptr, nullptr};  // variant 16 (64 registers)
   bool has_alt = false;
 };
 
@@ -1240,20 +1305,23 @@ K2Entry<T> make_k2_entry() {
   using C = K2Cfg<T, N>;
   K2Entry<T> e;
   e.N = N;
-  e.pencil = k2_pencil<T, N, -1, -1>;
-#ifndef NS_PENCIL_VARIANTS
-#define NS_PENCIL_VARIANTS 1
-#endif
-  // NS_PENCIL_VARIANTS=0 routes every pencil pass through the generic kernel (comparisons)
-  e.pencil1 = NS_PENCIL_VARIANTS ? k2_pencil<T, N, 1, 1> : e.pencil;
-  e.pencil1e = NS_PENCIL_VARIANTS ? k2_pencil<T, N, 1, 1, true> : e.pencil;
-#ifndef NS_PENCIL_MODE_VARIANTS
-#define NS_PENCIL_MODE_VARIANTS 1
-#endif
-  e.pencil1r[0] = NS_PENCIL_MODE_VARIANTS ? k2_pencil<T, N, 1, 1, false, MODE_ROG_1> : e.pencil1;
-  e.pencil1r[1] = NS_PENCIL_MODE_VARIANTS ? k2_pencil<T, N, 1, 1, false, MODE_ROG_2> : e.pencil1;
-  e.pencil1re = NS_PENCIL_VARIANTS && NS_PENCIL_MODE_VARIANTS ? k2_pencil<T, N, 1, 1, true, MODE_ROG_2> : e.pencil1e;
-  e.pencil2 = NS_PENCIL_VARIANTS ? k2_pencil<T, N, 2, 2> : e.pencil;
+  e.pencil01 = k2_pencil<T, N, 0, 1, false, MODE_INIT>;
+  e.pencil10 = k2_pencil<T, N, 1, 0>;
+  for (int m = MODE_RK2_1; m <= MODE_RK4_4; ++m) e.pencil1[m] = k2_pencil<T, N, 1, 1>;
+  if constexpr (C::F32 && N >= 64) {  // (elsewhere the run-time mode costs little)
+    e.pencil1[MODE_RK2_1] = k2_pencil<T, N, 1, 1, false, MODE_RK2_1>;
+    e.pencil1[MODE_RK2_2] = k2_pencil<T, N, 1, 1, false, MODE_RK2_2>;
+    e.pencil1[MODE_RK4_1] = k2_pencil<T, N, 1, 1, false, MODE_RK4_1>;
+    e.pencil1[MODE_RK4_2] = k2_pencil<T, N, 1, 1, false, MODE_RK4_2>;
+    e.pencil1[MODE_RK4_3] = k2_pencil<T, N, 1, 1, false, MODE_RK4_3>;
+    e.pencil1[MODE_RK4_4] = k2_pencil<T, N, 1, 1, false, MODE_RK4_4>;
+  }
+  e.pencil1[MODE_ROG_1] = k2_pencil<T, N, 1, 1, false, MODE_ROG_1>;
+  e.pencil1[MODE_ROG_2] = k2_pencil<T, N, 1, 1, false, MODE_ROG_2>;
+  e.pencil1e = k2_pencil<T, N, 1, 1, true>;
+  e.pencil1re = k2_pencil<T, N, 1, 1, true, MODE_ROG_2>;
+  e.pencil2 = k2_pencil<T, N, 2, 2>;
+  e.pencil02 = k2_pencil<T, N, 0, 2>;
   e.yinv = k2_yinv<T, N>;
   e.yfwd = k2_yfwd<T, N>;
   e.xrow = k2_xrow<T, N>;
@@ -1274,11 +1342,9 @@ K2Entry<T> make_k2_entry() {
   }
   e.TX = C::TX; e.NTP = C::NTP; e.TY = C::TY; e.NTY = C::NTY; e.RX = C::RX; e.NTX = C::NTX;
   e.TYI = C::TYI; e.NTYI = C::NTYI;
-  e.smYI = (4 * (size_t)lf_rows<T, C::TYI>(N) * C::TYI + tw_elems(N)) * sizeof(cpx<T>);
-  e.smP4 = (3 * (size_t)lf_rows<T, C::TX>(N) * C::TX + tw_elems(N)) * sizeof(cpx<T>);  // 3 tiles + twiddles
-  e.smP1 = NS_PENCIL_STAGE_STATE ? (6 * (size_t)lf_rows<T, C::TX>(N) * C::TX + tw_elems(N)) * sizeof(cpx<T>) : e.smP4;
-  e.smP5 = (4 * (size_t)lf_rows<T, C::TX>(N) * C::TX + tw_elems(N)) * sizeof(cpx<T>);  // 4 tiles + twiddles
-  e.smY = ((size_t)lf_rows<T, C::TY>(N) * C::TY + tw_elems(N)) * sizeof(cpx<T>);
+  e.smYI = (size_t)C::y_elems(C::TYI) * sizeof(cpx<T>);
+  e.smP = (size_t)C::p_elems * sizeof(cpx<T>);
+  e.smY = (size_t)C::y_elems(C::TY) * sizeof(cpx<T>);
   e.smX = ((size_t)C::XELEMS + tw_elems(N)) * sizeof(cpx<T>);
   if constexpr (k2_has_alt<T, N>()) {
     using A = K2Cfg<T, N, 15>;
@@ -1287,15 +1353,11 @@ K2Entry<T> make_k2_entry() {
     e.alt.pencil1r[1] = k2_pencil<T, N, 1, 1, false, MODE_ROG_2, 15>;
     e.alt.yinv = k2_yinv<T, N, 15>;
     e.alt.yfwd = k2_yfwd<T, N, 15>;
-    e.alt.xrow = k2_xrow<T, N, 15>;
     e.alt.TX = A::TX; e.alt.NTP = A::NTP; e.alt.TY = A::TY; e.alt.NTY = A::NTY;
-    e.alt.TYI = A::TYI; e.alt.NTYI = A::NTYI; e.alt.RX = A::RX; e.alt.NTX = A::NTX;
-    e.alt.smYI = (4 * (size_t)lf_rows<T, A::TYI>(N) * A::TYI + tw_elems(N)) * sizeof(cpx<T>);
-    e.alt.smP1 = (3 * (size_t)lf_rows<T, A::TX>(N) * A::TX + tw_elems(N)) * sizeof(cpx<T>);
-    e.alt.smY = ((size_t)lf_rows<T, A::TY>(N) * A::TY + tw_elems(N)) * sizeof(cpx<T>);
-    e.alt.smX = ((size_t)A::XELEMS + tw_elems(N)) * sizeof(cpx<T>);
-    e.pencil1r64[0] = k2_pencil<T, N, 1, 1, false, MODE_ROG_1, 16>;
-    e.pencil1r64[1] = k2_pencil<T, N, 1, 1, false, MODE_ROG_2, 16>;
+    e.alt.TYI = A::TYI; e.alt.NTYI = A::NTYI;
+    e.alt.smYI = (size_t)A::y_elems(A::TYI) * sizeof(cpx<T>);
+    e.alt.smP = (size_t)A::p_elems * sizeof(cpx<T>);
+    e.alt.smY = (size_t)A::y_elems(A::TY) * sizeof(cpx<T>);
   }
   return e;
 }
