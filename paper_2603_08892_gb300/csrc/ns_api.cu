@@ -34,7 +34,9 @@ bool k2_lookup_f32a(int N, K2Entry<float>* e);
 bool k2_lookup_f32b(int N, K2Entry<float>* e);
 bool k2_lookup_f32c(int N, K2Entry<float>* e);
 bool k2_lookup_f32d(int N, K2Entry<float>* e);
+bool k2_lookup_f32e(int N, K2Entry<float>* e);
 bool k2_lookup_f64a(int N, K2Entry<double>* e);
+bool k2_lookup_f64e(int N, K2Entry<double>* e);
 bool k2_lookup_f64b(int N, K2Entry<double>* e);
 bool k2_lookup_f64c(int N, K2Entry<double>* e);
 }  // namespace ns
@@ -178,11 +180,12 @@ EncodeTiledFn encode_tiled() {
 
 bool k2_find(int N, K2Entry<float>* e) {
   if (std::getenv("NS_GENERIC_KERNELS")) return false;
-  return k2_lookup_f32a(N, e) || k2_lookup_f32b(N, e) || k2_lookup_f32c(N, e) || k2_lookup_f32d(N, e);
+  return k2_lookup_f32a(N, e) || k2_lookup_f32b(N, e) || k2_lookup_f32c(N, e) || k2_lookup_f32d(N, e) ||
+         k2_lookup_f32e(N, e);
 }
 bool k2_find(int N, K2Entry<double>* e) {
   if (std::getenv("NS_GENERIC_KERNELS")) return false;
-  return k2_lookup_f64a(N, e) || k2_lookup_f64b(N, e) || k2_lookup_f64c(N, e);
+  return k2_lookup_f64a(N, e) || k2_lookup_f64b(N, e) || k2_lookup_f64c(N, e) || k2_lookup_f64e(N, e);
 }
 
 struct SolverBase {
@@ -293,6 +296,11 @@ struct Solver : SolverBase {
   // skips its INIT pass.  -1 whenever anything else wrote the state, the mixed fields or the
   // forcing record.
   int64_t carry_step = -1;
+  // the mixed fields, the state or the forcing record change other than by a step
+  void touched() {
+    carry_step = -1;
+    cut_known = false;
+  }
   // adaptive time step (ns_step_cfl): dt = min(dt_max, cfl dx / sum_i max|u_i|) per step
   double cfl = 0.0, cfl_dtmax = 0.0;
   unsigned long long* d_umax = nullptr;
@@ -422,12 +430,14 @@ struct Solver : SolverBase {
         CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
       };
       allow(k2.pencil01, k2.smP);
-      allow(k2.pencil10, k2.smP);
+      allow(k2.pencil10[0], k2.smP);
+      allow(k2.pencil10[1], k2.smP);
       for (auto* f : k2.pencil1)
         if (f) allow(f, k2.smP);
-      allow(k2.pencil1e, k2.smP);
-      allow(k2.pencil1re, k2.smP);
-      allow(k2.pencil2, k2.smP);
+      for (auto* f : k2.pencil1e)
+        if (f) allow(f, k2.smP);
+      allow(k2.pencil2[0], k2.smP);
+      allow(k2.pencil2[1], k2.smP);
       allow(k2.pencil02, k2.smP);
       allow(k2.yinv, k2.smYI);
       allow(k2.yfwd, k2.smY);
@@ -464,6 +474,9 @@ struct Solver : SolverBase {
     red_blocks = 2 * nsm;
     CUDA_TRY(cudaMalloc(&red, (size_t)red_blocks * 1024 * sizeof(double)));
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
+    CUDA_TRY(cudaMalloc(&d_cut, 3 * sizeof(int)));
+    const int one[3] = {0, 0, 1};
+    CUDA_TRY(cudaMemcpyAsync(d_cut, one, sizeof(one), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMalloc(&d_umax, 3 * sizeof(unsigned long long)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), st));
     CUDA_TRY(cudaMemsetAsync(state, 0, 3 * F1 * cs, st));
@@ -474,7 +487,7 @@ struct Solver : SolverBase {
 
   ~Solver() override {
     cudaFree(state); cudaFree(acc); cudaFree(mixed[0]); cudaFree(mixed[1]);
-    cudaFree(nlbuf); cudaFree(nltmp); cudaFree(d_umax); cudaFree(d_pipe);
+    cudaFree(nlbuf); cudaFree(nltmp); cudaFree(d_umax); cudaFree(d_pipe); cudaFree(d_cut);
     cudaFree(d_epart);
     if (h_err) cudaFreeHost(h_err);
     if (h_series) cudaFreeHost(h_series);
@@ -496,10 +509,13 @@ struct Solver : SolverBase {
     for (auto e : prof.pool) cudaEventDestroy(e);
   }
 
-  void* state_ptr() override { return state; }
+  void* state_ptr() override {
+    state_shared = true;
+    return state;
+  }
 
   void buffers(double dt, NsCtxBuffers* b) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     if (dt > 0) set_dt(dt);
     b->N = N; b->precision = c->p.precision; b->scheme = c->p.scheme; b->truncation = c->p.truncation;
     b->K2max = c->K2max; b->Kimax = c->Kimax; b->G = Gmax; b->nu = c->p.nu; b->kmax = c->p.kmax;
@@ -535,6 +551,28 @@ struct Solver : SolverBase {
   }
 
   // ---- passes -----------------------------------------------------------------------
+  // Truncated states.  d_cut[0]: the state vanishes outside the kept columns (column_kept);
+  // d_cut[1]: the same of the state from which the carried mixed fields were formed; d_cut[2] = 1.
+  // Steps keep the property, so the state is looked at when something else may have written it:
+  // before the first step after that, and, once its device address was handed out
+  // (ns_device_state), before the first step of every call.
+  int* d_cut = nullptr;
+  bool cut_known = false, state_shared = false;
+  int box() const { return fkind != NS_FORCE_NONE ? fK : -1; }
+  int kx_end() const {  // first kx none of whose columns is kept
+    int k = 0;
+    while (k < M && column_kept(c->p.truncation, c->K2max, c->Kimax, box(), k, 0)) ++k;
+    return k;
+  }
+  void cut_check() {
+    if (cut_known && !state_shared) return;
+    k_cut_begin<<<1, 1, 0, st>>>(d_cut);
+    k_cut_check<T><<<dim3(N, N < 256 ? 2 : 8), 256, 0, st>>>(state, N, c->p.truncation, c->K2max, c->Kimax, box(), d_cut);
+    LAUNCH_CHECK();
+    cut_known = true;
+  }
+  const int* cut_flag(int i) const { return use2 && !clus ? d_cut + i : nullptr; }
+
   // layout of the mixed fields and of Ft (mixed_index): interleaved for the compile-time kernels,
   // except when the cluster slab pass, whose TMA copies take one field at a time, reads them
   int pairs() const { return use2 && !clus; }
@@ -546,6 +584,7 @@ struct Solver : SolverBase {
     a.pairs = pairs();
     if (use2) {  // Ft columns that no pencil pass uses are left unwritten
       a.skip = 1;
+      a.kxn = kx_end();
       a.trunc = c->p.truncation; a.K2max = c->K2max; a.Kimax = c->Kimax;
       a.fK = fkind != NS_FORCE_NONE ? fK : -1;
     }
@@ -640,17 +679,19 @@ struct Solver : SolverBase {
     e = prof_begin(NS_PROF_YFWD, s);
     if (use2)
       if (vsel & 8)
-        k2.alt.yfwd<<<dim3(M / k2.alt.TY, a.G), k2.alt.NTY, k2.alt.smY, s>>>(a);
+        k2.alt.yfwd<<<dim3((a.kxn + k2.alt.TY - 1) / k2.alt.TY, a.G), k2.alt.NTY, k2.alt.smY, s>>>(a);
       else
-        k2.yfwd<<<dim3(M / k2.TY, a.G), k2.NTY, k2.smY, s>>>(a);
+        k2.yfwd<<<dim3((a.kxn + k2.TY - 1) / k2.TY, a.G), k2.NTY, k2.smY, s>>>(a);
     else
       k_yfwd<T><<<dim3(M / TY, a.G), bdYf, smYf, s>>>(a);
     prof_end(e, s);
   }
 
   // slab pass over every plane group: mixed (5 fields) -> Ft (3 fields)
-  void slab(const cpx<T>* mix, cpx<T>* out, bool umax = false) {
+  // (cut: flag under which `mix` was written, or null)
+  void slab(const cpx<T>* mix, cpx<T>* out, bool umax = false, const int* cut = nullptr) {
     SlabArgs<T> a = slab_args();
+    a.cut = cut;
     a.mixed = mix;
     a.Ft = out;
     a.xmode = XMODE_NONLINEAR;
@@ -724,6 +765,7 @@ struct Solver : SolverBase {
     a.trunc = c->p.truncation; a.K2max = c->K2max; a.Kimax = c->Kimax;
     a.err = d_err;
     a.pairs = pairs();
+    a.cutK = box();
     if (fkind != NS_FORCE_NONE) {
       a.shell = shell;
       a.fK = fK;
@@ -739,11 +781,11 @@ struct Solver : SolverBase {
     if (use2 && rog && (vsel & 1))  // the autotuner's alternative pencil width
       k2.alt.pencil1r[a.mode == MODE_ROG_1 ? 0 : 1]<<<(M / k2.alt.TX) * R, k2.alt.NTP, k2.alt.smP, st>>>(a);
     else if (use2)
-      (a.nF == 1 && a.nOut == 1   ? (a.epart ? (a.mode == MODE_ROG_2 ? k2.pencil1re : k2.pencil1e) : k2.pencil1[a.mode])
-       : a.nF == 2 && a.nOut == 2 ? k2.pencil2
+      (a.nF == 1 && a.nOut == 1   ? (a.epart ? k2.pencil1e[a.mode] : k2.pencil1[a.mode])
+       : a.nF == 2 && a.nOut == 2 ? k2.pencil2[a.mode == MODE_RK2_2]
        : a.nF == 0 && a.nOut == 2 ? k2.pencil02
        : a.nF == 0                ? k2.pencil01
-                                  : k2.pencil10)<<<(M / k2.TX) * R, k2.NTP, k2.smP, st>>>(a);
+                                  : k2.pencil10[a.mode == MODE_PROJECT])<<<(M / k2.TX) * R, k2.NTP, k2.smP, st>>>(a);
     else
       k_pencil<T><<<(M / TX) * R, bdP, smP, st>>>(a);
     prof_end(e);
@@ -765,7 +807,7 @@ struct Solver : SolverBase {
   // block [lo, hi) of the z (or kz) axis (axis 0) or the ky axis (axis 1) of buffer `which`
   // between the device and host FP64 (re, im): axis 0 [F][hi-lo][N][M], axis 1 [F][N][hi-lo][M]
   void rank_copy(int which, int axis, int lo, int hi, bool to_dev, double* host) override {
-    carry_step = -1;
+    touched();
     const int F = rank_fields(which), n = hi - lo;
     const size_t cs = sizeof(cpx<T>);
     if (!rank_stg) CUDA_TRY(cudaMalloc(&rank_stg, 5 * F1 * cs));
@@ -785,7 +827,7 @@ struct Solver : SolverBase {
   // pencil pass on the ky rows [lo, hi): NS_RANK_INIT: state -> mixed (shifted by delta);
   // NS_RANK_NL: Ft -> the shifted, de-shifted, truncated, projected nonlinear term (NL buffer)
   void rank_pencil(int kind, const double* delta, int lo, int hi) override {
-    carry_step = -1;
+    touched();
     std::vector<double> sh(delta, delta + 3);
     upload_shifts(sh);
     PencilArgs<T> p = pencil_args(kind == NS_RANK_INIT ? MODE_INIT : MODE_NL);
@@ -804,7 +846,7 @@ struct Solver : SolverBase {
   }
   // slab pass on the planes [lo, hi): mixed -> Ft (the three slab kernels, plane groups of G)
   void rank_slab(int lo, int hi) override {
-    carry_step = -1;
+    touched();
     SlabArgs<T> a = slab_args();
     a.mixed = mixed[0];
     a.Ft = Ft[0];
@@ -990,7 +1032,7 @@ struct Solver : SolverBase {
 
   void set_forcing(int kind, double kfmin, double kfmax, double eps, double tcorr,
                    uint64_t seed) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     tape.valid = false;  // a recorded adjoint run used the previous forcing
     fkind = kind;
     if (kind == NS_FORCE_NONE) return;
@@ -1104,7 +1146,7 @@ struct Solver : SolverBase {
     }
   }
   void autotune() {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     tuned = true;
     if (const char* e = std::getenv("NS_PIPE_SPIN")) pipe_spin = std::max(1ll, std::atoll(e));
     if (const char* e = std::getenv("NS_PIPE_TEST_STALL")) pipe_stall = std::atoi(e) ? 1 : 0;
@@ -1249,7 +1291,7 @@ struct Solver : SolverBase {
   }
 
   // ---- schemes ------------------------------------------------------------------------
-  void invalidate_carry() override { carry_step = -1; }
+  void invalidate_carry() override { touched(); }
 
   void step_cfl(double cfl_, double dt_max, int nsteps) override {
     cfl = cfl_;
@@ -1265,13 +1307,14 @@ struct Solver : SolverBase {
 
   void step(double dt, int nsteps) override {
     if (!tuned) autotune();
+    if (nsteps > 0) cut_check();
     set_dt(dt);
     const int sch = c->p.scheme;
     const double dx = 2.0 * M_PI / N;
     const int CH = 256;  // steps per chunk of shift tables
     for (int s0 = 0; s0 < nsteps; s0 += CH) {
       const int ns = (s0 + CH <= nsteps) ? CH : nsteps - s0;
-      const bool last_chunk = s0 + ns == nsteps;
+      chunk0 = s0 == 0;
       if (fkind != NS_FORCE_NONE) prepare_forcing(c->t, c->t + ns * dt);
       if (sch == NS_RK2_PS_RANDOM || sch == NS_RK2_PS_APPROX) {
         // shift vectors: [2n] alpha_n, [2n+1] beta_n, and alpha of the step after the chunk
@@ -1304,7 +1347,6 @@ struct Solver : SolverBase {
       } else {
         run_rk4(dt, ns);
       }
-      (void)last_chunk;
     }
     // stream-ordered: device-side checks are reported by the next synchronising call
   }
@@ -1312,6 +1354,7 @@ struct Solver : SolverBase {
   void init_pass(int nOut, const cpx<T>* o0, const cpx<T>* o1) {
     PencilArgs<T> a = pencil_args(MODE_INIT);
     a.src = state;
+    a.cut = cut_flag(0);
     a.nOut = nOut;
     a.osh[0] = o0; a.out[0] = mixed[0];
     a.osh[1] = o1; a.out[1] = mixed[1];
@@ -1338,22 +1381,31 @@ struct Solver : SolverBase {
     return d;
   }
 
+  // flag of the mixed fields that a chunk's first slab pass reads: carried from an earlier call of a
+  // shared state, the one of the state they were formed from; formed now, the state's
+  const int* first_cut() const {
+    return cut_flag(carry_step == c->step && chunk0 && state_shared ? 1 : 0);
+  }
+  bool chunk0 = false;  // the first chunk of a call
   void run_rogallo(double dt0, int ns, bool approx) {
     const T w = (T)(1.0 / ((double)N * N * N));
     auto alpha = [&](int n) -> const cpx<T>* { return approx ? nullptr : shift_tab(2 * n); };
     auto beta = [&](int n) -> const cpx<T>* { return shift_tab(2 * n + 1); };
+    const int* cin = first_cut();
     if (carry_step != c->step) init_pass(1, alpha(0), nullptr);
     for (int n = 0; n < ns; ++n) {
       const double t = c->t;
-      slab(mixed[0], Ft[0], cfl > 0.0);
+      slab(mixed[0], Ft[0], cfl > 0.0, n == 0 ? cin : cut_flag(0));
       const double dt = step_dt(dt0);
       PencilArgs<T> a = pencil_args(MODE_ROG_1);
       force_coef(t, a);
       a.nF = 1; a.F[0] = Ft[0]; a.dsh[0] = alpha(n); a.wF[0] = w;
       a.nOut = 1; a.osh[0] = beta(n); a.out[0] = mixed[0];
+      a.cut = cut_flag(0);
       pencil(a);
-      slab(mixed[0], Ft[0]);
+      slab(mixed[0], Ft[0], false, cut_flag(0));
       PencilArgs<T> b = pencil_args(MODE_ROG_2);
+      b.cut = cut_flag(0);
       force_coef(t + dt, b);
       b.nF = 1; b.F[0] = Ft[0]; b.dsh[0] = beta(n); b.wF[0] = w;
       b.nOut = 1;  // the last step of the chunk prepares the step after it
@@ -1369,15 +1421,18 @@ struct Solver : SolverBase {
   void run_rk2(double dt0, int ns, bool exact) {
     const T w = (T)(1.0 / ((double)N * N * N));
     const cpx<T>* iso = exact ? shift_tab(0) : nullptr;
+    const int* cin = first_cut();
     if (carry_step != c->step) init_pass(exact ? 2 : 1, nullptr, iso);
     for (int n = 0; n < ns; ++n) {
       const double t = c->t;
       double dt = dt0;
       for (int stg = 0; stg < 2; ++stg) {
-        slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0);
+        const int* cut = n == 0 && stg == 0 ? cin : cut_flag(0);
+        slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0, cut);
         if (stg == 0) dt = step_dt(dt0);
-        if (exact) slab(mixed[1], Ft[1]);
+        if (exact) slab(mixed[1], Ft[1], false, cut);
         PencilArgs<T> a = pencil_args(stg == 0 ? MODE_RK2_1 : MODE_RK2_2);
+        a.cut = cut_flag(0);
         force_coef(stg == 0 ? t : t + 0.5 * dt, a);
         a.nF = exact ? 2 : 1;
         a.F[0] = Ft[0]; a.dsh[0] = nullptr; a.wF[0] = exact ? (T)0.5 * w : w;
@@ -1398,6 +1453,7 @@ struct Solver : SolverBase {
 
   void run_rk4(double dt0, int ns) {
     const T w = (T)(1.0 / ((double)N * N * N));
+    const int* cin = first_cut();
     if (carry_step != c->step) init_pass(1, nullptr, nullptr);
     const int modes[4] = {MODE_RK4_1, MODE_RK4_2, MODE_RK4_3, MODE_RK4_4};
     const double ts[4] = {0.0, 0.5, 0.5, 1.0};
@@ -1405,9 +1461,10 @@ struct Solver : SolverBase {
       const double t = c->t;
       double dt = dt0;
       for (int stg = 0; stg < 4; ++stg) {
-        slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0);
+        slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0, n == 0 && stg == 0 ? cin : cut_flag(0));
         if (stg == 0) dt = step_dt(dt0);
         PencilArgs<T> a = pencil_args(modes[stg]);
+        a.cut = cut_flag(0);
         force_coef(t + ts[stg] * dt, a);
         a.nF = 1; a.F[0] = Ft[0]; a.wF[0] = w;
         a.nOut = 1;  // the last pass prepares the next step
@@ -1517,7 +1574,7 @@ struct Solver : SolverBase {
   }
 
   void set_velocity(const double* u) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     T* rin = reinterpret_cast<T*>(mixed[0]);  // 5 N^3 reals >= 3 N^3
     to_device(u, rin, 3 * (size_t)N * N * N);
     r2c_project(rin, state, 1.0 / ((double)N * N * N));
@@ -1528,7 +1585,7 @@ struct Solver : SolverBase {
 
   // spectral [3][N][N][M] -> physical host [3][N][N][N] (inverse z, y, x transforms)
   void to_physical(const cpx<T>* src, double* u) {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     T* rout = reinterpret_cast<T*>(Ft[0]);  // 3 N^3 reals
     c2r(src, rout);
     to_host(rout, u, 3 * (size_t)N * N * N);
@@ -1553,7 +1610,7 @@ struct Solver : SolverBase {
     sync_check();
   }
   void set_raw_state(const unsigned char* in, size_t n) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     if (n != 3 * F1 * sizeof(cpx<T>)) throw NsError{NS_ERR_IO, "checkpoint state size mismatch"};
     CUDA_TRY(cudaMemcpyAsync(state, in, n, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -1564,12 +1621,12 @@ struct Solver : SolverBase {
     *seed = fseed;
   }
   void set_state(const double* s) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     upload(s, state);
   }
 
   void nonlinear(const double* in, const double* delta, double* out) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     const cpx<T>* src = state;
     if (in) {
       upload(in, acc);
@@ -1607,14 +1664,15 @@ struct Solver : SolverBase {
     LAUNCH_CHECK();
   }
 
-  // Nt_D(S) -> out  (D = shift table or null)
-  void nl_eval(const cpx<T>* S, const cpx<T>* tab, cpx<T>* out) {
+  // Nt_D(S) -> out  (D = shift table or null; cut: flag of S)
+  void nl_eval(const cpx<T>* S, const cpx<T>* tab, cpx<T>* out, const int* cut) {
     PencilArgs<T> p = pencil_args(MODE_INIT);
+    p.cut = cut;
     p.shell = nullptr;
     p.src = S;
     p.nOut = 1; p.osh[0] = tab; p.out[0] = mixed[0];
     pencil(p);
-    slab(mixed[0], Ft[0]);
+    slab(mixed[0], Ft[0], false, cut);
     PencilArgs<T> q = pencil_args(MODE_NL);
     q.shell = nullptr;
     q.acc = out;
@@ -1748,16 +1806,16 @@ struct Solver : SolverBase {
     cpx<T>* N0 = vec(0);
     cpx<T>* N1 = vec(1);
     cpx<T>* S1 = vec(2);
-    nl_eval(S0, shift_tab(2 * n), N0);
+    nl_eval(S0, shift_tab(2 * n), N0, cut_flag(2));
     add_forcing(S0, times[n], N0);
     ew(EW_ROG_S1, S0, N0, nullptr, S1);
-    nl_eval(S1, shift_tab(2 * n + 1), N1);
+    nl_eval(S1, shift_tab(2 * n + 1), N1, cut_flag(2));
     add_forcing(S1, times[n] + dt, N1);
     ew(EW_ROG_SN, S0, N0, N1, Sout);
   }
   // forward sweep from `state` with the state kept every ckpt steps; leaves state = S_T
   void adj_forward(int nsteps, double dt, int ckpt) {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     adj_alloc(nsteps, ckpt);
     const std::vector<double> times = adj_tables(nsteps, dt);
     const size_t vb = 3 * F1 * sizeof(cpx<T>);
@@ -1806,7 +1864,7 @@ struct Solver : SolverBase {
         const cpx<T>* S0 = seg[n - seg0];
         const cpx<T>* ta = shift_tab(2 * n);
         const cpx<T>* tb = shift_tab(2 * n + 1);
-        nl_eval(S0, ta, N0);
+        nl_eval(S0, ta, N0, cut_flag(2));
         add_forcing(S0, times[n], N0);
         ew(EW_ROG_S1, S0, N0, nullptr, S1);
         ew(EW_RHO, lam, nullptr, nullptr, rho);
@@ -1866,7 +1924,7 @@ struct Solver : SolverBase {
 
   // device-buffer forms (the autograd path): u0, uT [3][N][N][N] reals of T on the device
   void tape_forward(const void* u0, int nsteps, double dt, int ckpt, void* uT) override {
-    carry_step = -1;
+    touched();
     r2c_project(static_cast<const T*>(u0), state, 1.0 / ((double)N * N * N));
     adj_forward(nsteps, dt, ckpt);
     c2r(state, static_cast<T*>(uT));
@@ -1875,7 +1933,7 @@ struct Solver : SolverBase {
   // gT: the cotangent of u(T) (device reals of T), or null for the built-in loss `loss`
   void tape_backward(const void* gT, int loss, void* grad) override {
     if (!tape.valid) throw NsError{NS_ERR_STATE, "no adjoint tape: call ns_tape_forward first"};
-    carry_step = -1;
+    touched();
     cpx<T>* lam = vec(3);
     if (gT)
       r2c_project(static_cast<const T*>(gT), lam, 1.0);
@@ -1920,17 +1978,18 @@ struct Solver : SolverBase {
   // Nonlinear energy flux and cumulative dissipation on shell bins (Sec. 3.4)
   cpx<T>* nlbuf = nullptr;
   void energy_flux(const double* delta, int nshift, double* flux, double* cumd, int nbins) override {
-    carry_step = -1;  // the mixed fields / state / forcing record change here
+    touched();
     if (flux) {
       if (!nlbuf) CUDA_TRY(cudaMalloc(&nlbuf, 3 * F1 * sizeof(cpx<T>)));
+      cut_check();
       if (nshift == 0) {
-        nl_eval(state, nullptr, nlbuf);
+        nl_eval(state, nullptr, nlbuf, cut_flag(0));
       } else {
         if (!nltmp && nshift > 1) CUDA_TRY(cudaMalloc(&nltmp, 3 * F1 * sizeof(cpx<T>)));
         for (int sidx = 0; sidx < nshift; ++sidx) {
           std::vector<double> sh(delta + 3 * sidx, delta + 3 * sidx + 3);
           upload_shifts(sh);
-          nl_eval(state, shift_tab(0), sidx == 0 ? nlbuf : nltmp);
+          nl_eval(state, shift_tab(0), sidx == 0 ? nlbuf : nltmp, cut_flag(0));
           if (sidx > 0) ew(EW_ADD, nlbuf, nltmp, nullptr, nlbuf);
         }
         if (nshift > 1) ew(EW_SCALE, nlbuf, nullptr, nullptr, nlbuf, 1.0 / nshift);

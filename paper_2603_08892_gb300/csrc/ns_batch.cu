@@ -171,6 +171,7 @@ int ns_batch_destroy(ns_batch* b) {
   cudaFree(b->d_flags);
   cudaFree(b->d_tab);
   cudaFree(b->d_cls);
+  cudaFree(b->d_cut);
   if (b->own_stream) cudaStreamDestroy(b->st);  // members were given the stream, not its ownership
   delete b;
   return NS_OK;

@@ -275,14 +275,14 @@ __global__ void __launch_bounds__(128) k_bgrid_tab(const BatchMem<T>* __restrict
                                                    int step, int nsteps) {
   batch_tab<T, N>(mems[__ldg(&cls[blockIdx.y])], step, nsteps);
 }
-template <typename T, int N>
-__global__ void __launch_bounds__(K2Cfg<T, N>::NTP, K2Cfg<T, N>::MINB_P) k_bgrid_pencil(const BatchMem<T>* __restrict__ mems,
-                                                                  const int* __restrict__ cls, int pass, int step,
-                                                                  int nsteps) {
+// NF, NO, MC: the pass's inputs, outputs and stage mode
+template <typename T, int N, int NF, int NO, int MC>
+__global__ void __launch_bounds__(K2Cfg<T, N>::NTP, K2Cfg<T, N>::MINB_P) k_bgrid_pencil(
+    const BatchMem<T>* __restrict__ mems, const int* __restrict__ cls, int pass, int step, int nsteps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const BatchMem<T>& bm = mems[__ldg(&cls[blockIdx.y])];
-  pencil_tile<T, N, MemNC>(batch_pencil_args(bm, pass, step, nsteps), (int)blockIdx.x,
-                           reinterpret_cast<cpx<T>*>(smem_raw));
+  pencil_tile<T, N, MemNC, NF, NO, false, MC>(batch_pencil_args(bm, pass, step, nsteps), (int)blockIdx.x,
+                                              reinterpret_cast<cpx<T>*>(smem_raw));
 }
 template <typename T, int N>
 __global__ void __launch_bounds__(K2Cfg<T, N>::NTYI, K2Cfg<T, N>::MINB_YI) k_bgrid_yinv(const BatchMem<T>* __restrict__ mems,
@@ -357,7 +357,10 @@ cudaError_t launch_class(const BatchMem<T>* dm, const int* cls, int nc, int nste
   const size_t smX = ((size_t)C::XELEMS + tw) * cz;
   static bool attr = false;  // (per template instance: the opt-in sizes set before the first launch)
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_bgrid_pencil<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smP);
+    cudaError_t e = cudaSuccess;
+    for (auto* f : {k_bgrid_pencil<T, N, 0, 1, MODE_INIT>, k_bgrid_pencil<T, N, 1, 1, MODE_ROG_1>,
+                    k_bgrid_pencil<T, N, 1, 1, MODE_ROG_2>, k_bgrid_pencil<T, N, 1, 0, MODE_ROG_2>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smP);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_bgrid_yinv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smYI);
     if (e == cudaSuccess)
@@ -370,14 +373,17 @@ cudaError_t launch_class(const BatchMem<T>* dm, const int* cls, int nc, int nste
   const int pen = (M / C::TX) * N, yi = (M / C::TYI) * N, yf = (M / C::TY) * N;
   const int xr = (N * N + C::RX - 1) / C::RX;
   k_bgrid_tab<T, N><<<dim3(1, nc), 128, 0, cs>>>(dm, cls, 0, nsteps);
-  k_bgrid_pencil<T, N><<<dim3(pen, nc), C::NTP, smP, cs>>>(dm, cls, -1, 0, nsteps);
+  k_bgrid_pencil<T, N, 0, 1, MODE_INIT><<<dim3(pen, nc), C::NTP, smP, cs>>>(dm, cls, -1, 0, nsteps);
   for (int s = 0; s < nsteps; ++s) {
     k_bgrid_tab<T, N><<<dim3(1, nc), 128, 0, cs>>>(dm, cls, s, nsteps);
     for (int h = 0; h < 2; ++h) {  // the two stages: slab pass, then the pencil pass P1 / P2
       k_bgrid_yinv<T, N><<<dim3(yi, nc), C::NTYI, smYI, cs>>>(dm, cls);
       k_bgrid_xrow<T, N><<<dim3(xr, nc), C::NTX, smX, cs>>>(dm, cls);
       k_bgrid_yfwd<T, N><<<dim3(yf, nc), C::NTY, smY, cs>>>(dm, cls);
-      k_bgrid_pencil<T, N><<<dim3(pen, nc), C::NTP, smP, cs>>>(dm, cls, h == 0 ? P_P1 : P_P2, s, nsteps);
+      const auto pk = h == 0           ? k_bgrid_pencil<T, N, 1, 1, MODE_ROG_1>
+                      : s + 1 < nsteps ? k_bgrid_pencil<T, N, 1, 1, MODE_ROG_2>
+                                       : k_bgrid_pencil<T, N, 1, 0, MODE_ROG_2>;  // (no next step)
+      pk<<<dim3(pen, nc), C::NTP, smP, cs>>>(dm, cls, h == 0 ? P_P1 : P_P2, s, nsteps);
     }
   }
   return cudaGetLastError();
@@ -396,6 +402,15 @@ cudaError_t launch_class_any(int sz, const BatchMem<T>* dm, const int* cls, int 
 }
 
 #endif  // NS_BATCH_GRID_DEFS
+
+// cut flags of the members (set to non-zero before): 0 where the state does not vanish outside
+// the truncation
+template <typename T>
+__global__ void __launch_bounds__(256) k_bcut_check(const BatchMem<T>* __restrict__ mems, int* flags) {
+  const PencilArgs<T>& a = mems[blockIdx.y].pa;
+  if ((int)blockIdx.x < a.N && !cut_clean(a.state, a.N, a.trunc, a.K2max, a.Kimax, -1, blockIdx.x, 0, 1))
+    flags[blockIdx.y] = 0;
+}
 
 inline uint64_t smix(uint64_t s, uint64_t n) {
   uint64_t z = s + (n + 1) * 0x9E3779B97F4A7C15ull;
@@ -435,6 +450,7 @@ struct ns_batch {
   bool tuned = false;
   // grid schedule (gran 0): member indices grouped by size class
   int* d_cls = nullptr;
+  int* d_cut = nullptr;  // the members' cut flags (PencilArgs::cut)
 };
 
 namespace nsb {
@@ -453,6 +469,7 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
     if (cudaMalloc(&b->d_shifts, (size_t)n * per * sizeof(double)) != cudaSuccess) return NS_ERR_OOM;
     b->shifts_cap = (size_t)n * per;
   }
+  if (!b->d_cut && cudaMalloc(&b->d_cut, kMaxMembers * sizeof(int)) != cudaSuccess) return NS_ERR_OOM;
   for (int m = 0; m < n; ++m) {
     NsCtxBuffers cb;
     int rc = ns_ctx_buffers(b->mem[m], dt[m], &cb);
@@ -468,9 +485,12 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
     a.state = (cpx<T>*)cb.state; a.acc = nullptr; a.trunc = cb.truncation; a.K2max = cb.K2max;
     a.Kimax = cb.Kimax; a.err = (int*)cb.err; a.wF[0] = (T)(1.0 / ((double)N * N * N));
     a.F[0] = (const cpx<T>*)cb.Ft; a.out[0] = (cpx<T>*)cb.mixed; a.pairs = 1;
+    a.cut = b->d_cut + m; a.cutK = -1;
     SlabArgs<T>& s = bm.sa;
     s.N = N; s.M = M; s.z0 = 0; s.G = N; s.tw = (const cpx<T>*)cb.tw; s.mixed = (const cpx<T>*)cb.mixed;
-    s.scr = (cpx<T>*)cb.scr; s.Ft = (cpx<T>*)cb.Ft; s.xmode = XMODE_NONLINEAR; s.pairs = 1; s.err = (int*)cb.err;
+    s.scr = (cpx<T>*)cb.scr; s.Ft = (cpx<T>*)cb.Ft; s.xmode = XMODE_NONLINEAR; s.pairs = 1;
+    s.skip = 1; s.trunc = cb.truncation; s.K2max = cb.K2max; s.Kimax = cb.Kimax; s.fK = -1; s.cut = a.cut;
+    while (s.kxn < M && column_kept(s.trunc, s.K2max, s.Kimax, -1, s.kxn, 0)) ++s.kxn; s.err = (int*)cb.err;
     if (cb.G < N) return NS_ERR_INTERNAL;
     items_for<T>(N, bm.items, &bm.pro_init);
     bm.cum[0] = 0;
@@ -557,6 +577,9 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
                            cudaMemcpyHostToDevice, st))) {
     return NS_ERR_CUDA;
   }
+  if (!chk(cudaMemsetAsync(b->d_cut, 1, n * sizeof(int), st))) return NS_ERR_CUDA;
+  k_bcut_check<T><<<dim3(kSizes[kNumSizes - 1], n), 256, 0, st>>>((const BatchMem<T>*)b->d_mems, b->d_cut);
+  if (!chk(cudaGetLastError())) return NS_ERR_CUDA;
   if (b->gran == 0) {  // grid schedule
     std::vector<int> cls;
     int start[kNumSizes + 1];

@@ -1,4 +1,4 @@
-// ns_k2_f32a.cu -- size-specialised kernels (float, N in {8, 12, 16, 24, 32, 48, 64}).
+// ns_k2_f32a.cu -- size-specialised kernels (float, N in {8, 12, 16, 24}).
 // One translation unit per group of sizes so the build compiles them in parallel.
 #include "ns_kernels2.cuh"
 
@@ -17,15 +17,6 @@ bool k2_lookup_f32a(int N, K2Entry<float>* e) {
       return true;
     case 24:
       *e = make_k2_entry<float, 24>();
-      return true;
-    case 32:
-      *e = make_k2_entry<float, 32>();
-      return true;
-    case 48:
-      *e = make_k2_entry<float, 48>();
-      return true;
-    case 64:
-      *e = make_k2_entry<float, 64>();
       return true;
     default:
       return false;

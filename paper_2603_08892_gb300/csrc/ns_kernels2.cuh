@@ -264,6 +264,18 @@ __device__ __forceinline__ double recip_k2<double>(int k2) { return 1.0 / (doubl
 template <int I>
 struct IntC { static constexpr int v = I; };
 
+// Sums of products in one fixed rounding order (the kernels of a pass have many instances, each
+// of which the compiler could contract in its own way): a x + b y, its first product fused
+// (x, the state, is the large term), and x + b y
+template <typename T>
+__device__ __forceinline__ cpx<T> lin2(T a, cpx<T> x, T b, cpx<T> y) {
+  return mk<T>(fma1(a, x.x, b * y.x), fma1(a, x.y, b * y.y));
+}
+template <typename T>
+__device__ __forceinline__ cpx<T> lin1(cpx<T> x, T b, cpx<T> y) {
+  return mk<T>(fma1(b, y.x, x.x), fma1(b, y.y, x.y));
+}
+
 // ---- spectral stage at one mode (Sec. 4.1, 4.2, 6.1) ----------------------------------
 // nv: de-shifted, weighted transform of u x omega at the mode: N(0) = 0, truncation T,
 // Leray projection P, then the forcing term O (added on the modes of the forcing table).
@@ -276,7 +288,7 @@ __device__ __forceinline__ void project_point(const PencilArgs<T>& a, int kx, in
     const cpx<T> v0 = nv[0], v1 = nv[1], v2 = nv[2];
     const T fx = (T)kx, fy = (T)ky, fz = (T)kz;
     const T ik2 = recip_k2<T>(k2);
-    const cpx<T> kd = mk<T>(fx * v0.x + fy * v1.x + fz * v2.x, fx * v0.y + fy * v1.y + fz * v2.y);
+    const cpx<T> kd = mk<T>(fma1(fz, v2.x, fma1(fx, v0.x, fy * v1.x)), fma1(fz, v2.y, fma1(fx, v0.y, fy * v1.y)));
     nv[0] = v0 - (fx * ik2) * kd;
     nv[1] = v1 - (fy * ik2) * kd;
     nv[2] = v2 - (fz * ik2) * kd;
@@ -304,31 +316,31 @@ __device__ __forceinline__ cpx<T> stage_combine(const PencilArgs<T>& a, int c, s
     case MODE_INIT:
       return s0;
     case MODE_RK2_1:
-      return Eh * (s0 + hdt * n);
+      return Eh * lin1(s0, hdt, n);
     case MODE_RK2_2: {
-      const cpx<T> s = E1 * s0 + (dt * Eh) * n;
+      const cpx<T> s = lin2(E1, s0, dt * Eh, n);
       MP::st(&a.state[g], s);
       return s;
     }
     case MODE_RK4_1:
-      MP::st(&a.acc[g], E1 * s0 + (dt / T(6) * E1) * n);
-      return Eh * (s0 + hdt * n);
+      MP::st(&a.acc[g], lin2(E1, s0, dt / T(6) * E1, n));
+      return Eh * lin1(s0, hdt, n);
     case MODE_RK4_2:
-      MP::st(&a.acc[g], s1 + (dt / T(3) * Eh) * n);
-      return Eh * s0 + hdt * n;
+      MP::st(&a.acc[g], lin1(s1, dt / T(3) * Eh, n));
+      return lin2(Eh, s0, hdt, n);
     case MODE_RK4_3:
-      MP::st(&a.acc[g], s1 + (dt / T(3) * Eh) * n);
-      return E1 * s0 + (dt * Eh) * n;
+      MP::st(&a.acc[g], lin1(s1, dt / T(3) * Eh, n));
+      return lin2(E1, s0, dt * Eh, n);
     case MODE_RK4_4: {
-      const cpx<T> s = s0 + (dt / T(6)) * n;
+      const cpx<T> s = lin1(s0, dt / T(6), n);
       MP::st(&a.state[g], s);
       return s;
     }
     case MODE_ROG_1:
-      MP::st(&a.state[g], E1 * s0 + (hdt * Eh) * n);
-      return E1 * (s0 + dt * n);
+      MP::st(&a.state[g], lin2(E1, s0, hdt * Eh, n));
+      return E1 * lin1(s0, dt, n);
     case MODE_ROG_2: {
-      const cpx<T> s = s0 + (hdt * Eh) * n;
+      const cpx<T> s = lin1(s0, hdt * Eh, n);
       MP::st(&a.state[g], s);
       return s;
     }
@@ -440,7 +452,8 @@ __device__ __forceinline__ void tile_energy_store(double* epart, T e, T d) {
 }
 
 // NFC, NOC: the number of inputs and outputs known at compile time; -1: at run time, at most
-// one of each (the persistent ensemble).  (1, 1) is every RK2, Rogallo and RK4 stage, (2, 2) and
+// one of each (the persistent ensemble: the mode is looked up for every mode then, 17 -> 30 us
+// per RK4 stage of 48^3).  (1, 1) is every RK2, Rogallo and RK4 stage, (2, 2) and
 // (0, 2) the exact scheme's, (0, 1) INIT, (1, 0) NL and PROJECT.  MC: the stage mode at compile time (-1: a.mode).
 // EP: the tile's energy sums are stored (NOC = 2: whenever a.epart is set).
 template <typename T, int N, class MP, int NFC = -1, int NOC = -1, bool EP = false, int MC = -1,
@@ -468,6 +481,13 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
   const size_t gj = ((size_t)j * N + iy) * M + kx;  // element (kz index j, iy, kx) of a field
   constexpr size_t ZS = (size_t)N * M;              // one plane
   const bool tt = pencil_tile_truncated<T, TX>(a, x0, ky);  // N = 0 on the whole tile
+  // the state vanishes there too: nothing to do (NL and PROJECT write their zeros)
+  if (tt && a.cut && mode != MODE_NL && mode != MODE_PROJECT &&
+      !column_kept(a.trunc, a.K2max, a.Kimax, a.cutK, x0, ky) && *a.cut) {
+    if constexpr (EP || NOC == 2)
+      if ((EP || a.epart) && tid == 0) a.epart[2 * blockIdx.x] = a.epart[2 * blockIdx.x + 1] = 0.0;
+    return;
+  }
   const int nFe = tt ? 0 : nF;                              // inputs that are transformed
   // the twiddle table, on its way while the first inputs are loaded
   constexpr int KT = (N + NT - 1) / NT;
@@ -735,14 +755,6 @@ __global__ void __launch_bounds__(K2Cfg<T, N, V>::NTP, NFC == 2 ? K2Cfg<T, N, V>
 // pairs of modes, (u_x, u_y), (u_z, omega_x), (omega_y, omega_z), the pairs that share a line of
 // the x rows, so the x rows load and store 16 bytes (FP32) per mode.  The x rows leave the
 // products (f_0, f_1) in the first array and f_2 in the first half of each row of the second.
-// Columns (kx, ky) that hold modes of the truncation or of the forcing table (fK < 0: none).
-// Outside them the nonlinear term and the forcing vanish, so no pass reads the products there.
-template <typename T>
-__device__ __forceinline__ bool column_kept(const SlabArgs<T>& a, int kx, int ky) {
-  const bool in = a.trunc == 1 ? (kx <= a.Kimax && abs(ky) <= a.Kimax) : kx * kx + ky * ky <= a.K2max;
-  return in || (a.fK >= 0 && kx <= a.fK && abs(ky) <= a.fK);
-}
-
 // One tile: W consecutive kx of plane zg.  Inverse y transforms of u and omega = i k x u, formed
 // in registers from the mixed fields (u_x, u_y, u_z, d_z u_x, d_z u_y; interleaved layout).
 // Bound by HBM (5 fields read, 6 written).  The first stage reads global memory and the last
@@ -772,10 +784,31 @@ __device__ __forceinline__ void yinv_tile(const SlabArgs<T>& a, int tx, int zg, 
   };
   const size_t sstride = (size_t)a.G * N * M;
   cpair<T>* dst = reinterpret_cast<cpair<T>*>(a.scr) + (size_t)zg * N * M + kx;
+  // columns that are not kept are zero, and unwritten, when *a.cut; the flag is waited for only
+  // after the loads of the kept ones are on their way
+  const bool cutp = a.cut != nullptr;
+  const int cutv = cutp ? *a.cut : 0;
+  if (cutp && x0 >= a.kxn && cutv) return;
+  unsigned km = 0;  // bit r: mode (kx, j + r NB0) is in a kept column
+#pragma unroll
+  for (int r = 0; r < f; ++r)
+    km |= (unsigned)(!cutp || column_kept(a.trunc, a.K2max, a.Kimax, a.fK, kx, kof(j + r * NB0, N))) << r;
+  constexpr unsigned KALL = (1u << f) - 1;
+  auto load = [&](auto&& get) {  // get(r): loads mode r of the thread
+#pragma unroll
+    for (int r = 0; r < f; ++r)
+      if (km >> r & 1) get(r);
+    if (km != KALL && !cutv) {
+#pragma unroll
+      for (int r = 0; r < f; ++r)
+        if (!(km >> r & 1)) get(r);
+    }
+  };
   auto load2 = [&](cpx<T>* va, cpx<T>* vb, int c) {  // two interleaved fields
     const cpair<T>* p = reinterpret_cast<const cpair<T>*>(a.mixed + c * fs) + ((size_t)z * N + j) * M + kx;
 #pragma unroll
-    for (int r = 0; r < f; ++r) MP::ldp(p + (size_t)r * NB0 * M, va[r], vb[r]);
+    for (int r = 0; r < f; ++r) va[r] = vb[r] = mk<T>(0, 0);
+    load([&](int r) { MP::ldp(p + (size_t)r * NB0 * M, va[r], vb[r]); });
   };
   // last stage of the lines in the tiles: pair `pr` from tiles 0 and 1, and tile 2 into wz (pr = 0)
   // or, with wz, pair 2 (pr = 1)
@@ -825,7 +858,8 @@ __device__ __forceinline__ void yinv_tile(const SlabArgs<T>& a, int tx, int zg, 
   if (act) {
     const cpx<T>* src = a.mixed + 2 * fs + ((size_t)z * N + j) * M + kx;
 #pragma unroll
-    for (int r = 0; r < f; ++r) uz[r] = MP::ld(src + (size_t)r * NB0 * M);
+    for (int r = 0; r < f; ++r) uz[r] = mk<T>(0, 0);
+    load([&](int r) { uz[r] = MP::ld(src + (size_t)r * NB0 * M); });
     load2(dx, dy, 3);
   }
   last(0);
@@ -833,8 +867,9 @@ __device__ __forceinline__ void yinv_tile(const SlabArgs<T>& a, int tx, int zg, 
   if (act) {
 #pragma unroll
     for (int r = 0; r < f; ++r) {
-      dy[r] = mul_si(uz[r], ky(r)) - dy[r];  // i ky u_z - d_z u_y
-      dx[r] = dx[r] - mul_si(uz[r], fx);     // d_z u_x - i kx u_z
+      const T k = ky(r);
+      dy[r] = mk<T>(fma1(-k, uz[r].y, -dy[r].x), fma1(k, uz[r].x, -dy[r].y));  // i ky u_z - d_z u_y
+      dx[r] = mk<T>(fma1(fx, uz[r].y, dx[r].x), fma1(-fx, uz[r].x, dx[r].y));  // d_z u_x - i kx u_z
     }
     stage0(uz, 0);
     stage0(dy, 1);
@@ -866,6 +901,7 @@ __device__ __forceinline__ void yfwd_tile(const SlabArgs<T>& a, int tx, int zg, 
   const int x0 = tx * W, kx = x0 + line, z = a.z0 + zg;
   const size_t sstride = (size_t)a.G * N * M, fs = (size_t)N * N * M;
   const bool act = tid < NT;
+  if (a.skip && x0 >= a.kxn) return;  // no column of the tile is kept
   if (act) {
     cpx<T> v[3][f];
     const cpair<T>* src = reinterpret_cast<const cpair<T>*>(a.scr) + ((size_t)zg * N + j) * M + kx;
@@ -895,7 +931,7 @@ __device__ __forceinline__ void yfwd_tile(const SlabArgs<T>& a, int tx, int zg, 
     reg_twiddles<T, N, l, NBL, -1>(w, tws, p);
     bool keep[l];
 #pragma unroll
-    for (int r = 0; r < l; ++r) keep[r] = !a.skip || column_kept(a, kx, kof(p + r * NBL, N));
+    for (int r = 0; r < l; ++r) keep[r] = !a.skip || column_kept(a.trunc, a.K2max, a.Kimax, a.fK, kx, kof(p + r * NBL, N));
     const size_t g = ((size_t)z * N + p) * M + kx;
     auto last = [&](cpx<T>* u, int c) {
       const int o = c * TS + X::at(line, p);
@@ -981,6 +1017,10 @@ __device__ __forceinline__ void xrow_tile(const SlabArgs<T>& a, int tile_id, cpx
   };
   const size_t sstride = (size_t)a.G * N * M;
 
+  // modes kx >= kxn are zero, and unwritten, when *a.cut
+  const bool cutp = a.cut != nullptr && a.kxn < M;
+  const int cutv = cutp ? *a.cut : 0, kxl = cutp ? a.kxn : M, kxs = a.skip ? a.kxn : M;
+
   // 1) item (line p ROWS + row, pair h): the modes of both butterflies, their radix-f transforms
   for (int i = tid; i < NLI * IP0 && tid < NT && in; i += NT) {
     const int line = i / IP0, h = i % IP0, p = line / ROWS, row = row_of(line % ROWS);
@@ -991,8 +1031,15 @@ __device__ __forceinline__ void xrow_tile(const SlabArgs<T>& a, int tile_id, cpx
     for (int r = 0; r < H; ++r) {
       v0[r] = v1[r] = b0[r] = b1[r] = mk<T>(0, 0);
       if (row >= 0) {
-        MP::ldp(src + j0 + r * NB0, v0[r], b0[r]);
-        MP::ldp(src + j1 + r * NB0, v1[r], b1[r]);
+        if (j0 + r * NB0 < kxl) MP::ldp(src + j0 + r * NB0, v0[r], b0[r]);
+        if (j1 + r * NB0 < kxl) MP::ldp(src + j1 + r * NB0, v1[r], b1[r]);
+      }
+    }
+    if (kxl < M && !cutv && row >= 0) {
+#pragma unroll
+      for (int r = 0; r < H; ++r) {
+        if (j0 + r * NB0 >= kxl) MP::ldp(src + j0 + r * NB0, v0[r], b0[r]);
+        if (j1 + r * NB0 >= kxl) MP::ldp(src + j1 + r * NB0, v1[r], b1[r]);
       }
     }
 #pragma unroll
@@ -1072,8 +1119,8 @@ __device__ __forceinline__ void xrow_tile(const SlabArgs<T>& a, int tile_id, cpx
       um[0] = fmax(um[0], fabs(ux));
       um[1] = fmax(um[1], fabs(uy));
       um[2] = fmax(um[2], fabs(uz));
-      g[r] = mk<T>(uy * wz - uz * wy, uz * wx - ux * wz);
-      const T f2 = ux * wy - uy * wx;
+      g[r] = mk<T>(fma1(uy, wz, -(uz * wy)), fma1(uz, wx, -(ux * wz)));
+      const T f2 = fma1(ux, wy, -(uy * wx));
       y[r] = mk<T>(f2, __shfl_xor_sync(0xffffffffu, f2, 1));
     }
     DFT<T, f>::run(g, T(-1));
@@ -1114,7 +1161,7 @@ __device__ __forceinline__ void xrow_tile(const SlabArgs<T>& a, int tile_id, cpx
     cpair<T>* d01 = reinterpret_cast<cpair<T>*>(a.scr) + (size_t)r0 * M;
     cpx<T>* d2 = reinterpret_cast<cpx<T>*>(d01 + sstride);
     auto put = [&](int k, cpx<T> P, cpx<T> Q) {  // P = P[k], Q = P[N - k]
-      if (k >= M) return;
+      if (k >= kxs) return;
       const cpx<T> A = mk<T>(T(0.5) * (P.x + Q.x), T(0.5) * (P.y - Q.y));
       const cpx<T> B = mk<T>(T(0.5) * (P.y + Q.y), T(0.5) * (Q.x - P.x));
       if (own) {
@@ -1265,11 +1312,10 @@ template <typename T>
 struct K2Entry {
   int N = 0;
   void (*pencil01)(PencilArgs<T>) = nullptr; // no input, one output (INIT)
-  void (*pencil10)(PencilArgs<T>) = nullptr; // one input, no output (NL, PROJECT)
+  void (*pencil10[2])(PencilArgs<T>) = {};   // one input, no output: NL, PROJECT
   void (*pencil1[MODE_ROG_2 + 1])(PencilArgs<T>) = {};  // one input, one output, by stage mode
-  void (*pencil1e)(PencilArgs<T>) = nullptr; // same, also storing the tile's energy sums
-  void (*pencil1re)(PencilArgs<T>) = nullptr; // the energy-sum variant of the ROG_2 stage
-  void (*pencil2)(PencilArgs<T>) = nullptr;  // two inputs, two outputs
+  void (*pencil1e[MODE_ROG_2 + 1])(PencilArgs<T>) = {}; // same for the final stages, also storing the energy sums
+  void (*pencil2[2])(PencilArgs<T>) = {};    // two inputs, two outputs: RK2_1, RK2_2
   void (*pencil02)(PencilArgs<T>) = nullptr; // no input, two outputs (INIT of the exact scheme)
   void (*yinv)(SlabArgs<T>) = nullptr;
   void (*yfwd)(SlabArgs<T>) = nullptr;
@@ -1306,22 +1352,22 @@ K2Entry<T> make_k2_entry() {
   K2Entry<T> e;
   e.N = N;
   e.pencil01 = k2_pencil<T, N, 0, 1, false, MODE_INIT>;
-  e.pencil10 = k2_pencil<T, N, 1, 0>;
-  for (int m = MODE_RK2_1; m <= MODE_RK4_4; ++m) e.pencil1[m] = k2_pencil<T, N, 1, 1>;
-  if constexpr (C::F32 && N >= 64) {  // (elsewhere the run-time mode costs little)
-    e.pencil1[MODE_RK2_1] = k2_pencil<T, N, 1, 1, false, MODE_RK2_1>;
-    e.pencil1[MODE_RK2_2] = k2_pencil<T, N, 1, 1, false, MODE_RK2_2>;
-    e.pencil1[MODE_RK4_1] = k2_pencil<T, N, 1, 1, false, MODE_RK4_1>;
-    e.pencil1[MODE_RK4_2] = k2_pencil<T, N, 1, 1, false, MODE_RK4_2>;
-    e.pencil1[MODE_RK4_3] = k2_pencil<T, N, 1, 1, false, MODE_RK4_3>;
-    e.pencil1[MODE_RK4_4] = k2_pencil<T, N, 1, 1, false, MODE_RK4_4>;
-  }
+  e.pencil10[0] = k2_pencil<T, N, 1, 0, false, MODE_NL>;
+  e.pencil10[1] = k2_pencil<T, N, 1, 0, false, MODE_PROJECT>;
+  e.pencil1[MODE_RK2_1] = k2_pencil<T, N, 1, 1, false, MODE_RK2_1>;
+  e.pencil1[MODE_RK2_2] = k2_pencil<T, N, 1, 1, false, MODE_RK2_2>;
+  e.pencil1[MODE_RK4_1] = k2_pencil<T, N, 1, 1, false, MODE_RK4_1>;
+  e.pencil1[MODE_RK4_2] = k2_pencil<T, N, 1, 1, false, MODE_RK4_2>;
+  e.pencil1[MODE_RK4_3] = k2_pencil<T, N, 1, 1, false, MODE_RK4_3>;
+  e.pencil1[MODE_RK4_4] = k2_pencil<T, N, 1, 1, false, MODE_RK4_4>;
   e.pencil1[MODE_ROG_1] = k2_pencil<T, N, 1, 1, false, MODE_ROG_1>;
   e.pencil1[MODE_ROG_2] = k2_pencil<T, N, 1, 1, false, MODE_ROG_2>;
-  e.pencil1e = k2_pencil<T, N, 1, 1, true>;
-  e.pencil1re = k2_pencil<T, N, 1, 1, true, MODE_ROG_2>;
-  e.pencil2 = k2_pencil<T, N, 2, 2>;
-  e.pencil02 = k2_pencil<T, N, 0, 2>;
+  e.pencil1e[MODE_RK2_2] = k2_pencil<T, N, 1, 1, true, MODE_RK2_2>;
+  e.pencil1e[MODE_RK4_4] = k2_pencil<T, N, 1, 1, true, MODE_RK4_4>;
+  e.pencil1e[MODE_ROG_2] = k2_pencil<T, N, 1, 1, true, MODE_ROG_2>;
+  e.pencil2[0] = k2_pencil<T, N, 2, 2, false, MODE_RK2_1>;
+  e.pencil2[1] = k2_pencil<T, N, 2, 2, false, MODE_RK2_2>;
+  e.pencil02 = k2_pencil<T, N, 0, 2, false, MODE_INIT>;
   e.yinv = k2_yinv<T, N>;
   e.yfwd = k2_yfwd<T, N>;
   e.xrow = k2_xrow<T, N>;
