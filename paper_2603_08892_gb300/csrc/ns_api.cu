@@ -81,6 +81,11 @@ FFTPlan make_plan(int n, int Ntab) {
   if (a2 == 2) p.radix[p.nst++] = 4;
   if (a2 == 1) p.radix[p.nst++] = 2;
   for (int i = 0; i < a3; ++i) p.radix[p.nst++] = 3;
+  for (int i = 0, ns = 1; i < p.nst; ns *= p.radix[i++]) {
+    p.ns[i] = fast_div(ns);
+    p.nb[i] = fast_div(n / p.radix[i]);
+    p.tstep[i] = n / (ns * p.radix[i]) * p.tw_stride;
+  }
   return p;
 }
 
@@ -90,48 +95,48 @@ int largest_divisor_le(int m, int cap) {
   return 1;
 }
 
-// block size for a batch of nl lines of length n (every stage holds <= 15 values / thread)
-int fft_block(int nl, int n) {
-  const int need = (nl * n + 14) / 15;
-  int bd = 128;
-  while (bd < need) bd *= 2;
-  return bd;
+// threads for nv values, at 8 a thread (what a stage holds), whole warps, 128 to 384
+int fft_block(int nv) {
+  const int bd = ((nv + 7) / 8 + 31) / 32 * 32;
+  return bd < 128 ? 128 : bd > 384 ? 384 : bd;
 }
 
 // splitmix64 (Steele, Lea & Flood 2014): n-th output of the generator seeded with s
 // Tile shapes and launch sizes of the generic (run-time radix) kernels for a grid of N
 // points, elements of cs bytes; shared by the contexts and the allocation-free entry point.
 struct GenericShapes {
-  int TX, bdP;        // pencil: TX columns, threads
-  size_t smP;         // pencil shared memory (4 tiles)
-  int TY, bdY;        // y passes: TY columns, threads
-  size_t smYi, smYf;  // inverse (6 tiles) / forward (3 tiles) shared memory
-  int RX, bdX;        // x rows: RX rows, threads
+  int TX, LX, bdP;    // pencil: TX columns, LX transformed at a time, threads
+  size_t smP;         // pencil shared memory (4 tiles and the shifts' factors)
+  int TY, LY, bdY;    // y passes, likewise
+  size_t smY;         // one tile
+  int RX, bdX;        // x rows: RX rows, threads (six groups)
   size_t smX;         // x-row shared memory (6 fields)
 };
+// Columns: up to 16, fewer until two pencil blocks (three y blocks) fit an SM, but not below 64
+// bytes a row for that.  Rows: as many as groups of 64 threads hold (N <= 1024: at least one).
 GenericShapes generic_shapes(int N, size_t cs) {
   const int M = N / 2;
-  const size_t smax = 200 * 1024;
   GenericShapes g;
   g.TX = largest_divisor_le(M, 16);
-  while (g.TX > 1 && (4 * N * g.TX * cs > smax || fft_block(g.TX, N) > 512)) g.TX = largest_divisor_le(M, g.TX - 1);
-  g.bdP = fft_block(g.TX, N) < 256 ? 256 : fft_block(g.TX, N);
-  g.smP = 4 * (size_t)N * g.TX * cs;
+  while (g.TX > 1 && 4 * N * g.TX * cs > (g.TX * cs > 64 ? 100 : 200) * 1024)
+    g.TX = largest_divisor_le(M, g.TX - 1);
+  g.LX = largest_divisor_le(g.TX, 384 * 8 / N);
+  g.bdP = fft_block(g.LX * N);
+  g.smP = 4 * (size_t)N * g.TX * cs + 64 * cs;
   g.TY = largest_divisor_le(M, 16);
-  while (g.TY > 1 && (6 * N * g.TY * cs > smax || fft_block(g.TY, N) > 512)) g.TY = largest_divisor_le(M, g.TY - 1);
-  g.bdY = fft_block(g.TY, N) < 256 ? 256 : fft_block(g.TY, N);
-  g.smYi = 6 * (size_t)N * g.TY * cs;
-  g.smYf = 3 * (size_t)N * g.TY * cs;
+  while (g.TY > 1 && N * g.TY * cs > 64 * 1024) g.TY = largest_divisor_le(M, g.TY - 1);
+  g.LY = largest_divisor_le(g.TY, 384 * 8 / N);
+  g.bdY = fft_block(g.LY * N);
+  g.smY = (size_t)N * g.TY * cs;
   g.RX = 16;
-  while (g.RX > 1 && (6 * (size_t)g.RX * M * cs > 100 * 1024 || fft_block(g.RX, M) > 512)) g.RX /= 2;
-  g.bdX = fft_block(g.RX, M) < 256 ? 256 : fft_block(g.RX, M);
+  while (g.RX > 1 && g.RX * M > 64 * 8) g.RX /= 2;
+  g.bdX = 6 * (g.RX * M <= 32 * 8 ? 32 : 64);
   g.smX = 6 * (size_t)g.RX * M * cs;
   return g;
 }
 // true when every generic kernel's shared memory fits the device's opt-in limit
 bool generic_shapes_fit(const GenericShapes& g, int optin) {
-  return (long long)g.smP <= optin && (long long)g.smYi <= optin && (long long)g.smYf <= optin &&
-         (long long)g.smX <= optin;
+  return (long long)g.smP <= optin && (long long)g.smY <= optin && (long long)g.smX <= optin;
 }
 
 // Integer bounds of the strict truncation test (Sec. 3.2: modes with |k| >= kmax zeroed):
@@ -314,10 +319,10 @@ struct Solver : SolverBase {
   cpx<T>* shell = nullptr;
   // plans and launch shapes
   FFTPlan pz, py, px;
-  int TX, bdP;
+  int TX, LX, bdP;
   size_t smP;
-  int TY, bdYi, bdYf;
-  size_t smYi, smYf;
+  int TY, LY, bdY;
+  size_t smY;
   int RX, bdX;
   size_t smX;
   int G, Gmax;
@@ -393,8 +398,8 @@ struct Solver : SolverBase {
     px = make_plan(M, N);
     const size_t cs = sizeof(cpx<T>);
     const GenericShapes gs = generic_shapes(N, cs);
-    TX = gs.TX; bdP = gs.bdP; smP = gs.smP;
-    TY = gs.TY; bdYi = bdYf = gs.bdY; smYi = gs.smYi; smYf = gs.smYf;
+    TX = gs.TX; LX = gs.LX; bdP = gs.bdP; smP = gs.smP;
+    TY = gs.TY; LY = gs.LY; bdY = gs.bdY; smY = gs.smY;
     RX = gs.RX; bdX = gs.bdX; smX = gs.smX;
     // initial plane group: a scratch (6 fields) of 48 MB, small enough for L2
     const size_t plane6 = 6 * (size_t)N * M * cs;
@@ -581,6 +586,7 @@ struct Solver : SolverBase {
     memset(&a, 0, sizeof(a));
     a.N = N; a.M = M; a.py = py; a.px = px; a.tw = tw; a.scr = scr;
     a.TY = TY; a.RX = RX; a.err = d_err;
+    a.LY = LY; a.dLY = fast_div(LY); a.dNP = fast_div(M / 2 + 1);
     a.pairs = pairs();
     if (use2) {  // Ft columns that no pencil pass uses are left unwritten
       a.skip = 1;
@@ -668,7 +674,7 @@ struct Solver : SolverBase {
       else
         k2.yinv<<<dim3(M / k2.TYI, a.G), k2.NTYI, k2.smYI, s>>>(a);
     else
-      k_yinv<T><<<dim3(M / TY, a.G), bdYi, smYi, s>>>(a);
+      k_yinv<T><<<dim3(M / TY, a.G, 6), bdY, smY, s>>>(a);
     prof_end(e, s);
     e = prof_begin(NS_PROF_XROW, s);
     if (use2)
@@ -683,7 +689,7 @@ struct Solver : SolverBase {
       else
         k2.yfwd<<<dim3((a.kxn + k2.TY - 1) / k2.TY, a.G), k2.NTY, k2.smY, s>>>(a);
     else
-      k_yfwd<T><<<dim3(M / TY, a.G), bdYf, smYf, s>>>(a);
+      k_yfwd<T><<<dim3(M / TY, a.G, 3), bdY, smY, s>>>(a);
     prof_end(e, s);
   }
 
@@ -760,7 +766,7 @@ struct Solver : SolverBase {
   PencilArgs<T> pencil_args(int mode) {
     PencilArgs<T> a;
     memset(&a, 0, sizeof(a));
-    a.N = N; a.M = M; a.TX = TX; a.pz = pz; a.tw = tw; a.mode = mode;
+    a.N = N; a.M = M; a.TX = TX; a.LX = LX; a.dTX = fast_div(TX); a.dLX = fast_div(LX); a.pz = pz; a.tw = tw; a.mode = mode;
     a.dt = (T)cur_dt; a.ifac = ifac; a.state = state; a.acc = acc;
     a.trunc = c->p.truncation; a.K2max = c->K2max; a.Kimax = c->Kimax;
     a.err = d_err;
@@ -1541,7 +1547,7 @@ struct Solver : SolverBase {
       a.z0 = z0;
       a.G = (z0 + G <= N) ? G : N - z0;
       k_xrow<T><<<(a.G * N + RX - 1) / RX, bdX, smX, st>>>(a);
-      k_yfwd<T><<<dim3(M / TY, a.G), bdYf, smYf, st>>>(a);
+      k_yfwd<T><<<dim3(M / TY, a.G, 3), bdY, smY, st>>>(a);
     }
     LAUNCH_CHECK();
     PencilArgs<T> p = pencil_args(MODE_PROJECT);
@@ -1567,7 +1573,7 @@ struct Solver : SolverBase {
     for (int z0 = 0; z0 < N; z0 += G) {
       a.z0 = z0;
       a.G = (z0 + G <= N) ? G : N - z0;
-      k_yinv<T><<<dim3(M / TY, a.G), bdYi, smYi, st>>>(a);
+      k_yinv<T><<<dim3(M / TY, a.G, 3), bdY, smY, st>>>(a);
       k_xrow<T><<<(a.G * N + RX - 1) / RX, bdX, smX, st>>>(a);
     }
     LAUNCH_CHECK();
@@ -1691,9 +1697,9 @@ struct Solver : SolverBase {
     for (int z0 = 0; z0 < N; z0 += G) {
       a.z0 = z0;
       a.G = (z0 + G <= N) ? G : N - z0;
-      k_yinv<T><<<dim3(M / TY, a.G), bdYi, smYi, st>>>(a);
+      k_yinv<T><<<dim3(M / TY, a.G, 6), bdY, smY, st>>>(a);
       k_xrow<T><<<(a.G * N + RX - 1) / RX, bdX, smX, st>>>(a);
-      k_yfwd<T><<<dim3(M / TY, a.G), bdYf, smYf, st>>>(a);
+      k_yfwd<T><<<dim3(M / TY, a.G, 3), bdY, smY, st>>>(a);
     }
     LAUNCH_CHECK();
   }
@@ -2588,7 +2594,7 @@ extern "C" int ns_nonlinear_noalloc(const void* state, void* out, int N, double 
 
   PencilArgs<float> p;
   memset(&p, 0, sizeof(p));
-  p.N = N; p.M = M; p.TX = g.TX; p.pz = pz; p.tw = tw; p.mode = MODE_INIT;
+  p.N = N; p.M = M; p.TX = g.TX; p.LX = g.LX; p.dTX = fast_div(g.TX); p.dLX = fast_div(g.LX); p.pz = pz; p.tw = tw; p.mode = MODE_INIT;
   p.src = static_cast<const cpx<float>*>(state);
   p.trunc = truncation; p.K2max = K2max; p.Kimax = Kimax; p.err = err;
   p.nOut = 1; p.osh[0] = sh; p.out[0] = mixed;
@@ -2597,10 +2603,11 @@ extern "C" int ns_nonlinear_noalloc(const void* state, void* out, int N, double 
   SlabArgs<float> a;
   memset(&a, 0, sizeof(a));
   a.N = N; a.M = M; a.py = pz; a.px = px; a.tw = tw; a.scr = scr; a.TY = g.TY; a.RX = g.RX;
+  a.LY = g.LY; a.dLY = fast_div(g.LY); a.dNP = fast_div(M / 2 + 1);
   a.err = err; a.mixed = mixed; a.Ft = Ft; a.xmode = XMODE_NONLINEAR; a.z0 = 0; a.G = N;
-  k_yinv<float><<<dim3(M / g.TY, N), g.bdY, g.smYi, st>>>(a);
+  k_yinv<float><<<dim3(M / g.TY, N, 6), g.bdY, g.smY, st>>>(a);
   k_xrow<float><<<(N * N + g.RX - 1) / g.RX, g.bdX, g.smX, st>>>(a);
-  k_yfwd<float><<<dim3(M / g.TY, N), g.bdY, g.smYf, st>>>(a);
+  k_yfwd<float><<<dim3(M / g.TY, N, 3), g.bdY, g.smY, st>>>(a);
 
   PencilArgs<float> q = p;
   q.mode = MODE_NL;

@@ -39,6 +39,9 @@ template <typename T>
 __device__ __forceinline__ cpx<T> operator*(T s, cpx<T> a) { return mk(s * a.x, s * a.y); }
 template <typename T>
 __device__ __forceinline__ cpx<T> conjg(cpx<T> a) { return mk(a.x, -a.y); }
+// a b + c in one rounding, whatever the compiler would have contracted
+__device__ __forceinline__ float fma1(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma1(double a, double b, double c) { return __fma_rn(a, b, c); }
 // Complex product in one fixed rounding order (the a.y products rounded, then one fused
 // multiply-add per part), the same bits wherever it is compiled: used where two kernels must
 // form the same value (the shifted fields carried from a step's last pass and the same fields
@@ -114,12 +117,29 @@ __device__ __forceinline__ cpx<double> ldg(const cpx<double>* p) {
   return mk<double>(v.x, v.y);
 }
 
+// Quotients by a small divisor known to the host: t / d = umulhi(t, ceil(2^32 / d)), exact for
+// t, d < 2^16 (m = 0 stands for d = 1).  A run-time division is about 20 instructions, more than a
+// radix-3 butterfly's arithmetic, and a stage needs two per butterfly.
+struct FastDiv {
+  unsigned d, m;
+};
+inline FastDiv fast_div(int d) {
+  FastDiv f;
+  f.d = (unsigned)d;
+  f.m = d > 1 ? (unsigned)(((1ull << 32) + d - 1) / d) : 0u;
+  return f;
+}
+__device__ __forceinline__ int fdiv(int t, FastDiv f) { return f.m ? (int)__umulhi((unsigned)t, f.m) : t; }
+
 // Radix plan of a length-n transform: n = prod radix[s].
 struct FFTPlan {
   int n;          // transform length
   int nst;        // number of stages
   int tw_stride;  // (table length N) / n
   int radix[16];
+  FastDiv ns[16];  // product of the earlier stages' radices
+  FastDiv nb[16];  // butterflies of a line, n / radix
+  int tstep[16];   // twiddle table step, n / (ns radix) tw_stride
 };
 
 // ----------------------------------------------------------------------------------------
@@ -235,48 +255,60 @@ struct DFT<float, 8> {
 };
 #endif
 
-// Butterflies held per thread per stage (R * KB <= 16 values in registers).
+// Butterflies held per thread per stage: 8 or 9 values in registers (16 and fewer threads spill).
 template <int R>
 struct StageKB {
-  static constexpr int value = (R == 2) ? 8 : (R == 3) ? 5 : (R == 4) ? 4 : 2;
+  static constexpr int value = (R == 2) ? 4 : (R == 3) ? 3 : (R == 4) ? 2 : 1;
 };
 
-// One Stockham radix-R stage over a batch of nl lines of length n in shared memory.
-// Element e of line l is buf[l * ls + e * es].  line_fast: consecutive threads take
-// consecutive lines (use when es > 1) rather than consecutive butterflies of one line.
-// Requires nl * n / R <= StageKB<R> * blockDim.x (checked; *err set otherwise).
-template <typename T, int R>
-__device__ __forceinline__ void stockham_stage(cpx<T>* buf, int n, int nl, int es, int ls,
-                                               bool line_fast, int Ns,
-                                               const cpx<T>* __restrict__ tw, int tw_stride,
-                                               T s, int* err) {
+// A batch of lines of length pl.n, nl at a time (chunks times), worked on by nt threads (t0: this
+// thread's index among them); element e of line l is buf[l * ls + e * es].  line_fast: consecutive
+// threads take consecutive lines (use when es > 1) rather than consecutive butterflies of one line.
+struct LineBatch {
+  int nl, chunks, es, ls, t0, nt;
+  bool line_fast;
+  FastDiv dl;  // nl (line_fast)
+};
+
+// One Stockham radix-R stage: the first reads rd(line, e) unless the batch is in buf already
+// (from_buf), the last writes wr(line, e, v); the others go through buf in place.
+// Requires nl * n / R <= StageKB<R> * nt (checked; *err set otherwise).
+template <typename T, int R, class Rd, class Wr>
+__device__ __forceinline__ void stockham_stage(cpx<T>* buf, const FFTPlan& pl, int st, const LineBatch& lb,
+                                               int l0, bool first, bool last, const cpx<T>* __restrict__ tw, T s,
+                                               int* err, Rd& rd, Wr& wr) {
   constexpr int KB = StageKB<R>::value;
-  const int nb = n / R;
-  const int total = nb * nl;
-  if (total > KB * (int)blockDim.x) {
-    if (threadIdx.x == 0 && err) atomicOr(err, 1);
-    return;
+  const FastDiv dnb = pl.nb[st], dns = pl.ns[st];
+  const int nb = dnb.d, Ns = dns.d;
+  int total = nb * lb.nl;
+  if (total > KB * lb.nt) {
+    if (lb.t0 == 0 && err) atomicOr(err, 1);
+    total = 0;
   }
+  auto place = [&](int b, int& line, int& j) {
+    const int q = fdiv(b, lb.line_fast ? lb.dl : dnb);
+    const int r = b - q * (lb.line_fast ? lb.nl : nb);
+    line = l0 + (lb.line_fast ? r : q);
+    j = lb.line_fast ? q : r;
+  };
   cpx<T> v[KB][R];
-  const int tstep = (n / (Ns * R)) * tw_stride;
+  const int tstep = pl.tstep[st];
 #pragma unroll
   for (int c = 0; c < KB; ++c) {
-    const int b = threadIdx.x + c * blockDim.x;
+    const int b = lb.t0 + c * lb.nt;
     if (b < total) {
       int line, j;
-      if (line_fast) {
-        line = b % nl;
-        j = b / nl;
-      } else {
-        j = b % nb;
-        line = b / nb;
-      }
-      const cpx<T>* src = buf + line * ls;
+      place(b, line, j);
+      if (first) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[c][r] = src[(j + r * nb) * es];
+        for (int r = 0; r < R; ++r) v[c][r] = rd(line, j + r * nb);
+      } else {
+        const cpx<T>* src = buf + line * lb.ls;
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[c][r] = src[(j + r * nb) * lb.es];
+      }
       if (Ns > 1) {
-        const int p = j % Ns;
-        const int base = p * tstep;
+        const int base = (j - fdiv(j, dns) * Ns) * tstep;
 #pragma unroll
         for (int r = 1; r < R; ++r) {
           cpx<T> w = ldg(&tw[r * base]);
@@ -287,52 +319,52 @@ __device__ __forceinline__ void stockham_stage(cpx<T>* buf, int n, int nl, int e
       DFT<T, R>::run(v[c], s);
     }
   }
-  __syncthreads();
+  if (!first) __syncthreads();  // all reads of buf before its values are written over
 #pragma unroll
   for (int c = 0; c < KB; ++c) {
-    const int b = threadIdx.x + c * blockDim.x;
+    const int b = lb.t0 + c * lb.nt;
     if (b < total) {
       int line, j;
-      if (line_fast) {
-        line = b % nl;
-        j = b / nl;
-      } else {
-        j = b % nb;
-        line = b / nb;
-      }
-      const int p = j % Ns, q = j / Ns;
-      cpx<T>* dst = buf + line * ls;
-      const int o = q * Ns * R + p;
+      place(b, line, j);
+      const int q = fdiv(j, dns);
+      const int o = q * Ns * R + (j - q * Ns);
+      if (last) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) dst[(o + r * Ns) * es] = v[c][r];
+        for (int r = 0; r < R; ++r) wr(line, o + r * Ns, v[c][r]);
+      } else {
+        cpx<T>* dst = buf + line * lb.ls;
+#pragma unroll
+        for (int r = 0; r < R; ++r) dst[(o + r * Ns) * lb.es] = v[c][r];
+      }
     }
   }
-  __syncthreads();
+  if (!last) __syncthreads();
 }
 
-// Full transform of a batch of lines (forward if s = -1, inverse if s = +1).
-template <typename T>
-__device__ __forceinline__ void fft_lines(cpx<T>* buf, const FFTPlan& pl, int nl, int es, int ls,
-                                          bool line_fast, const cpx<T>* __restrict__ tw, T s,
-                                          int* err) {
-  int Ns = 1;
-  for (int st = 0; st < pl.nst; ++st) {
-    const int R = pl.radix[st];
-    switch (R) {
+// Full transforms of a batch of lines (forward if s = -1, inverse if s = +1), called by every
+// thread of the block.  rd may not read buf; after the call buf is free unless wr writes to it (then
+// the caller synchronises before those values are read by other threads).
+template <typename T, class Rd, class Wr>
+__device__ __forceinline__ void fft_lines(cpx<T>* buf, const FFTPlan& pl, const LineBatch& lb, bool from_buf,
+                                          const cpx<T>* __restrict__ tw, T s, int* err, Rd rd, Wr wr) {
+#pragma unroll 1
+  for (int it = 0; it < lb.chunks * pl.nst; ++it) {
+    const int ch = it / pl.nst, st = it - ch * pl.nst, l0 = ch * lb.nl;
+    const bool first = st == 0 && !from_buf, last = st == pl.nst - 1;
+    switch (pl.radix[st]) {
       case 2:
-        stockham_stage<T, 2>(buf, pl.n, nl, es, ls, line_fast, Ns, tw, pl.tw_stride, s, err);
+        stockham_stage<T, 2>(buf, pl, st, lb, l0, first, last, tw, s, err, rd, wr);
         break;
       case 3:
-        stockham_stage<T, 3>(buf, pl.n, nl, es, ls, line_fast, Ns, tw, pl.tw_stride, s, err);
+        stockham_stage<T, 3>(buf, pl, st, lb, l0, first, last, tw, s, err, rd, wr);
         break;
       case 4:
-        stockham_stage<T, 4>(buf, pl.n, nl, es, ls, line_fast, Ns, tw, pl.tw_stride, s, err);
+        stockham_stage<T, 4>(buf, pl, st, lb, l0, first, last, tw, s, err, rd, wr);
         break;
       default:
-        stockham_stage<T, 8>(buf, pl.n, nl, es, ls, line_fast, Ns, tw, pl.tw_stride, s, err);
+        stockham_stage<T, 8>(buf, pl, st, lb, l0, first, last, tw, s, err, rd, wr);
         break;
     }
-    Ns *= R;
   }
 }
 

@@ -11,10 +11,6 @@
 
 namespace ns {
 
-// a b + c in one rounding, whatever the compiler would have contracted
-__device__ __forceinline__ float fma1(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma1(double a, double b, double c) { return __fma_rn(a, b, c); }
-
 // a + b, a - b: packed in FP32 (ns_fft.cuh)
 template <typename T>
 __device__ __forceinline__ cpx<T> cadd(cpx<T> a, cpx<T> b) {

@@ -155,7 +155,8 @@ __global__ void k_shift_tables(cpx<T>* out, int N, const double* __restrict__ de
 // ----------------------------------------------------------------------------------------
 template <typename T>
 struct PencilArgs {
-  int N, M, TX;
+  int N, M, TX, LX;  // LX: columns transformed at a time (the run-time kernels)
+  FastDiv dTX, dLX;
   FFTPlan pz;
   const cpx<T>* tw;
   int nF;                // number of nonlinear inputs (0, 1, 2)
@@ -190,28 +191,13 @@ __device__ __forceinline__ cpx<T> phase3(const cpx<T>* tab, int N, int ix, int i
   return (ldg(&tab[ix]) * ldg(&tab[N + iy])) * ldg(&tab[2 * N + iz]);
 }
 
+// Run-time sizes: one block per ky row and TX columns.  The z transforms' first stages read global
+// memory (or form the shifted values) and their last ones write it: only the stages between them
+// go through shared memory.  216^3 FP32, one in and one out: 394 us a launch, 834 before.  A step of 216^3 (all
+// run-time kernels): 6180 us with run-time divisions, six-tile y passes and 15 values a thread, 3240
+// now; issue-bound (index arithmetic, radix-8 and radix-3 stages).
 template <typename T>
-__device__ __forceinline__ void load_tile(cpx<T>* dst, const cpx<T>* __restrict__ src, int N,
-                                          int M, int TX, int iy, int x0) {
-  const int n = N * TX;
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    int z = e / TX, x = e - z * TX;
-    dst[e] = src[((size_t)z * N + iy) * M + x0 + x];
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void store_tile(cpx<T>* __restrict__ dst, const cpx<T>* src, int N,
-                                           int M, int TX, int iy, int x0) {
-  const int n = N * TX;
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    int z = e / TX, x = e - z * TX;
-    dst[((size_t)z * N + iy) * M + x0 + x] = src[e];
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(512) k_pencil(PencilArgs<T> a) {
+__global__ void __launch_bounds__(384, sizeof(T) == 4 ? 2 : 1) k_pencil(const __grid_constant__ PencilArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   const int N = a.N, M = a.M, TX = a.TX;
@@ -219,43 +205,46 @@ __global__ void __launch_bounds__(512) k_pencil(PencilArgs<T> a) {
   const int iy = a.iy0 + blockIdx.x / ntx;
   const int x0 = (blockIdx.x % ntx) * TX;
   const int tile = N * TX;
-  cpx<T>* b[4] = {buf, buf + tile, buf + 2 * tile, buf + 3 * tile};
   const size_t fstride = (size_t)N * N * M;
   const int ky = kof(iy, N);
+  const LineBatch lb = {a.LX, TX / a.LX, TX, 1, (int)threadIdx.x, (int)blockDim.x, true, a.dLX};
+  cpx<T>* sxy = buf + 4 * tile;  // [4][16]: x and y factors of the shifts' phases (phase3's association)
+  const size_t gz = (size_t)N * M;  // z stride
+  const size_t g0 = (size_t)iy * M + x0;
+  if (threadIdx.x < 64) {
+    const int i = threadIdx.x >> 4, x = threadIdx.x & 15;
+    const cpx<T>* tab = i < 2 ? (i < a.nF ? a.dsh[i] : nullptr) : (i - 2 < a.nOut ? a.osh[i - 2] : nullptr);
+    if (tab && x < TX) sxy[threadIdx.x] = ldg(&tab[x0 + x]) * ldg(&tab[N + iy]);
+  }
+  __syncthreads();
 
   // 1) forward z transforms of the nonlinear inputs, de-shift, weights
-  if (a.nF > 0) {
-    for (int c = 0; c < 3; ++c) {
-      load_tile(b[c], a.F[0] + c * fstride, N, M, TX, iy, x0);
-      __syncthreads();
-      fft_lines(b[c], a.pz, TX, TX, 1, true, a.tw, T(-1), a.err);
-      if (a.nF > 1) {
-        load_tile(b[3], a.F[1] + c * fstride, N, M, TX, iy, x0);
-        __syncthreads();
-        fft_lines(b[3], a.pz, TX, TX, 1, true, a.tw, T(-1), a.err);
-      }
-      for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-        int iz = e / TX, x = e - iz * TX;
-        cpx<T> v = b[c][e];
-        if (a.dsh[0]) v = mul_conj(v, phase3(a.dsh[0], N, x0 + x, iy, iz));
-        v = a.wF[0] * v;
-        if (a.nF > 1) {
-          cpx<T> w = b[3][e];
-          if (a.dsh[1]) w = mul_conj(w, phase3(a.dsh[1], N, x0 + x, iy, iz));
-          v = v + a.wF[1] * w;
-        }
-        b[c][e] = v;
-      }
-      __syncthreads();
+#pragma unroll 1
+  for (int c = 0; c < (a.nF > 0 ? 3 : 0); ++c) {
+    cpx<T>* bc = buf + c * tile;
+    const cpx<T>* F0 = a.F[0] + c * fstride + g0;
+    fft_lines(bc, a.pz, lb, false, a.tw, T(-1), a.err, [&](int x, int z) { return F0[z * gz + x]; },
+              [&](int x, int z, cpx<T> v) {
+                if (a.dsh[0]) v = mul_conj(v, sxy[x] * ldg(&a.dsh[0][2 * N + z]));
+                bc[z * TX + x] = a.wF[0] * v;
+              });
+    if (a.nF > 1) {
+      const cpx<T>* F1 = a.F[1] + c * fstride + g0;
+      fft_lines(buf + 3 * tile, a.pz, lb, false, a.tw, T(-1), a.err, [&](int x, int z) { return F1[z * gz + x]; },
+                [&](int x, int z, cpx<T> w) {
+                  if (a.dsh[1]) w = mul_conj(w, sxy[16 + x] * ldg(&a.dsh[1][2 * N + z]));
+                  bc[z * TX + x] = bc[z * TX + x] + a.wF[1] * w;
+                });
     }
   }
+  __syncthreads();
 
   // 2) pointwise: N(0) = 0, truncation T, projection P, forcing, stage combine
   const T dt = a.dt, hdt = T(0.5) * a.dt;
   const int D1 = 2 * a.fK + 1;
   const int D = D1 * D1 * (a.fK + 1);
   for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-    const int iz = e / TX, x = e - iz * TX;
+    const int iz = fdiv(e, a.dTX), x = e - iz * TX;
     const int kx = x0 + x, kz = kof(iz, N);
     const size_t g = ((size_t)iz * N + iy) * M + kx;
     cpx<T> nv[3];
@@ -263,7 +252,7 @@ __global__ void __launch_bounds__(512) k_pencil(PencilArgs<T> a) {
       const int k2 = kx * kx + ky * ky + kz * kz;
       const bool keep = trunc_keep(a.trunc, kx, ky, kz, N, a.K2max, a.Kimax) && (k2 != 0);
       if (keep) {
-        cpx<T> v0 = b[0][e], v1 = b[1][e], v2 = b[2][e];
+        cpx<T> v0 = buf[e], v1 = buf[tile + e], v2 = buf[2 * tile + e];
         const T fx = (T)kx, fy = (T)ky, fz = (T)kz;
         const T ik2 = T(1) / (T)k2;
         cpx<T> kd = mk<T>(fx * v0.x + fy * v1.x + fz * v2.x, fx * v0.y + fy * v1.y + fz * v2.y);
@@ -336,7 +325,7 @@ __global__ void __launch_bounds__(512) k_pencil(PencilArgs<T> a) {
           a.state[gi] = nv[c];
           break;
       }
-      b[c][e] = sn;
+      buf[c * tile + e] = sn;
       if (a.shell && kx <= a.fK && abs(ky) <= a.fK && abs(kz) <= a.fK) {
         const int fi = ((kz + a.fK) * D1 + (ky + a.fK)) * (a.fK + 1) + kx;
         a.shell[c * D + fi] = sn;
@@ -346,20 +335,21 @@ __global__ void __launch_bounds__(512) k_pencil(PencilArgs<T> a) {
   __syncthreads();
 
   // 3) outputs: shift, z-derivatives, inverse z transforms
+#pragma unroll 1
   for (int o = 0; o < a.nOut; ++o) {
+    const cpx<T>* osh = a.osh[o];
+#pragma unroll 1
     for (int f = 0; f < 5; ++f) {
-      const int c = f < 3 ? f : f - 3;
-      for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-        const int iz = e / TX, x = e - iz * TX;
-        cpx<T> v = b[c][e];
-        if (a.osh[o]) v = v * phase3(a.osh[o], N, x0 + x, iy, iz);
-        if (f >= 3) v = mul_si(v, (T)kof(iz, N));  // i kz v
-        b[3][e] = v;
-      }
-      __syncthreads();
-      fft_lines(b[3], a.pz, TX, TX, 1, true, a.tw, T(1), a.err);
-      store_tile(a.out[o] + f * fstride, b[3], N, M, TX, iy, x0);
-      __syncthreads();
+      const cpx<T>* S = buf + (f < 3 ? f : f - 3) * tile;
+      cpx<T>* dst = a.out[o] + f * fstride + g0;
+      fft_lines(buf + 3 * tile, a.pz, lb, false, a.tw, T(1), a.err,
+                [&](int x, int z) {
+                  cpx<T> v = S[z * TX + x];
+                  if (osh) v = v * (sxy[32 + 16 * o + x] * ldg(&osh[2 * N + z]));
+                  if (f >= 3) v = mul_si(v, (T)kof(z, N));  // i kz v
+                  return v;
+                },
+                [&](int x, int z, cpx<T> v) { dst[z * gz + x] = v; });
     }
   }
 }
@@ -370,6 +360,8 @@ __global__ void __launch_bounds__(512) k_pencil(PencilArgs<T> a) {
 template <typename T>
 struct SlabArgs {
   int N, M, z0, G;
+  int LY;              // columns transformed at a time (the run-time kernels)
+  FastDiv dLY, dNP;    // dNP: M / 2 + 1
   FFTPlan py, px;
   const cpx<T>* tw;
   const cpx<T>* mixed;  // [5][N][N][M]
@@ -421,120 +413,91 @@ __device__ void block_max3(T m0, T m1, T m2, T* scratch, void* umax) {
   __syncthreads();
 }
 
-// inverse y transforms; forms omega = i k x u from the mixed fields (nonlinear mode) or
-// passes the velocity only (C2R mode).  grid (M/TY, G)
+// Inverse y transforms of one field per block: the velocity, or omega = i k x u formed from the
+// mixed fields as they are read.  grid (M/TY, G, fields).  One field per block reads some mixed
+// fields twice (from L2) and needs one tile of shared memory instead of six, so that enough blocks
+// are resident to cover the loads: 216^3 FP32, per 100 planes: 160 us, 400 to 435 before (8 warps an SM).  The
+// products are fused in writing: the compiler merges the branches' subtractions otherwise.
 template <typename T>
-__global__ void __launch_bounds__(512) k_yinv(SlabArgs<T> a) {
+__global__ void __launch_bounds__(384, sizeof(T) == 4 ? 2 : 1) k_yinv(const __grid_constant__ SlabArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   const int N = a.N, M = a.M, TY = a.TY;
   const int x0 = blockIdx.x * TY, zg = blockIdx.y, z = a.z0 + zg;
-  const int tile = N * TY;
+  const int f = blockIdx.z, c = f < 3 ? f : f - 3;
   const size_t fstride = (size_t)N * N * M;
-  const int nf = xmode_cross(a.xmode) ? 6 : 3;
-  for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-    const int iy = e / TY, x = e - iy * TY;
-    const size_t g = ((size_t)z * N + iy) * M + x0 + x;
-    auto mx = [&](const cpx<T>* m, int f) { return m[mixed_index(a.pairs, f, g, fstride)]; };
-    cpx<T> ux = mx(a.mixed, 0), uy = mx(a.mixed, 1), uz = mx(a.mixed, 2);
-    // slots 0..2 and 3..5 of the pair whose cross product the x rows form
-    int su = 0, sw = 3, sr = -1;
-    if (a.xmode == XMODE_ADJ_WR) { sw = 0; sr = 3; su = -1; }
-    if (a.xmode == XMODE_ADJ_RU) { sr = 0; su = 3; sw = -1; }
-    if (su >= 0) {
-      buf[su * tile + e] = ux;
-      buf[(su + 1) * tile + e] = uy;
-      buf[(su + 2) * tile + e] = uz;
-    }
-    if (nf == 6 && sw >= 0) {
-      cpx<T> dzx = mx(a.mixed, 3), dzy = mx(a.mixed, 4);
-      const T kx = (T)(x0 + x), ky = (T)kof(iy, N);
-      buf[sw * tile + e] = mul_si(uz, ky) - dzy;                  // w_x = i ky uz - dz uy
-      buf[(sw + 1) * tile + e] = dzx - mul_si(uz, kx);            // w_y = dz ux - i kx uz
-      buf[(sw + 2) * tile + e] = mul_si(uy, kx) - mul_si(ux, ky); // w_z = i kx uy - i ky ux
-    }
-    if (sr >= 0) {
-      buf[sr * tile + e] = mx(a.mixedB, 0);
-      buf[(sr + 1) * tile + e] = mx(a.mixedB, 1);
-      buf[(sr + 2) * tile + e] = mx(a.mixedB, 2);
-    }
-  }
-  __syncthreads();
-  for (int f = 0; f < nf; ++f) fft_lines(buf + f * tile, a.py, TY, TY, 1, true, a.tw, T(1), a.err);
-  const size_t sstride = (size_t)a.G * N * M;
-  for (int f = 0; f < nf; ++f) {
-    for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-      const int iy = e / TY, x = e - iy * TY;
-      a.scr[f * sstride + ((size_t)zg * N + iy) * M + x0 + x] = buf[f * tile + e];
-    }
-  }
+  // fields 0..2 and 3..5: the pair whose cross product the x rows form (u, omega, or the cotangent r)
+  enum { U, W, RB };
+  int kind = f < 3 ? U : W;
+  if (a.xmode == XMODE_ADJ_WR) kind = f < 3 ? W : RB;
+  if (a.xmode == XMODE_ADJ_RU) kind = f < 3 ? RB : U;
+  const LineBatch lb = {a.LY, TY / a.LY, TY, 1, (int)threadIdx.x, (int)blockDim.x, true, a.dLY};
+  cpx<T>* dst = a.scr + f * (size_t)a.G * N * M + (size_t)zg * N * M + x0;
+  fft_lines(buf, a.py, lb, false, a.tw, T(1), a.err,
+            [&](int x, int iy) {
+              const size_t g = ((size_t)z * N + iy) * M + x0 + x;
+              auto mx = [&](const cpx<T>* m, int i) { return m[mixed_index(a.pairs, i, g, fstride)]; };
+              if (kind == RB) return mx(a.mixedB, c);
+              if (kind == U) return mx(a.mixed, c);
+              const T kx = (T)(x0 + x), ky = (T)kof(iy, N);
+              if (c == 0) {  // w_x = i ky uz - dz uy
+                const cpx<T> uz = mx(a.mixed, 2), d = mx(a.mixed, 4);
+                return mk<T>(fma1(-ky, uz.y, -d.x), fma1(ky, uz.x, -d.y));
+              }
+              if (c == 1) {  // w_y = dz ux - i kx uz
+                const cpx<T> uz = mx(a.mixed, 2), d = mx(a.mixed, 3);
+                return mk<T>(fma1(kx, uz.y, d.x), fma1(-kx, uz.x, d.y));
+              }
+              const cpx<T> uy = mx(a.mixed, 1), ux = mx(a.mixed, 0);  // w_z = i kx uy - i ky ux
+              return mk<T>(fma1(ky, ux.y, -(kx * uy.y)), fma1(kx, uy.x, -(ky * ux.x)));
+            },
+            [&](int x, int iy, cpx<T> v) { dst[(size_t)iy * M + x] = v; });
 }
 
-// forward y transforms of the 3 components of the x-transformed product.  grid (M/TY, G)
+// forward y transforms of one component of the x-transformed product.  grid (M/TY, G, 3)
 template <typename T>
-__global__ void __launch_bounds__(512) k_yfwd(SlabArgs<T> a) {
+__global__ void __launch_bounds__(384, sizeof(T) == 4 ? 2 : 1) k_yfwd(const __grid_constant__ SlabArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   const int N = a.N, M = a.M, TY = a.TY;
-  const int x0 = blockIdx.x * TY, zg = blockIdx.y, z = a.z0 + zg;
-  const int tile = N * TY;
+  const int x0 = blockIdx.x * TY, zg = blockIdx.y, z = a.z0 + zg, f = blockIdx.z;
   const size_t fstride = (size_t)N * N * M;
-  const size_t sstride = (size_t)a.G * N * M;
-  for (int f = 0; f < 3; ++f) {
-    for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-      const int iy = e / TY, x = e - iy * TY;
-      buf[f * tile + e] = a.scr[f * sstride + ((size_t)zg * N + iy) * M + x0 + x];
-    }
-  }
-  __syncthreads();
-  for (int f = 0; f < 3; ++f) fft_lines(buf + f * tile, a.py, TY, TY, 1, true, a.tw, T(-1), a.err);
-  for (int f = 0; f < 3; ++f) {
-    for (int e = threadIdx.x; e < tile; e += blockDim.x) {
-      const int iy = e / TY, x = e - iy * TY;
-      a.Ft[ft_index(a.pairs, f, ((size_t)z * N + iy) * M + x0 + x, fstride)] = buf[f * tile + e];
-    }
-  }
+  const LineBatch lb = {a.LY, TY / a.LY, TY, 1, (int)threadIdx.x, (int)blockDim.x, true, a.dLY};
+  const cpx<T>* src = a.scr + f * (size_t)a.G * N * M + (size_t)zg * N * M + x0;
+  fft_lines(buf, a.py, lb, false, a.tw, T(-1), a.err, [&](int x, int iy) { return src[(size_t)iy * M + x]; },
+            [&](int x, int iy, cpx<T> v) {
+              a.Ft[ft_index(a.pairs, f, ((size_t)z * N + iy) * M + x0 + x, fstride)] = v;
+            });
 }
 
-// Hermitian half spectrum X_0..X_{M-1} (X_M = 0) -> Z'_k whose inverse M-point DFT is the
-// packed real row z_m = x_{2m} + i x_{2m+1}, x_j = sum_{k=0}^{N-1} X_k exp(2 pi i jk/N).
-template <typename T>
-__device__ __forceinline__ void c2r_pre(cpx<T>* row, int M, const cpx<T>* __restrict__ tw,
-                                        int k) {
-  if (k == 0) {
-    const T r = row[0].x;
-    row[0] = mk<T>(r, r);
-    if (M % 2 == 0 && M > 1) {
-      // k = M/2: X_{M-k} = X_k; e^{2 pi i k/N} = e^{i pi/2} = i
-      cpx<T> X = row[M / 2];
-      cpx<T> A = X + conjg(X), B = X - conjg(X);
-      row[M / 2] = A - B;  // A + i * i * B
-    }
-    return;
-  }
-  const int km = M - k;
-  cpx<T> Xk = row[k], Xm = row[km];
-  cpx<T> w = conjg(ldg(&tw[k]));  // e^{+2 pi i k / N}
-  cpx<T> A = Xk + conjg(Xm), B = Xk - conjg(Xm);
-  row[k] = A + mul_si(w * B, T(1));
-  // for M-k: e^{2 pi i (M-k)/N} = -e^{-2 pi i k/N} = -tw[k]
-  cpx<T> A2 = Xm + conjg(Xk), B2 = Xm - conjg(Xk);
-  row[km] = A2 - mul_si(ldg(&tw[k]) * B2, T(1));
+// Hermitian half spectrum X_0..X_{M-1} (X_M = 0; x(i) reads X_i) -> Z'_k whose inverse M-point DFT
+// is the packed real row z_m = x_{2m} + i x_{2m+1}, x_j = sum_{k=0}^{N-1} X_k exp(2 pi i jk/N).
+template <typename T, class X>
+__device__ __forceinline__ cpx<T> c2r_pre(X x, int M, const cpx<T>* __restrict__ tw, int k) {
+  const int km = k ? M - k : 0;
+  const bool low = k < km;
+  const cpx<T> Xk = x(k), Xm = x(km);
+  const cpx<T> A = Xk + conjg(Xm), B = Xk - conjg(Xm);
+  cpx<T> w = ldg(&tw[low ? k : km]);
+  if (low) w.y = -w.y;  // e^{+2 pi i k / N}; above M/2 it is -e^{-2 pi i (M-k)/N}
+  const cpx<T> z = A + mul_si(w * B, low ? T(1) : T(-1));
+  return k ? z : mk<T>(Xk.x, Xk.x);
 }
 
-// Z_k (forward M-point DFT of the packed real row) -> X_k = sum_j x_j e^{-2 pi i jk/N}, k < M
+// Z_k (row: forward M-point DFT of the packed real row) -> X_k = sum_j x_j e^{-2 pi i jk/N}, k < M:
+// out[k] and out[M - k]
 template <typename T>
-__device__ __forceinline__ void r2c_post(cpx<T>* row, int M, const cpx<T>* __restrict__ tw,
+__device__ __forceinline__ void r2c_post(cpx<T>* out, const cpx<T>* row, int M, const cpx<T>* __restrict__ tw,
                                          int k) {
   if (k == 0) {
     const cpx<T> Z = row[0];
-    row[0] = mk<T>(Z.x + Z.y, T(0));
+    out[0] = mk<T>(Z.x + Z.y, T(0));
     if (M % 2 == 0 && M > 1) {
       // k = M/2: W^k = e^{-i pi/2} = -i
       cpx<T> Zk = row[M / 2];
       cpx<T> A = Zk + conjg(Zk), B = Zk - conjg(Zk);
       // X = A/2 - i/2 (-i) B = A/2 - B/2
-      row[M / 2] = T(0.5) * (A - B);
+      out[M / 2] = T(0.5) * (A - B);
     }
     return;
   }
@@ -542,16 +505,18 @@ __device__ __forceinline__ void r2c_post(cpx<T>* row, int M, const cpx<T>* __res
   cpx<T> Zk = row[k], Zm = row[km];
   cpx<T> W = ldg(&tw[k]);  // e^{-2 pi i k/N}
   cpx<T> A = Zk + conjg(Zm), B = Zk - conjg(Zm);
-  row[k] = T(0.5) * (A - mul_si(W * B, T(1)));
+  out[k] = T(0.5) * (A - mul_si(W * B, T(1)));
   // W^{M-k} = -conj(W)
   cpx<T> A2 = Zm + conjg(Zk), B2 = Zm - conjg(Zk);
-  row[km] = T(0.5) * (A2 + mul_si(conjg(W) * B2, T(1)));
+  out[km] = T(0.5) * (A2 + mul_si(conjg(W) * B2, T(1)));
 }
 
 // x rows: c2r of 6 fields, u x omega, r2c of 3 fields (nonlinear mode); c2r of 3 fields to
-// physical rows (C2R); r2c of 3 physical rows (R2C).  grid ceil(G*N / RX)
+// physical rows (C2R); r2c of 3 physical rows (R2C).  grid ceil(G*N / RX).  The block's threads form
+// six groups that each transform the rows of one field at a time, so that the fields share the
+// barriers of a stage; first stages read global memory (with c2r_pre's combination).
 template <typename T>
-__global__ void __launch_bounds__(512) k_xrow(SlabArgs<T> a) {
+__global__ void __launch_bounds__(384, sizeof(T) == 4 ? 2 : 1) k_xrow(const __grid_constant__ SlabArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* buf = reinterpret_cast<cpx<T>*>(smem_raw);
   const int N = a.N, M = a.M, RX = a.RX;
@@ -562,48 +527,45 @@ __global__ void __launch_bounds__(512) k_xrow(SlabArgs<T> a) {
   const int tile = RX * M;
   const size_t sstride = (size_t)a.G * N * M;
   const int nin = xmode_cross(a.xmode) ? 6 : 3;
-  const size_t plane = (size_t)N * N;
-
-  // load
-  for (int f = 0; f < nin; ++f) {
-    for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
-      const int r = e / M, k = e - r * M;
-      if (a.xmode == XMODE_R2C) {
-        const int rr = r0 + r, zg = rr / N, y = rr - zg * N;
-        const T* src = a.rio + (size_t)f * plane * N + ((size_t)(a.z0 + zg) * N + y) * N;
-        buf[f * tile + e] = mk<T>(src[2 * k], src[2 * k + 1]);
-      } else {
-        buf[f * tile + e] = a.scr[f * sstride + (size_t)(r0 + r) * M + k];
-      }
-    }
-  }
-  // zero unused rows so the FFT batch is well defined
-  for (int f = 0; f < nin; ++f)
-    for (int e = nr * M + threadIdx.x; e < tile; e += blockDim.x) buf[f * tile + e] = mk<T>(0, 0);
-  __syncthreads();
+  constexpr int XG = 6;
+  const int gt = blockDim.x / XG;  // threads of a group
+  const int grp = threadIdx.x / gt, t0 = threadIdx.x - grp * gt;
+  auto real_row = [&](int f, int r) {
+    const int rr = r0 + r, zg = rr / N, y = rr - zg * N;
+    return a.rio + ((size_t)f * N + a.z0 + zg) * N * N + (size_t)y * N;
+  };
+  // the group's field when nf fields are transformed, and its rows from l0 on (a field's rows are shared
+  // by two groups when the groups are twice the fields); nl = 0: nothing to do, but the barriers of it
+  auto batch = [&](int nf, int& f, int& l0) {
+    const bool halves = XG == 2 * nf && RX % 2 == 0;
+    f = grp % nf;
+    l0 = halves && grp >= nf ? RX / 2 : 0;
+    const int nl = halves ? RX / 2 : grp < nf ? RX : 0;
+    return LineBatch{nl, 1, 1, M, t0, gt, false, FastDiv{1, 0}};
+  };
 
   if (a.xmode != XMODE_R2C) {
-    const int npair = M / 2 + 1;
-    for (int e = threadIdx.x; e < nin * RX * npair; e += blockDim.x) {
-      const int fr = e / npair, k = e - fr * npair;
-      if (k == 0 || k < M - k) c2r_pre(buf + fr * M, M, a.tw, k);
-    }
+    int f, l0;
+    const LineBatch lb = batch(nin, f, l0);
+    const cpx<T>* src = a.scr + f * sstride + (size_t)(r0 + l0) * M;
+    cpx<T>* fb = buf + f * tile + l0 * M;
+    const bool phys = a.xmode == XMODE_C2R;
+    fft_lines(fb, a.px, lb, false, a.tw, T(1), a.err,
+              [&](int l, int k) {
+                if (l0 + l >= nr) return mk<T>(0, 0);
+                return c2r_pre<T>([&](int i) { return src[(size_t)l * M + i]; }, M, a.tw, k);
+              },
+              [&](int l, int k, cpx<T> v) {
+                if (!phys) {
+                  fb[l * M + k] = v;
+                } else if (l0 + l < nr) {
+                  T* dst = real_row(f, l0 + l);
+                  dst[2 * k] = v.x;
+                  dst[2 * k + 1] = v.y;
+                }
+              });
+    if (phys) return;
     __syncthreads();
-    for (int f = 0; f < nin; ++f) fft_lines(buf + f * tile, a.px, RX, 1, M, false, a.tw, T(1), a.err);
-  }
-
-  if (a.xmode == XMODE_C2R) {
-    for (int f = 0; f < 3; ++f) {
-      for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
-        const int r = e / M, k = e - r * M;
-        const int rr = r0 + r, zg = rr / N, y = rr - zg * N;
-        T* dst = a.rio + (size_t)f * plane * N + ((size_t)(a.z0 + zg) * N + y) * N;
-        cpx<T> v = buf[f * tile + e];
-        dst[2 * k] = v.x;
-        dst[2 * k + 1] = v.y;
-      }
-    }
-    return;
   }
 
   if (xmode_cross(a.xmode)) {
@@ -617,9 +579,9 @@ __global__ void __launch_bounds__(512) k_xrow(SlabArgs<T> a) {
       m0 = fmax(m0, fabs(u0));
       m1 = fmax(m1, fabs(u1));
       m2 = fmax(m2, fabs(u2));
-      re[e] = u1 * w2 - u2 * w1;
-      re[rt + e] = u2 * w0 - u0 * w2;
-      re[2 * rt + e] = u0 * w1 - u1 * w0;
+      re[e] = fma1(u1, w2, -(u2 * w1));
+      re[rt + e] = fma1(u2, w0, -(u0 * w2));
+      re[2 * rt + e] = fma1(u0, w1, -(u1 * w0));
     }
     __syncthreads();
     // CFL: max |u_i| of the rows (omega, fields 3..5, is no longer needed: scratch)
@@ -627,19 +589,25 @@ __global__ void __launch_bounds__(512) k_xrow(SlabArgs<T> a) {
   }
 
   // forward r2c of fields 0..2
-  for (int f = 0; f < 3; ++f) fft_lines(buf + f * tile, a.px, RX, 1, M, false, a.tw, T(-1), a.err);
   {
-    const int npair = M / 2 + 1;
-    for (int e = threadIdx.x; e < 3 * RX * npair; e += blockDim.x) {
-      const int fr = e / npair, k = e - fr * npair;
-      if (k == 0 || k < M - k) r2c_post(buf + fr * M, M, a.tw, k);
-    }
+    int f, l0;
+    const LineBatch lb = batch(3, f, l0);
+    cpx<T>* fb = buf + f * tile + l0 * M;
+    fft_lines(fb, a.px, lb, a.xmode != XMODE_R2C, a.tw, T(-1), a.err,
+              [&](int l, int k) {
+                if (l0 + l >= nr) return mk<T>(0, 0);
+                const T* src = real_row(f, l0 + l);
+                return mk<T>(src[2 * k], src[2 * k + 1]);
+              },
+              [&](int l, int k, cpx<T> v) { fb[l * M + k] = v; });
   }
   __syncthreads();
+  const int npair = a.dNP.d;
   for (int f = 0; f < 3; ++f) {
-    for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
-      const int r = e / M, k = e - r * M;
-      a.scr[f * sstride + (size_t)(r0 + r) * M + k] = buf[f * tile + e];
+    cpx<T>* dst = a.scr + f * sstride + (size_t)r0 * M;
+    for (int e = threadIdx.x; e < nr * npair; e += blockDim.x) {
+      const int r = fdiv(e, a.dNP), k = e - r * npair;
+      if (k == 0 || k < M - k) r2c_post(dst + (size_t)r * M, buf + f * tile + r * M, M, a.tw, k);
     }
   }
 }
