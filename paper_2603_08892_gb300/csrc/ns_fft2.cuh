@@ -285,52 +285,6 @@ __device__ __forceinline__ void cstage(const Src& src, const Dst& dst, const cpx
   }
 }
 
-template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, int S, int NS,
-          bool HOLD0 = false, int MR = NS_MAX_RADIX>
-struct CStages {
-  static constexpr CPlan P = cplan(n, MR);
-  template <class Src, class Dst>
-  static __device__ __forceinline__ void run(const Src& src, const Dst& dst, cpx<T>* work,
-                                             const cpx<T>* __restrict__ tw) {
-    constexpr int R = P.r[S];
-    constexpr bool first = S == 0;
-    constexpr bool last = S == P.nst - 1;
-    const WorkTile<T, n, NL, LF> W{work};
-    if constexpr (first && last) {
-      cstage<T, n, R, NS, TWS, NL, NT, LF, DIR, true>(src, dst, tw);
-    } else if constexpr (first) {
-      cstage<T, n, R, NS, TWS, NL, NT, LF, DIR, HOLD0>(src, W, tw);
-      __syncthreads();
-      CStages<T, n, TWS, NL, NT, LF, DIR, S + 1, NS * R, false, MR>::run(src, dst, work, tw);
-    } else if constexpr (last) {
-      cstage<T, n, R, NS, TWS, NL, NT, LF, DIR, false>(W, dst, tw);
-    } else {
-      cstage<T, n, R, NS, TWS, NL, NT, LF, DIR, true>(W, W, tw);
-      __syncthreads();
-      CStages<T, n, TWS, NL, NT, LF, DIR, S + 1, NS * R, false, MR>::run(src, dst, work, tw);
-    }
-  }
-};
-
-// Transform of NL lines of length n: src -> dst through the shared work tile `work`
-// (WorkTile<T, n, NL, LF>::elems() values).  DIR = -1 forward, +1 inverse.  TWS = table
-// length / n.  The caller places a barrier after it before dst is read by other threads.
-template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, int MR = NS_MAX_RADIX,
-          class Src, class Dst>
-__device__ __forceinline__ void cfft(const Src& src, const Dst& dst, cpx<T>* work,
-                                     const cpx<T>* __restrict__ tw) {
-  CStages<T, n, TWS, NL, NT, LF, DIR, 0, 1, false, MR>::run(src, dst, work, tw);
-}
-
-// Same, for a source that reads the work tile itself: stage 0 reads every input before it
-// writes the work tile.
-template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, int MR = NS_MAX_RADIX,
-          class Src, class Dst>
-__device__ __forceinline__ void cfft_src_in_work(const Src& src, const Dst& dst, cpx<T>* work,
-                                                 const cpx<T>* __restrict__ tw) {
-  CStages<T, n, TWS, NL, NT, LF, DIR, 0, 1, true, MR>::run(src, dst, work, tw);
-}
-
 // In place: stage 0 reads src (ALIAS: src is the tile itself) and writes the tile B; every
 // later stage runs in place on B with its inputs held in registers across a barrier.  The
 // last stage writes through dst (an accessor over the same tile, e.g. applying a pointwise
@@ -359,21 +313,6 @@ struct CStagesIP {
   }
 };
 
-template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, bool ALIAS,
-          int MR = NS_MAX_RADIX, class Src>
-__device__ __forceinline__ void cfft_ip(const Src& src, cpx<T>* tile, const cpx<T>* __restrict__ tw) {
-  const WorkTile<T, n, NL, LF> B{tile};
-  CStagesIP<T, n, TWS, NL, NT, LF, DIR, ALIAS, 0, 1, MR>::run(src, B, B, tw);
-}
-
-// Same, the last stage writing through dst (which must address the same tile)
-template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, bool ALIAS,
-          int MR = NS_MAX_RADIX, class Src, class Dst>
-__device__ __forceinline__ void cfft_ip_to(const Src& src, cpx<T>* tile, const Dst& dst,
-                                           const cpx<T>* __restrict__ tw) {
-  CStagesIP<T, n, TWS, NL, NT, LF, DIR, ALIAS, 0, 1, MR>::run(src, WorkTile<T, n, NL, LF>{tile}, dst, tw);
-}
-
 // In-place transform of NL lines over any tile accessor B (get / put of (line, e)); the last
 // stage writes through dst.  tid as in cstage.
 template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, bool ALIAS,
@@ -381,13 +320,6 @@ template <typename T, int n, int TWS, int NL, int NT, bool LF, int DIR, bool ALI
 __device__ __forceinline__ void cfft_ip_tid(const Src& src, const Tile& B, const Dst& dst,
                                             const cpx<T>* __restrict__ tw, int tid) {
   CStagesIP<T, n, TWS, NL, NT, LF, DIR, ALIAS, 0, 1, MR>::run(src, B, dst, tw, tid);
-}
-
-// copy of the twiddle table into shared memory (all threads of the block participate)
-template <typename T>
-__device__ __forceinline__ void load_twiddles(cpx<T>* dst, const cpx<T>* __restrict__ tw, int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[tw_pad(i)] = ldg(&tw[i]);
-  __syncthreads();
 }
 
 }  // namespace ns

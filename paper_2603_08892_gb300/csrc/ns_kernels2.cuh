@@ -23,7 +23,6 @@ __host__ __device__ constexpr int pick_div(int m, int target, int cap) {
     if (m % d == 0) return d;
   return 1;
 }
-__host__ __device__ constexpr int round_warps(int t) { return cmin(cmax((t + 31) / 32 * 32, 64), 512); }
 __host__ __device__ constexpr int cgcd(int a, int b) { return b == 0 ? a : cgcd(b, a % b); }
 // thread count: >= t, >= 64, a multiple of the warp size and of w (each thread keeps one line)
 __host__ __device__ constexpr int round_lines(int t, int w) {
@@ -99,37 +98,6 @@ struct MemCG {
     st(&p->b, b);
   }
 };
-
-// Asynchronous 16-byte global -> shared copies (cp.async.cg: through L2 only, so data written
-// by other blocks of a persistent launch is never read from a stale L1 line).
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\ncp.async.wait_all;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// wait until at most P of this thread's committed groups are still in flight
-template <int P>
-__device__ __forceinline__ void cp_async_wait_pending() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(P) : "memory");
-}
-// Stage a column tile [e][line] (W lines, n elements) of a [z|kz][ky][kx] field from global
-// memory; W * sizeof(cpx<T>) is a multiple of 16 bytes and x0 a multiple of W.
-// PLANE: the tile of a fixed plane p of a [p][e][kx] field (element e = ky or y) instead.
-template <typename T, int N, int W, int NT, bool PLANE = false>
-__device__ __forceinline__ void stage_col_tile(cpx<T>* dst, const cpx<T>* src, int iy, int x0) {
-  constexpr int PER = 16 / (int)sizeof(cpx<T>);  // complex values per 16-byte chunk
-  constexpr int CH = W / PER;                     // chunks per row
-  static_assert(W % PER == 0, "tile rows must be whole 16-byte chunks");
-  if (threadIdx.x >= NT) return;
-  for (int i = threadIdx.x; i < N * CH; i += NT) {
-    const int e = i / CH, xc = (i % CH) * PER;
-    const size_t row = PLANE ? (size_t)iy * N + e : (size_t)e * N + iy;
-    cp_async16(&dst[lf_idx<T, W>(e, xc)], &src[row * (N / 2) + x0 + xc]);
-  }
-}
 
 // The alternative width of a tile (lines per tile): twice the default where that divides
 // the half length m within the cap, else half (down to minw), else the default.
