@@ -113,7 +113,9 @@ struct GenericShapes {
   size_t smX;         // x-row shared memory (6 fields)
 };
 // Columns: up to 16, fewer until two pencil blocks (three y blocks) fit an SM, but not below 64
-// bytes a row for that.  Rows: as many as groups of 64 threads hold (N <= 1024: at least one).
+// bytes a row for that.  Rows: an even number that groups of 32 threads hold up to
+// N = 128, of 64 above (N <= 1024: at least one).  Measured, 32 and 64 threads: 72^3 FP64 step 634
+// and 665 us, 216^3 FP32 step 3337 and 3237.
 GenericShapes generic_shapes(int N, size_t cs) {
   const int M = N / 2;
   GenericShapes g;
@@ -128,9 +130,10 @@ GenericShapes generic_shapes(int N, size_t cs) {
   g.LY = largest_divisor_le(g.TY, 384 * 8 / N);
   g.bdY = fft_block(g.LY * N);
   g.smY = (size_t)N * g.TY * cs;
-  g.RX = 16;
-  while (g.RX > 1 && g.RX * M > 64 * 8) g.RX /= 2;
-  g.bdX = 6 * (g.RX * M <= 32 * 8 ? 32 : 64);
+  const int gt = M <= 64 ? 32 : 64;
+  g.RX = gt * 8 / M;
+  g.RX = g.RX > 16 ? 16 : g.RX < 2 ? 1 : g.RX / 2 * 2;
+  g.bdX = 6 * gt;
   g.smX = 6 * (size_t)g.RX * M * cs;
   return g;
 }
