@@ -558,6 +558,7 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
   // 2) spectral stage: every mode's N(0) = 0, truncation, projection and forcing, then the RK
   //    stage combine; v becomes S_next, shifted for the output when there is one
   const bool pre = nOut == 1 && a.osh[0] != nullptr;
+  const bool ep = EP || (NOC == 2 && a.epart != nullptr);  // the same for the whole block
   T eacc = 0, dacc = 0;  // energy sums of the written state
   bool nz = false;
   if (act) {
@@ -600,24 +601,25 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
           const cpx<T> s1 = rd1 ? MP::ldw(&a.acc[c * fstride + g]) : mk<T>(0, 0);
           cpx<T> sn = stage_combine<T, MP>(a, c, c * fstride + g, nv[c], s0[c][i], s1, E1, Eh, mode);
           shell_record<T, MP>(a, c, kx, ky, kz, sn);
-          if (EP || NOC == 2) m2 += sn.x * sn.x + sn.y * sn.y;
+          if (ep) m2 += sn.x * sn.x + sn.y * sn.y;
           nz = nz || sn.x != T(0) || sn.y != T(0);
           v[c][r] = pre ? cmul_fixed(sn, shz) : sn;
         }
-        if (EP || NOC == 2) {
+        if (ep) {
           const T wm = (kx == 0 ? T(1) : T(2)) * m2;
           if constexpr (ED == NB0) {
             eacc += wm;
             dacc += wm * (T)(kx * kx + ky * ky + kz * kz);
           } else {
-            reinterpret_cast<T*>(buf)[iz * TX + line] = wm;  // (the tiles are free here)
+            // the tiles are free here, until the barriers that follow the sums
+            reinterpret_cast<T*>(buf)[iz * TX + line] = wm;
           }
         }
       }
     }
   }
   if constexpr (EP || NOC == 2) {
-    if (EP || a.epart) {
+    if (ep) {
       if constexpr (ED != NB0) {
         __syncthreads();
         for (int i = tid; i < TX * ED; i += blockDim.x) {
