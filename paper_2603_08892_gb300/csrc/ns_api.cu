@@ -304,10 +304,12 @@ struct Solver : SolverBase {
   // skips its INIT pass.  -1 whenever anything else wrote the state, the mixed fields or the
   // forcing record.
   int64_t carry_step = -1;
-  // the mixed fields, the state or the forcing record change other than by a step
-  void touched() {
+  // the mixed fields or the forcing record change other than by a step
+  void fields_changed() { carry_step = -1; }
+  // so does the state
+  void state_changed() {
     carry_step = -1;
-    cut_known = false;
+    cut_cur = nullptr;
   }
   // adaptive time step (ns_step_cfl): dt = min(dt_max, cfl dx / sum_i max|u_i|) per step
   double cfl = 0.0, cfl_dtmax = 0.0;
@@ -482,8 +484,9 @@ struct Solver : SolverBase {
     red_blocks = 2 * nsm;
     CUDA_TRY(cudaMalloc(&red, (size_t)red_blocks * 1024 * sizeof(double)));
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
-    CUDA_TRY(cudaMalloc(&d_cut, 3 * sizeof(int)));
-    const int one[3] = {0, 0, 1};
+    decide_cut();
+    CUDA_TRY(cudaMalloc(&d_cut, 4 * sizeof(int)));
+    const int one[4] = {1, 1, 1, 1};
     CUDA_TRY(cudaMemcpyAsync(d_cut, one, sizeof(one), cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMalloc(&d_umax, 3 * sizeof(unsigned long long)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), st));
@@ -523,7 +526,7 @@ struct Solver : SolverBase {
   }
 
   void buffers(double dt, NsCtxBuffers* b) override {
-    touched();
+    state_changed();
     if (dt > 0) set_dt(dt);
     b->N = N; b->precision = c->p.precision; b->scheme = c->p.scheme; b->truncation = c->p.truncation;
     b->K2max = c->K2max; b->Kimax = c->Kimax; b->G = Gmax; b->nu = c->p.nu; b->kmax = c->p.kmax;
@@ -559,27 +562,50 @@ struct Solver : SolverBase {
   }
 
   // ---- passes -----------------------------------------------------------------------
-  // Truncated states.  d_cut[0]: the state vanishes outside the kept columns (column_kept);
-  // d_cut[1]: the same of the state from which the carried mixed fields were formed; d_cut[2] = 1.
-  // Steps keep the property, so the state is looked at when something else may have written it:
-  // before the first step after that, and, once its device address was handed out
-  // (ns_device_state), before the first step of every call.
+  // Truncated states.  A flag is a device word, not 0 when the state vanishes outside the kept
+  // columns (column_kept): cut_cur that of the state (null: not known), cut_mix that of the state
+  // from which the carried mixed fields were formed.  After a projection it is the constant
+  // d_cut[3]; a state that something else may have written is looked at (k_cut_check, into the next
+  // of the words d_cut[0 .. 2]) before the first step after that and, once its device address was
+  // handed out (ns_device_state), before the first step of every call.  Steps keep the property.
   int* d_cut = nullptr;
-  bool cut_known = false, state_shared = false;
+  int cut_slot = 0;
+  const int *cut_cur = nullptr, *cut_mix = nullptr;
+  bool state_shared = false;
   int box() const { return fkind != NS_FORCE_NONE ? fK : -1; }
   int kx_end() const {  // first kx none of whose columns is kept
     int k = 0;
     while (k < M && column_kept(c->p.truncation, c->K2max, c->Kimax, box(), k, 0)) ++k;
     return k;
   }
-  void cut_check() {
-    if (cut_known && !state_shared) return;
-    k_cut_begin<<<1, 1, 0, st>>>(d_cut);
-    k_cut_check<T><<<dim3(N, N < 256 ? 2 : 8), 256, 0, st>>>(state, N, c->p.truncation, c->K2max, c->Kimax, box(), d_cut);
-    LAUNCH_CHECK();
-    cut_known = true;
+  // Whether columns are left out at all (with the launch that looks at the state, where needed): from
+  // 20 MB of state on when a quarter of the columns goes, from 40 MB on always.  Below, the fields stay
+  // in L2 and the launches are short.  Measured, steps with all columns and without, us: FP32 96^3
+  // (11 MB) 397 and 401 at C_t = 1, 380 and 381 at 2/3; 128^3 (25 MB) 619 and 625 at 1, 592 and 573 at
+  // 0.8, 590 and 470 at 2/3; 192^3 (85 MB) 2200 and 2110 at 1; FP64 96^3 (21 MB) 6179 and 6190 at 1,
+  // 5381 and 5091 at 2/3; 128^3 (50 MB) 10467 and 10310 at 1.
+  bool cut_pays = false;
+  void decide_cut() {
+    const size_t bytes = 3 * F1 * sizeof(cpx<T>);
+    size_t kept = 0;
+    for (int iy = 0; iy < N; ++iy)
+      for (int k = 0; k < M && column_kept(c->p.truncation, c->K2max, c->Kimax, -1, k, iy < M ? iy : iy - N); ++k) ++kept;
+    cut_pays = use2 && (bytes >= 40000000 || (bytes >= 20000000 && 4 * kept <= 3 * (size_t)N * M));
   }
-  const int* cut_flag(int i) const { return use2 && !clus ? d_cut + i : nullptr; }
+  bool cut_on() const { return cut_pays && !clus; }
+  void cut_check() {
+    cut_mix = cut_cur;
+    if (!cut_on() || (cut_cur && !state_shared)) return;
+    int* flag = d_cut + cut_slot;
+    cut_slot = (cut_slot + 1) % 3;
+    k_cut_check<T><<<dim3(N, (3 * N + 63) / 64), 256, 0, st>>>(state, N, c->p.truncation, c->K2max, c->Kimax, box(), flag,
+                                                             d_cut + cut_slot);
+    LAUNCH_CHECK();
+    cut_cur = flag;
+  }
+  const int* cut_flag(const int* f) const { return cut_on() ? f : nullptr; }
+  const int* cut_state() const { return cut_flag(cut_cur); }
+  const int* cut_clean() const { return cut_flag(d_cut + 3); }  // of a state that was projected
 
   // layout of the mixed fields and of Ft (mixed_index): interleaved for the compile-time kernels,
   // except when the cluster slab pass, whose TMA copies take one field at a time, reads them
@@ -816,7 +842,7 @@ struct Solver : SolverBase {
   // block [lo, hi) of the z (or kz) axis (axis 0) or the ky axis (axis 1) of buffer `which`
   // between the device and host FP64 (re, im): axis 0 [F][hi-lo][N][M], axis 1 [F][N][hi-lo][M]
   void rank_copy(int which, int axis, int lo, int hi, bool to_dev, double* host) override {
-    touched();
+    state_changed();
     const int F = rank_fields(which), n = hi - lo;
     const size_t cs = sizeof(cpx<T>);
     if (!rank_stg) CUDA_TRY(cudaMalloc(&rank_stg, 5 * F1 * cs));
@@ -836,7 +862,7 @@ struct Solver : SolverBase {
   // pencil pass on the ky rows [lo, hi): NS_RANK_INIT: state -> mixed (shifted by delta);
   // NS_RANK_NL: Ft -> the shifted, de-shifted, truncated, projected nonlinear term (NL buffer)
   void rank_pencil(int kind, const double* delta, int lo, int hi) override {
-    touched();
+    fields_changed();
     std::vector<double> sh(delta, delta + 3);
     upload_shifts(sh);
     PencilArgs<T> p = pencil_args(kind == NS_RANK_INIT ? MODE_INIT : MODE_NL);
@@ -855,7 +881,7 @@ struct Solver : SolverBase {
   }
   // slab pass on the planes [lo, hi): mixed -> Ft (the three slab kernels, plane groups of G)
   void rank_slab(int lo, int hi) override {
-    touched();
+    fields_changed();
     SlabArgs<T> a = slab_args();
     a.mixed = mixed[0];
     a.Ft = Ft[0];
@@ -1041,7 +1067,7 @@ struct Solver : SolverBase {
 
   void set_forcing(int kind, double kfmin, double kfmax, double eps, double tcorr,
                    uint64_t seed) override {
-    touched();
+    state_changed();
     tape.valid = false;  // a recorded adjoint run used the previous forcing
     fkind = kind;
     if (kind == NS_FORCE_NONE) return;
@@ -1155,7 +1181,7 @@ struct Solver : SolverBase {
     }
   }
   void autotune() {
-    touched();
+    fields_changed();
     tuned = true;
     if (const char* e = std::getenv("NS_PIPE_SPIN")) pipe_spin = std::max(1ll, std::atoll(e));
     if (const char* e = std::getenv("NS_PIPE_TEST_STALL")) pipe_stall = std::atoi(e) ? 1 : 0;
@@ -1300,7 +1326,7 @@ struct Solver : SolverBase {
   }
 
   // ---- schemes ------------------------------------------------------------------------
-  void invalidate_carry() override { touched(); }
+  void invalidate_carry() override { fields_changed(); }
 
   void step_cfl(double cfl_, double dt_max, int nsteps) override {
     cfl = cfl_;
@@ -1363,7 +1389,7 @@ struct Solver : SolverBase {
   void init_pass(int nOut, const cpx<T>* o0, const cpx<T>* o1) {
     PencilArgs<T> a = pencil_args(MODE_INIT);
     a.src = state;
-    a.cut = cut_flag(0);
+    a.cut = cut_state();
     a.nOut = nOut;
     a.osh[0] = o0; a.out[0] = mixed[0];
     a.osh[1] = o1; a.out[1] = mixed[1];
@@ -1390,11 +1416,9 @@ struct Solver : SolverBase {
     return d;
   }
 
-  // flag of the mixed fields that a chunk's first slab pass reads: carried from an earlier call of a
-  // shared state, the one of the state they were formed from; formed now, the state's
-  const int* first_cut() const {
-    return cut_flag(carry_step == c->step && chunk0 && state_shared ? 1 : 0);
-  }
+  // flag of the mixed fields that a chunk's first slab pass reads: carried from an earlier call, the
+  // one of the state they were formed from; formed now, the state's
+  const int* first_cut() const { return cut_flag(carry_step == c->step && chunk0 ? cut_mix : cut_cur); }
   bool chunk0 = false;  // the first chunk of a call
   void run_rogallo(double dt0, int ns, bool approx) {
     const T w = (T)(1.0 / ((double)N * N * N));
@@ -1404,17 +1428,17 @@ struct Solver : SolverBase {
     if (carry_step != c->step) init_pass(1, alpha(0), nullptr);
     for (int n = 0; n < ns; ++n) {
       const double t = c->t;
-      slab(mixed[0], Ft[0], cfl > 0.0, n == 0 ? cin : cut_flag(0));
+      slab(mixed[0], Ft[0], cfl > 0.0, n == 0 ? cin : cut_state());
       const double dt = step_dt(dt0);
       PencilArgs<T> a = pencil_args(MODE_ROG_1);
       force_coef(t, a);
       a.nF = 1; a.F[0] = Ft[0]; a.dsh[0] = alpha(n); a.wF[0] = w;
       a.nOut = 1; a.osh[0] = beta(n); a.out[0] = mixed[0];
-      a.cut = cut_flag(0);
+      a.cut = cut_state();
       pencil(a);
-      slab(mixed[0], Ft[0], false, cut_flag(0));
+      slab(mixed[0], Ft[0], false, cut_state());
       PencilArgs<T> b = pencil_args(MODE_ROG_2);
-      b.cut = cut_flag(0);
+      b.cut = cut_state();
       force_coef(t + dt, b);
       b.nF = 1; b.F[0] = Ft[0]; b.dsh[0] = beta(n); b.wF[0] = w;
       b.nOut = 1;  // the last step of the chunk prepares the step after it
@@ -1436,12 +1460,12 @@ struct Solver : SolverBase {
       const double t = c->t;
       double dt = dt0;
       for (int stg = 0; stg < 2; ++stg) {
-        const int* cut = n == 0 && stg == 0 ? cin : cut_flag(0);
+        const int* cut = n == 0 && stg == 0 ? cin : cut_state();
         slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0, cut);
         if (stg == 0) dt = step_dt(dt0);
         if (exact) slab(mixed[1], Ft[1], false, cut);
         PencilArgs<T> a = pencil_args(stg == 0 ? MODE_RK2_1 : MODE_RK2_2);
-        a.cut = cut_flag(0);
+        a.cut = cut_state();
         force_coef(stg == 0 ? t : t + 0.5 * dt, a);
         a.nF = exact ? 2 : 1;
         a.F[0] = Ft[0]; a.dsh[0] = nullptr; a.wF[0] = exact ? (T)0.5 * w : w;
@@ -1470,10 +1494,10 @@ struct Solver : SolverBase {
       const double t = c->t;
       double dt = dt0;
       for (int stg = 0; stg < 4; ++stg) {
-        slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0, n == 0 && stg == 0 ? cin : cut_flag(0));
+        slab(mixed[0], Ft[0], stg == 0 && cfl > 0.0, n == 0 && stg == 0 ? cin : cut_state());
         if (stg == 0) dt = step_dt(dt0);
         PencilArgs<T> a = pencil_args(modes[stg]);
-        a.cut = cut_flag(0);
+        a.cut = cut_state();
         force_coef(t + ts[stg] * dt, a);
         a.nF = 1; a.F[0] = Ft[0]; a.wF[0] = w;
         a.nOut = 1;  // the last pass prepares the next step
@@ -1583,10 +1607,11 @@ struct Solver : SolverBase {
   }
 
   void set_velocity(const double* u) override {
-    touched();
+    state_changed();
     T* rin = reinterpret_cast<T*>(mixed[0]);  // 5 N^3 reals >= 3 N^3
     to_device(u, rin, 3 * (size_t)N * N * N);
     r2c_project(rin, state, 1.0 / ((double)N * N * N));
+    cut_cur = d_cut + 3;
     sync_check();
   }
 
@@ -1594,7 +1619,7 @@ struct Solver : SolverBase {
 
   // spectral [3][N][N][M] -> physical host [3][N][N][N] (inverse z, y, x transforms)
   void to_physical(const cpx<T>* src, double* u) {
-    touched();
+    fields_changed();
     T* rout = reinterpret_cast<T*>(Ft[0]);  // 3 N^3 reals
     c2r(src, rout);
     to_host(rout, u, 3 * (size_t)N * N * N);
@@ -1619,7 +1644,7 @@ struct Solver : SolverBase {
     sync_check();
   }
   void set_raw_state(const unsigned char* in, size_t n) override {
-    touched();
+    state_changed();
     if (n != 3 * F1 * sizeof(cpx<T>)) throw NsError{NS_ERR_IO, "checkpoint state size mismatch"};
     CUDA_TRY(cudaMemcpyAsync(state, in, n, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -1630,12 +1655,12 @@ struct Solver : SolverBase {
     *seed = fseed;
   }
   void set_state(const double* s) override {
-    touched();
+    state_changed();
     upload(s, state);
   }
 
   void nonlinear(const double* in, const double* delta, double* out) override {
-    touched();
+    fields_changed();
     const cpx<T>* src = state;
     if (in) {
       upload(in, acc);
@@ -1815,16 +1840,16 @@ struct Solver : SolverBase {
     cpx<T>* N0 = vec(0);
     cpx<T>* N1 = vec(1);
     cpx<T>* S1 = vec(2);
-    nl_eval(S0, shift_tab(2 * n), N0, cut_flag(2));
+    nl_eval(S0, shift_tab(2 * n), N0, cut_clean());
     add_forcing(S0, times[n], N0);
     ew(EW_ROG_S1, S0, N0, nullptr, S1);
-    nl_eval(S1, shift_tab(2 * n + 1), N1, cut_flag(2));
+    nl_eval(S1, shift_tab(2 * n + 1), N1, cut_clean());
     add_forcing(S1, times[n] + dt, N1);
     ew(EW_ROG_SN, S0, N0, N1, Sout);
   }
   // forward sweep from `state` with the state kept every ckpt steps; leaves state = S_T
   void adj_forward(int nsteps, double dt, int ckpt) {
-    touched();
+    state_changed();
     adj_alloc(nsteps, ckpt);
     const std::vector<double> times = adj_tables(nsteps, dt);
     const size_t vb = 3 * F1 * sizeof(cpx<T>);
@@ -1873,7 +1898,7 @@ struct Solver : SolverBase {
         const cpx<T>* S0 = seg[n - seg0];
         const cpx<T>* ta = shift_tab(2 * n);
         const cpx<T>* tb = shift_tab(2 * n + 1);
-        nl_eval(S0, ta, N0, cut_flag(2));
+        nl_eval(S0, ta, N0, cut_clean());
         add_forcing(S0, times[n], N0);
         ew(EW_ROG_S1, S0, N0, nullptr, S1);
         ew(EW_RHO, lam, nullptr, nullptr, rho);
@@ -1933,7 +1958,7 @@ struct Solver : SolverBase {
 
   // device-buffer forms (the autograd path): u0, uT [3][N][N][N] reals of T on the device
   void tape_forward(const void* u0, int nsteps, double dt, int ckpt, void* uT) override {
-    touched();
+    state_changed();
     r2c_project(static_cast<const T*>(u0), state, 1.0 / ((double)N * N * N));
     adj_forward(nsteps, dt, ckpt);
     c2r(state, static_cast<T*>(uT));
@@ -1942,7 +1967,7 @@ struct Solver : SolverBase {
   // gT: the cotangent of u(T) (device reals of T), or null for the built-in loss `loss`
   void tape_backward(const void* gT, int loss, void* grad) override {
     if (!tape.valid) throw NsError{NS_ERR_STATE, "no adjoint tape: call ns_tape_forward first"};
-    touched();
+    state_changed();
     cpx<T>* lam = vec(3);
     if (gT)
       r2c_project(static_cast<const T*>(gT), lam, 1.0);
@@ -1987,18 +2012,18 @@ struct Solver : SolverBase {
   // Nonlinear energy flux and cumulative dissipation on shell bins (Sec. 3.4)
   cpx<T>* nlbuf = nullptr;
   void energy_flux(const double* delta, int nshift, double* flux, double* cumd, int nbins) override {
-    touched();
+    fields_changed();
     if (flux) {
       if (!nlbuf) CUDA_TRY(cudaMalloc(&nlbuf, 3 * F1 * sizeof(cpx<T>)));
       cut_check();
       if (nshift == 0) {
-        nl_eval(state, nullptr, nlbuf, cut_flag(0));
+        nl_eval(state, nullptr, nlbuf, cut_state());
       } else {
         if (!nltmp && nshift > 1) CUDA_TRY(cudaMalloc(&nltmp, 3 * F1 * sizeof(cpx<T>)));
         for (int sidx = 0; sidx < nshift; ++sidx) {
           std::vector<double> sh(delta + 3 * sidx, delta + 3 * sidx + 3);
           upload_shifts(sh);
-          nl_eval(state, shift_tab(0), sidx == 0 ? nlbuf : nltmp, cut_flag(0));
+          nl_eval(state, shift_tab(0), sidx == 0 ? nlbuf : nltmp, cut_state());
           if (sidx > 0) ew(EW_ADD, nlbuf, nltmp, nullptr, nlbuf);
         }
         if (nshift > 1) ew(EW_SCALE, nlbuf, nullptr, nullptr, nlbuf, 1.0 / nshift);

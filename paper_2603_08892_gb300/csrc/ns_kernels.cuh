@@ -81,41 +81,50 @@ __host__ __device__ __forceinline__ bool column_kept(int trunc, int K2max, int K
   return in || (kx <= box && ay <= box);
 }
 
-// flag[1] = flag[0] and flag[0] = 1, before k_cut_check
-static __global__ void k_cut_begin(int* flag) {
-  flag[1] = flag[0];
-  flag[0] = 1;
-}
-// true when the modes of S [3][N][N][M] in the columns (kx, ky = kof(iy)) that are not kept vanish.
-// One block per ky and part (of `parts`); reads only those modes (21 % of the state at C_t = 1),
-// four loads per thread in flight.
+// true (to some threads at least false otherwise) when the modes of S [3][N][N][M] in the columns
+// (kx, ky = kof(iy)) that are not kept vanish.  One block of 256 threads per ky and part (of
+// `parts`); reads only those modes (21 % of the state at C_t = 1), 16 bytes a load, four in flight.
+// A row is given the next power of two of threads, so that no index needs a division.
 template <typename T>
 __device__ __forceinline__ bool cut_clean(const cpx<T>* S, int N, int trunc, int K2max, int Kimax, int box, int iy,
                                           int part, int parts) {
+  constexpr int PER = 16 / (int)sizeof(cpx<T>);  // modes of a load
   const int M = N / 2, ky = kof(iy, N);
-  int lo = 0, hi = M;  // the first kx that is not kept (the kept ones are an interval from 0)
-  while (lo < hi) {
-    const int m = (lo + hi) / 2;
-    if (column_kept(trunc, K2max, Kimax, box, m, ky)) lo = m + 1;
-    else hi = m;
+  int lo = 0;  // the first kx that is not kept (the kept ones are an interval from 0)
+  for (int k0 = 0; k0 < M; k0 += blockDim.x) {
+    const int k = k0 + threadIdx.x;
+    lo += __syncthreads_count(k < M && column_kept(trunc, K2max, Kimax, box, k, ky));
   }
-  const int len = M - lo, total = 3 * N * len;
+  if (lo == M) return true;
+  const int c0 = lo / PER, nch = M / PER - c0;  // loads of a row
+  const int lw = nch > 1 ? 32 - __clz(nch - 1) : 0, rows = blockDim.x >> lw;
+  const int ch = threadIdx.x & ((1 << lw) - 1), r1 = threadIdx.x >> lw, kx = (c0 + ch) * PER;
   bool nz = false;
-  for (int i0 = part * 4 * blockDim.x + threadIdx.x; i0 < total; i0 += parts * 4 * blockDim.x) {
-    cpx<T> v[4];
+  if (ch < nch)
+    for (int r0 = part * 4 * rows + r1; r0 < 3 * N; r0 += parts * 4 * rows) {
+      cpx<T> v[4][PER];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = i0 + q * blockDim.x, r = i / len;  // r: component and kz
-      v[q] = i < total ? S[((size_t)r * N + iy) * M + lo + (i - r * len)] : mk<T>(0, 0);
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + q * rows;  // component and kz
+#pragma unroll
+        for (int i = 0; i < PER; ++i) v[q][i] = mk<T>(0, 0);
+        if (r < 3 * N) {
+          const float4 w = *reinterpret_cast<const float4*>(&S[((size_t)r * N + iy) * M + kx]);
+          memcpy(v[q], &w, 16);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < PER; ++i) nz = nz || (kx + i >= lo && (!(v[q][i].x == T(0)) || !(v[q][i].y == T(0))));
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) nz = nz || !(v[q].x == T(0)) || !(v[q].y == T(0));
-  }
   return !nz;
 }
+// *flag = 0 (it is 1 before) where they do not; *next = 1, the flag of the next check
 template <typename T>
 __global__ void __launch_bounds__(256) k_cut_check(const cpx<T>* S, int N, int trunc, int K2max, int Kimax, int box,
-                                                   int* flag) {
+                                                   int* flag, int* next) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *next = 1;
   if (!cut_clean(S, N, trunc, K2max, Kimax, box, blockIdx.x, blockIdx.y, gridDim.y)) *flag = 0;
 }
 
