@@ -133,10 +133,14 @@ __host__ __device__ constexpr bool plan_has_radix2(int n, int mr) {
 __host__ __device__ constexpr int slab_radix(int n) {
   return n <= 128 && plan_has_radix2(n, 16) && !plan_has_radix2(n, 8) ? 8 : 16;
 }
-// FP64 at N = 24 and 32: radix 4, as the few columns of those grids must spread over every SM's
-// FP64 pipe.  The x rows of sizes whose FP32 tiles of x_rows rows do not divide the planes (192, 384)
-// have no reproducible pairing of rows to keep and take the plan with the fewest stages.
-__host__ __device__ constexpr bool small64(int n) { return n >= 24 && n <= 32; }
+// FP64 from N = 16 to 96: radix 4.  The FP64 pipes bound these grids, and an SM needs several full
+// warps to keep its share of them busy: radix 4 gives 2 to 3 times the threads of radix 8 and 12 (a y
+// tile of 48^3 has 48 instead of 16).  Steps with radix 4 and with 8 or 12, us: 16^3 133 and 138,
+// 48^3 235 and 325, 64^3 389 and 403, 96^3 1260 and 1540; 128^3 2616 and 2578, 192^3 9740 and 9590.
+// (24 and 32 were set to radix 4 before: 32^3 161 and 268.)
+// The x rows of sizes whose FP32 tiles of x_rows rows do not divide the planes (192, 384) have no
+// reproducible pairing of rows to keep and take the plan with the fewest stages.
+__host__ __device__ constexpr bool small64(int n) { return n >= 16 && n <= 96; }
 __host__ __device__ constexpr int x_rows(int n, int cs) { return cmin(cmax(8192 / (n / 2 * cs), 1), 16); }
 template <typename T, int N>
 struct ZPlan { static constexpr CPlan P = fplan<T>(N, 8, small64(N) ? 4 : 8); };
@@ -151,13 +155,19 @@ struct XPlan {
 
 // Tile shapes of size N.  V selects compiled alternatives for the autotuner, one bit per
 // kernel family: bit 0 the pencil width TX, bit 1 the inverse-y width TYI, bit 3 the forward-y
-// width TY (V = 0: the defaults).
+// width TY (V = 0: the defaults).  Bit 2: a single grid of N <= 64, whose launches put one or two
+// blocks of a few warps on an SM and last for as long as one thread's loads and stages follow one
+// another: the pencil may take every register and loads the state before the first transform
+// (pencil_tile, EARLY), the x rows take twice the threads of their products for the stages, which
+// have more lines than that.  A step at 48^3 FP32 64.0 us (70.6 without, 66.7 with the kernels that
+// staged every tile), 24^3 47.3 (52.6, 56.6); 24^3 FP64 164 (177).
 template <typename T, int N, int V = 0>
 struct K2Cfg {
   static constexpr int M = N / 2;
   static constexpr int CS = (int)sizeof(cpx<T>);
   static constexpr int MINW = 32 / CS;  // 32-byte global segments
   static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr bool FEW = (V & 4) && N <= 64;  // bit 2
   // pencil: TX columns of N, three tiles in shared memory, one thread per column and first-stage
   // butterfly (radix f); registers hold 3 f modes
   static constexpr int ZF = ZPlan<T, N>::P.r[0], ZNB = N / ZF;
@@ -170,13 +180,13 @@ struct K2Cfg {
   // small grids whose N / 8 threads per column are not whole warps), kept as it was recorded with
   static constexpr int EDX = pick_div(M, cmax(16384 / (N * CS), MINW), 16);
   static constexpr int EDZ = F32 && N >= 24 ? round_lines(EDX * N / 8, EDX) / EDX : ZNB;
-  // blocks per SM the register budget must allow (variant bit 16: one more)
-  static constexpr int PREGS = F32 ? 128 : 168;
+  // blocks per SM the register budget must allow
+  static constexpr int PREGS = FEW ? 255 : F32 ? 128 : 168;
   static constexpr int p_blocks(int regs) {
     return cmax(1, cmin(cmin(16, 65536 / (NTP * regs)), (227 * 1024) / (p_elems * CS + 1024)));
   }
   static constexpr int MINB_P = p_blocks(PREGS);
-  static constexpr int MINB_P2 = p_blocks(F32 ? 168 : 255);  // two inputs and outputs
+  static constexpr int MINB_P2 = p_blocks(F32 && !FEW ? 168 : 255);  // two inputs and outputs
   // y passes: tiles of TYI / TY columns, three in shared memory, one thread per column and
   // last-stage butterfly
   static constexpr CPlan YP = YPlan<T, N>::P;
@@ -194,7 +204,7 @@ struct K2Cfg {
   static constexpr int MINB_Y = y_blocks(TY, YFREGS);
   // x rows: tiles of RX rows in pairs (q, q + RXH), whose third products share a line; N / f
   // threads per row.  Two-stage plans whose threads of some pairs make one warp run warp by warp
-  // (XWP pairs each), without block barriers.
+  // (XWP pairs each), without block barriers; the others take twice the threads when FEW.
   static constexpr CPlan XP = XPlan<T, N>::P;
   static constexpr int XF0 = XP.r[0], XNB = N / XF0;
   static constexpr int RXT = x_rows(N, CS);
@@ -204,7 +214,7 @@ struct K2Cfg {
   static constexpr int RX = RX0, RXH = (RX0 + 1) / 2;
   static constexpr int XWP = XWARP ? 32 / (2 * XNB) : RXH;       // pairs of a group
   static constexpr int XNG = XWARP ? RXH / XWP : 1;              // groups of a tile
-  static constexpr int XGT = XWARP ? 32 : (2 * RXH * XNB + 31) / 32 * 32;  // threads of a group
+  static constexpr int XGT = XWARP ? 32 : (2 * RXH * XNB * (FEW ? 2 : 1) + 31) / 32 * 32;  // threads of a group
   static constexpr int NTX = XNG * XGT;
   static constexpr int XGEL = Xchg<T, N, XF0, 6 * XWP, false>::elems;
   static constexpr int XELEMS = XNG * XGEL + 32;                 // and the scratch of the block's maxima
@@ -448,6 +458,8 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
   const bool act = tid < NT;
   const size_t gj = ((size_t)j * N + iy) * M + kx;  // element (kz index j, iy, kx) of a field
   constexpr size_t ZS = (size_t)N * M;              // one plane
+  // the state is loaded first, in one piece, where registers hold it beside the transforms' values
+  constexpr bool EARLY = C::FEW && f * sizeof(cpx<T>) <= 64 && NFC == 1 && MC >= 0 && MC != MODE_NL && MC != MODE_PROJECT;
   const bool tt = pencil_tile_truncated<T, TX>(a, x0, ky);  // N = 0 on the whole tile
   // the state vanishes there too: nothing to do (NL and PROJECT write their zeros)
   if (tt && a.cut && mode != MODE_NL && mode != MODE_PROJECT &&
@@ -470,6 +482,13 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
 
   const bool rd0 = mode != MODE_NL && mode != MODE_PROJECT;
   const cpx<T>* base0 = (mode == MODE_INIT ? a.src : (mode == MODE_RK4_4 ? a.acc : a.state)) + gj;
+  cpx<T> s0e[3][f];
+  if constexpr (EARLY)
+    if (act)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int r = 0; r < f; ++r) s0e[c][r] = MP::ldw(base0 + c * fstride + r * NB0 * ZS);
 
   // 1) forward z transforms of the inputs: de-shifted by e^{-i k.delta} and weighted (products in
   //    one fixed rounding order, as the compiler may contract them differently in each instance)
@@ -571,17 +590,33 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
       ehxy = a.ifac[N + kx] * a.ifac[N + iy];
     }
     const bool rd1 = mode == MODE_RK4_2 || mode == MODE_RK4_3;
-    constexpr int CHK = f % 4 == 0 ? 4 : (f % 3 == 0 ? 3 : 2);  // modes whose state loads are in flight
+    // modes whose loads are in flight together (the stores of a chunk hold back the next one's)
+    constexpr int CHK = EARLY ? f : f % 4 == 0 ? 4 : (f % 3 == 0 ? 3 : 2);
 #pragma unroll
     for (int r0 = 0; r0 < f; r0 += CHK) {
-      cpx<T> s0[3][CHK];
+      cpx<T> s0[3][CHK], s1[3][CHK];
 #pragma unroll
       for (int i = 0; i < CHK; ++i)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          s0[c][i] = mk<T>(0, 0);
-          if (rd0) s0[c][i] = MP::ldw(base0 + c * fstride + (r0 + i) * NB0 * ZS);
+          s0[c][i] = s1[c][i] = mk<T>(0, 0);
+          if constexpr (EARLY) s0[c][i] = s0e[c][r0 + i];
+          else if (rd0) s0[c][i] = MP::ldw(base0 + c * fstride + (r0 + i) * NB0 * ZS);
+          if (rd1) s1[c][i] = MP::ldw(&a.acc[c * fstride + gj + (r0 + i) * NB0 * ZS]);
         }
+      T e1z[CHK], ehz[CHK];
+      cpx<T> oz[CHK];
+#pragma unroll
+      for (int i = 0; i < CHK; ++i) {
+        const int iz = j + (r0 + i) * NB0;
+        e1z[i] = ehz[i] = 1;
+        if (useE) {
+          e1z[i] = a.ifac[iz];
+          ehz[i] = a.ifac[N + iz];
+        }
+        oz[i] = mk<T>(1, 0);
+        if (pre) oz[i] = MP::ld(&a.osh[0][2 * N + iz]);
+      }
 #pragma unroll
       for (int i = 0; i < CHK; ++i) {
         const int r = r0 + i, iz = j + r * NB0, kz = kof(iz, N);
@@ -590,16 +625,15 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
         if (nFe > 0) project_point(a, kx, ky, kz, nv);
         T E1 = 1, Eh = 1;
         if (useE) {
-          E1 = e1xy * a.ifac[iz];
-          Eh = ehxy * a.ifac[N + iz];
+          E1 = e1xy * e1z[i];
+          Eh = ehxy * ehz[i];
         }
         cpx<T> shz = oxy;
-        if (pre) shz = cmul_fixed(oxy, MP::ld(&a.osh[0][2 * N + iz]));
+        if (pre) shz = cmul_fixed(oxy, oz[i]);
         T m2 = 0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const cpx<T> s1 = rd1 ? MP::ldw(&a.acc[c * fstride + g]) : mk<T>(0, 0);
-          cpx<T> sn = stage_combine<T, MP>(a, c, c * fstride + g, nv[c], s0[c][i], s1, E1, Eh, mode);
+          cpx<T> sn = stage_combine<T, MP>(a, c, c * fstride + g, nv[c], s0[c][i], s1[c][i], E1, Eh, mode);
           shell_record<T, MP>(a, c, kx, ky, kz, sn);
           if (ep) m2 += sn.x * sn.x + sn.y * sn.y;
           nz = nz || sn.x != T(0) || sn.y != T(0);
@@ -1318,29 +1352,30 @@ __host__ __device__ constexpr bool k2_has_alt() { return sizeof(T) == 4 && N >= 
 
 template <typename T, int N>
 K2Entry<T> make_k2_entry() {
-  using C = K2Cfg<T, N>;
+  constexpr int FV = N <= 64 ? 4 : 0;  // (a single grid: FEW)
+  using C = K2Cfg<T, N, FV>;
   K2Entry<T> e;
   e.N = N;
-  e.pencil01 = k2_pencil<T, N, 0, 1, false, MODE_INIT>;
-  e.pencil10[0] = k2_pencil<T, N, 1, 0, false, MODE_NL>;
-  e.pencil10[1] = k2_pencil<T, N, 1, 0, false, MODE_PROJECT>;
-  e.pencil1[MODE_RK2_1] = k2_pencil<T, N, 1, 1, false, MODE_RK2_1>;
-  e.pencil1[MODE_RK2_2] = k2_pencil<T, N, 1, 1, false, MODE_RK2_2>;
-  e.pencil1[MODE_RK4_1] = k2_pencil<T, N, 1, 1, false, MODE_RK4_1>;
-  e.pencil1[MODE_RK4_2] = k2_pencil<T, N, 1, 1, false, MODE_RK4_2>;
-  e.pencil1[MODE_RK4_3] = k2_pencil<T, N, 1, 1, false, MODE_RK4_3>;
-  e.pencil1[MODE_RK4_4] = k2_pencil<T, N, 1, 1, false, MODE_RK4_4>;
-  e.pencil1[MODE_ROG_1] = k2_pencil<T, N, 1, 1, false, MODE_ROG_1>;
-  e.pencil1[MODE_ROG_2] = k2_pencil<T, N, 1, 1, false, MODE_ROG_2>;
-  e.pencil1e[MODE_RK2_2] = k2_pencil<T, N, 1, 1, true, MODE_RK2_2>;
-  e.pencil1e[MODE_RK4_4] = k2_pencil<T, N, 1, 1, true, MODE_RK4_4>;
-  e.pencil1e[MODE_ROG_2] = k2_pencil<T, N, 1, 1, true, MODE_ROG_2>;
-  e.pencil2[0] = k2_pencil<T, N, 2, 2, false, MODE_RK2_1>;
-  e.pencil2[1] = k2_pencil<T, N, 2, 2, false, MODE_RK2_2>;
-  e.pencil02 = k2_pencil<T, N, 0, 2, false, MODE_INIT>;
+  e.pencil01 = k2_pencil<T, N, 0, 1, false, MODE_INIT, FV>;
+  e.pencil10[0] = k2_pencil<T, N, 1, 0, false, MODE_NL, FV>;
+  e.pencil10[1] = k2_pencil<T, N, 1, 0, false, MODE_PROJECT, FV>;
+  e.pencil1[MODE_RK2_1] = k2_pencil<T, N, 1, 1, false, MODE_RK2_1, FV>;
+  e.pencil1[MODE_RK2_2] = k2_pencil<T, N, 1, 1, false, MODE_RK2_2, FV>;
+  e.pencil1[MODE_RK4_1] = k2_pencil<T, N, 1, 1, false, MODE_RK4_1, FV>;
+  e.pencil1[MODE_RK4_2] = k2_pencil<T, N, 1, 1, false, MODE_RK4_2, FV>;
+  e.pencil1[MODE_RK4_3] = k2_pencil<T, N, 1, 1, false, MODE_RK4_3, FV>;
+  e.pencil1[MODE_RK4_4] = k2_pencil<T, N, 1, 1, false, MODE_RK4_4, FV>;
+  e.pencil1[MODE_ROG_1] = k2_pencil<T, N, 1, 1, false, MODE_ROG_1, FV>;
+  e.pencil1[MODE_ROG_2] = k2_pencil<T, N, 1, 1, false, MODE_ROG_2, FV>;
+  e.pencil1e[MODE_RK2_2] = k2_pencil<T, N, 1, 1, true, MODE_RK2_2, FV>;
+  e.pencil1e[MODE_RK4_4] = k2_pencil<T, N, 1, 1, true, MODE_RK4_4, FV>;
+  e.pencil1e[MODE_ROG_2] = k2_pencil<T, N, 1, 1, true, MODE_ROG_2, FV>;
+  e.pencil2[0] = k2_pencil<T, N, 2, 2, false, MODE_RK2_1, FV>;
+  e.pencil2[1] = k2_pencil<T, N, 2, 2, false, MODE_RK2_2, FV>;
+  e.pencil02 = k2_pencil<T, N, 0, 2, false, MODE_INIT, FV>;
   e.yinv = k2_yinv<T, N>;
   e.yfwd = k2_yfwd<T, N>;
-  e.xrow = k2_xrow<T, N>;
+  e.xrow = k2_xrow<T, N, FV>;
   if constexpr (ClCfg<T, N>::ok) {
     e.slabcl[0] = k2_slabcl<T, N, 384>;
     e.slabcl[1] = k2_slabcl<T, N, 768>;
