@@ -484,7 +484,6 @@ struct Solver : SolverBase {
     red_blocks = 2 * nsm;
     CUDA_TRY(cudaMalloc(&red, (size_t)red_blocks * 1024 * sizeof(double)));
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
-    decide_cut();
     CUDA_TRY(cudaMalloc(&d_cut, 4 * sizeof(int)));
     const int one[4] = {1, 1, 1, 1};
     CUDA_TRY(cudaMemcpyAsync(d_cut, one, sizeof(one), cudaMemcpyHostToDevice, st));
@@ -579,20 +578,12 @@ struct Solver : SolverBase {
     return k;
   }
   // Whether columns are left out at all (with the launch that looks at the state, where needed): from
-  // 20 MB of state on when a quarter of the columns goes, from 40 MB on always.  Below, the fields stay
-  // in L2 and the launches are short.  Measured, steps with all columns and without, us: FP32 96^3
-  // (11 MB) 397 and 401 at C_t = 1, 380 and 381 at 2/3; 128^3 (25 MB) 619 and 625 at 1, 592 and 573 at
-  // 0.8, 590 and 470 at 2/3; 192^3 (85 MB) 2200 and 2110 at 1; FP64 96^3 (21 MB) 6179 and 6190 at 1,
-  // 5381 and 5091 at 2/3; 128^3 (50 MB) 10467 and 10310 at 1.
-  bool cut_pays = false;
-  void decide_cut() {
-    const size_t bytes = 3 * F1 * sizeof(cpx<T>);
-    size_t kept = 0;
-    for (int iy = 0; iy < N; ++iy)
-      for (int k = 0; k < M && column_kept(c->p.truncation, c->K2max, c->Kimax, -1, k, iy < M ? iy : iy - N); ++k) ++kept;
-    cut_pays = use2 && (bytes >= 40000000 || (bytes >= 20000000 && 4 * kept <= 3 * (size_t)N * M));
-  }
-  bool cut_on() const { return cut_pays && !clus; }
+  // 20 MB of state on.  Below, the fields stay in L2 and the launches are short.  Measured, steps with
+  // all columns and without, us: FP32 96^3 (11 MB) 397 and 401 at C_t = 1, 380 and 381 at 2/3; 128^3
+  // (25 MB) 619 and 625 at 1 (three grids at once: 808 and 788), 592 and 573 at 0.8, 590 and 470 at 2/3;
+  // 192^3 (85 MB) 2200 and 2110 at 1; FP64 64^3 (6 MB) 2318 and 2333 at 2/3; 96^3 (21 MB) 5381 and
+  // 5091 at 2/3.
+  bool cut_on() const { return use2 && !clus && 3 * F1 * sizeof(cpx<T>) >= 20000000; }
   void cut_check() {
     cut_mix = cut_cur;
     if (!cut_on() || (cut_cur && !state_shared)) return;
