@@ -115,10 +115,15 @@ __host__ __device__ constexpr int x_rows(int per, int n, int line_bytes) {
 }
 
 // columns of a tile of `per` threads per column: 64-byte rows (128 bytes for an interleaved pair),
-// fewer where that makes more than `lim` threads or, on small grids, fewer than 152 blocks
-__host__ __device__ constexpr int y_cols(int n, int per, int minw, int lim) {
-  int w = pick_div(n / 2, 2 * minw, 16);
-  while (w > minw && w % 2 == 0 && (w * per > lim || (n / 2 / w * n < 152 && w / 2 * per >= 32))) w /= 2;
+// fewer where that makes more than `lim` threads or, on small grids, fewer than a block for each of the
+// 152 SMs; twice as many where that fills the warps and leaves 128 blocks (a step of 48^3 FP64 217 us
+// with 8 columns, 96 threads, and 234 with 4).  wide (single FP32 grids of N <= 64): 128-byte rows, however
+// few the blocks (fewer, fuller warps; a step at 24^3 48.0 us and 52.3 with 6 columns in the y passes, 32^3 51.1 and
+// 52.5; at 48^3 with two other grids stepping 26.9 and 28.3, at 64^3 29.0 and 30.2).
+__host__ __device__ constexpr int y_cols(int n, int per, int minw, int lim, bool wide) {
+  int w = pick_div(n / 2, (wide ? 4 : 2) * minw, 16);
+  while (w > minw && w % 2 == 0 && (w * per > lim || (!wide && n / 2 / w * n < 152 && w / 2 * per >= 32))) w /= 2;
+  if (!wide && w * per % 32 && 2 * w * per % 32 == 0 && n / 2 % (2 * w) == 0 && n / (4 * w) * n >= 128) w *= 2;
   return w;
 }
 
@@ -171,15 +176,18 @@ struct K2Cfg {
   // pencil: TX columns of N, three tiles in shared memory, one thread per column and first-stage
   // butterfly (radix f); registers hold 3 f modes
   static constexpr int ZF = ZPlan<T, N>::P.r[0], ZNB = N / ZF;
-  static constexpr int TX0 = y_cols(N, ZNB, MINW, 512);
+  // FP32 energy sums: the grouping of the modes that one thread adds in FP32 (N / 8, except on the
+  // small grids whose N / 8 threads per column are not whole warps), kept as it was recorded with;
+  // a wide tile needs a thread for each of its groups (not so at N = 24)
+  static constexpr int EDX = pick_div(M, cmax(16384 / (N * CS), MINW), 16);
+  static constexpr int EDZ = F32 && N >= 24 ? round_lines(EDX * N / 8, EDX) / EDX : ZNB;
+  static constexpr int TXW = y_cols(N, ZNB, MINW, 512, true);
+  static constexpr bool ZWIDE = FEW && F32 && (EDZ == ZNB || TXW * EDZ <= (TXW * ZNB + 31) / 32 * 32);
+  static constexpr int TX0 = ZWIDE ? TXW : y_cols(N, ZNB, MINW, 512, false);
   static constexpr int TX = (V & 1) ? alt_width(TX0, M, 512 / ZNB, MINW) : TX0;
   static constexpr int NTP = (TX * ZNB + 31) / 32 * 32;  // (whole warps: the energy sums shuffle)
   static constexpr int PTS = Xchg<T, N, ZF, TX, true>::elems;
   static constexpr int p_elems = 3 * PTS + tw_elems(N);
-  // FP32 energy sums: the grouping of the modes that one thread adds in FP32 (N / 8, except on the
-  // small grids whose N / 8 threads per column are not whole warps), kept as it was recorded with
-  static constexpr int EDX = pick_div(M, cmax(16384 / (N * CS), MINW), 16);
-  static constexpr int EDZ = F32 && N >= 24 ? round_lines(EDX * N / 8, EDX) / EDX : ZNB;
   // blocks per SM the register budget must allow
   static constexpr int PREGS = FEW ? 255 : F32 ? 128 : 168;
   static constexpr int p_blocks(int regs) {
@@ -191,7 +199,7 @@ struct K2Cfg {
   // last-stage butterfly
   static constexpr CPlan YP = YPlan<T, N>::P;
   static constexpr int YNB = N / YP.r[0];
-  static constexpr int TY0 = y_cols(N, YNB, MINW, 192), TYI0 = TY0;
+  static constexpr int TY0 = y_cols(N, YNB, MINW, 192, FEW && F32), TYI0 = TY0;
   static constexpr int TY = (V & 8) ? alt_width(TY0, M, 512 / YNB, MINW) : TY0;
   static constexpr int TYI = (V & 2) ? alt_width(TYI0, M, 512 / YNB, MINW) : TYI0;
   static constexpr int NTY = TY * YNB, NTYI = TYI * YNB;
@@ -1373,8 +1381,8 @@ K2Entry<T> make_k2_entry() {
   e.pencil2[0] = k2_pencil<T, N, 2, 2, false, MODE_RK2_1, FV>;
   e.pencil2[1] = k2_pencil<T, N, 2, 2, false, MODE_RK2_2, FV>;
   e.pencil02 = k2_pencil<T, N, 0, 2, false, MODE_INIT, FV>;
-  e.yinv = k2_yinv<T, N>;
-  e.yfwd = k2_yfwd<T, N>;
+  e.yinv = k2_yinv<T, N, FV>;
+  e.yfwd = k2_yfwd<T, N, FV>;
   e.xrow = k2_xrow<T, N, FV>;
   if constexpr (ClCfg<T, N>::ok) {
     e.slabcl[0] = k2_slabcl<T, N, 384>;
