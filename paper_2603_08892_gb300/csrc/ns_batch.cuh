@@ -27,6 +27,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -77,16 +78,27 @@ struct BatchCtl {
   int gran;         // tiles per ticket
 };
 
+// Tile variant (K2Cfg) of the persistent kernel's items: y tiles of twice the columns for the FP32
+// classes of 96^3 and 128^3, which set the block (192 threads, two of them on an SM) and would leave
+// two thirds of it idle in those passes.  64 members, 16 each of 32, 64, 96 and 128, ten steps, 1 / 4
+// tiles a ticket: 101 / 90 ms, 121 / 107 with the single grids' tiles, 139 / 135 with those, the pencil's
+// mode looked up at run time and one block size for every ensemble.  Smaller classes: 16 members of
+// 48^3, four steps, 1.65 ms as they are, 2.26 with wide y tiles.
+template <typename T, int N>
+constexpr int kPV = sizeof(T) == 4 && N >= 96 ? 10 : 0;
+template <typename T, int N>
+using PCfg = K2Cfg<T, N, kPV<T, N>>;
+
 template <typename T>
 struct BCfg {
   template <int N>
   static constexpr int nt() {
-    using C = K2Cfg<T, N>;
+    using C = PCfg<T, N>;
     return cmax(cmax(C::NTP, C::NTYI), cmax(C::NTY, C::NTX));
   }
   template <int N>
   static constexpr size_t sm() {
-    using C = K2Cfg<T, N>;
+    using C = PCfg<T, N>;
     const size_t cs = sizeof(cpx<T>);
     const size_t tw = (size_t)tw_elems(N);
     const size_t p = (size_t)C::p_elems * cs;
@@ -103,6 +115,15 @@ struct BCfg {
   static constexpr size_t SM_c = sm<96>() > sm<128>() ? sm<96>() : sm<128>();
   static constexpr size_t SM_ab = SM_a > SM_b ? SM_a : SM_b;
   static constexpr size_t SM = SM_ab > SM_c ? SM_ab : SM_c;
+  // threads and shared memory of the items of size class z
+  static int threads(int z) {
+    constexpr int t[kNumSizes] = {nt<16>(), nt<32>(), nt<48>(), nt<64>(), nt<96>(), nt<128>()};
+    return (t[z] + 31) / 32 * 32;
+  }
+  static size_t smem(int z) {
+    constexpr size_t t[kNumSizes] = {sm<16>(), sm<32>(), sm<48>(), sm<64>(), sm<96>(), sm<128>()};
+    return t[z];
+  }
 };
 
 
@@ -164,7 +185,7 @@ __device__ __forceinline__ PencilArgs<T> batch_pencil_args(const BatchMem<T>& bm
 template <typename T, int N>
 __device__ __noinline__ void run_item(const BatchMem<T>& bm, int pass, int step, int nsteps,
                                       int tile, cpx<T>* smem) {
-  using C = K2Cfg<T, N>;
+  using C = PCfg<T, N>;
   constexpr int M = N / 2;
   if (pass == P_TAB) {
     batch_tab<T, N>(bm, step, nsteps);
@@ -176,7 +197,7 @@ __device__ __noinline__ void run_item(const BatchMem<T>& bm, int pass, int step,
     return;
   }
   if (pass == P_X1 || pass == P_X2) {
-    xrow_tile<T, N, MemCG>(bm.sa, tile, smem);
+    xrow_tile<T, N, MemCG, kPV<T, N>>(bm.sa, tile, smem);
     return;
   }
   if (pass == P_F1 || pass == P_F2) {
@@ -184,8 +205,14 @@ __device__ __noinline__ void run_item(const BatchMem<T>& bm, int pass, int step,
     yfwd_tile<T, N, MemCG, C::TY>(bm.sa, tile % ntx, tile / ntx, smem);
     return;
   }
-  // pencil passes: INIT (pass < 0), P1, P2
-  pencil_tile<T, N, MemCG>(batch_pencil_args(bm, pass, step, nsteps), tile, smem);
+  // pencil passes: INIT (pass < 0), P1, P2 (without an output in the last step)
+  const PencilArgs<T> a = batch_pencil_args(bm, pass, step, nsteps);
+  if (pass < 0)
+    pencil_tile<T, N, MemCG, 0, 1, false, MODE_INIT, kPV<T, N>>(a, tile, smem);
+  else if (pass == P_P1)
+    pencil_tile<T, N, MemCG, 1, 1, false, MODE_ROG_1, kPV<T, N>>(a, tile, smem);
+  else
+    pencil_tile<T, N, MemCG, 1, -1, false, MODE_ROG_2, kPV<T, N>>(a, tile, smem);
 }
 
 template <typename T>
@@ -311,7 +338,7 @@ __global__ void __launch_bounds__(K2Cfg<T, N>::NTY, K2Cfg<T, N>::MINB_Y) k_bgrid
 
 template <typename T, int N>
 void member_items(int* items, int* pro_init) {
-  using C = K2Cfg<T, N>;
+  using C = PCfg<T, N>;
   constexpr int M = N / 2;
   const int pen = (M / C::TX) * N, yi = (M / C::TYI) * N, yf = (M / C::TY) * N;
   const int xr = (N * N + C::RX - 1) / C::RX;
@@ -490,7 +517,8 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
     s.N = N; s.M = M; s.z0 = 0; s.G = N; s.tw = (const cpx<T>*)cb.tw; s.mixed = (const cpx<T>*)cb.mixed;
     s.scr = (cpx<T>*)cb.scr; s.Ft = (cpx<T>*)cb.Ft; s.xmode = XMODE_NONLINEAR; s.pairs = 1;
     s.skip = 1; s.trunc = cb.truncation; s.K2max = cb.K2max; s.Kimax = cb.Kimax; s.fK = -1; s.cut = a.cut;
-    while (s.kxn < M && column_kept(s.trunc, s.K2max, s.Kimax, -1, s.kxn, 0)) ++s.kxn; s.err = (int*)cb.err;
+    while (s.kxn < M && column_kept(s.trunc, s.K2max, s.Kimax, -1, s.kxn, 0)) ++s.kxn;
+    s.err = (int*)cb.err;
     if (cb.G < N) return NS_ERR_INTERNAL;
     items_for<T>(N, bm.items, &bm.pro_init);
     bm.cum[0] = 0;
@@ -612,13 +640,20 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
   c.abort = b->d_flags + 1;
   c.mem_off = b->d_off;
   c.pro_mem_off = b->d_off + kPasses * (kMaxMembers + 1);
-  const size_t smem = BCfg<T>::SM;
+  // the block and its shared memory are those of the widest item of the sizes present: narrower
+  // blocks leave an SM room for more of them
+  int nt = 0;
+  size_t smem = 0;
+  for (int m = 0; m < n; ++m) {
+    nt = std::max(nt, BCfg<T>::threads(hm[m].sz));
+    smem = std::max(smem, BCfg<T>::smem(hm[m].sz));
+  }
   if (!chk(cudaFuncSetAttribute(k_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
     return NS_ERR_CUDA;
   int per_sm = 0, nsm = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch<T>, BCfg<T>::NT, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch<T>, nt, smem);
   if (per_sm < 1) per_sm = 1;
   if (b->per_sm_req > 0 && b->per_sm_req < per_sm) per_sm = b->per_sm_req;
   const int grid = nsm * per_sm;
@@ -637,7 +672,7 @@ int batch_step_t(ns_batch* b, const double* dt, int nsteps) {
       cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long), st);
       cudaMemsetAsync(b->d_done, 0, n * sizeof(int), st);
       cudaMemsetAsync(b->d_flags, 0, 2 * sizeof(int), st);
-      k_batch<T><<<grid, BCfg<T>::NT, smem, st>>>(c, dm);
+      k_batch<T><<<grid, nt, smem, st>>>(c, dm);
       ok = chk(cudaStreamEndCapture(st, &g));
     }
     if (ok) {

@@ -437,13 +437,11 @@ __device__ __forceinline__ void tile_energy_store(double* epart, T e, T d) {
   }
 }
 
-// NFC, NOC: the number of inputs and outputs known at compile time; -1: at run time, at most
-// one of each (the persistent ensemble: the mode is looked up for every mode then, 17 -> 30 us
-// per RK4 stage of 48^3).  (1, 1) is every RK2, Rogallo and RK4 stage, (2, 2) and
-// (0, 2) the exact scheme's, (0, 1) INIT, (1, 0) NL and PROJECT.  MC: the stage mode at compile time (-1: a.mode).
+// NFC, NOC: the number of inputs and outputs (NOC -1: a.nOut, at most one: the persistent ensemble's
+// last pass, which has an output but in the last step); MC: the stage mode.  (1, 1) is every RK2,
+// Rogallo and RK4 stage, (2, 2) and (0, 2) the exact scheme's, (0, 1) INIT, (1, 0) NL and PROJECT.
 // EP: the tile's energy sums are stored (NOC = 2: whenever a.epart is set).
-template <typename T, int N, class MP, int NFC = -1, int NOC = -1, bool EP = false, int MC = -1,
-          int V = 0>
+template <typename T, int N, class MP, int NFC, int NOC, bool EP, int MC, int V = 0>
 __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id, cpx<T>* buf) {
   using C = K2Cfg<T, N, V>;
   using PL = ZPlan<T, N>;
@@ -454,8 +452,8 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
   using X = Xchg<T, N, f, TX, true>;
   static_assert(NT <= C::NTP, "one first-stage butterfly per thread");
   constexpr int ED = C::EDZ;  // the energy sums add a column's modes iz = i (mod ED) in T, then in FP64
-  const int nF = NFC >= 0 ? NFC : a.nF, nOut = NOC >= 0 ? NOC : a.nOut;
-  const int mode = MC >= 0 ? MC : a.mode;
+  const int nF = NFC, nOut = NOC >= 0 ? NOC : a.nOut;
+  constexpr int mode = MC;
   cpx<T>* tws = buf + 3 * TS;
   constexpr int ntx = M / TX;
   const int iy = a.iy0 + tile_id / ntx;  // (iy0: first ky row of a rank-range launch)
@@ -467,7 +465,7 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
   const size_t gj = ((size_t)j * N + iy) * M + kx;  // element (kz index j, iy, kx) of a field
   constexpr size_t ZS = (size_t)N * M;              // one plane
   // the state is loaded first, in one piece, where registers hold it beside the transforms' values
-  constexpr bool EARLY = C::FEW && f * sizeof(cpx<T>) <= 64 && NFC == 1 && MC >= 0 && MC != MODE_NL && MC != MODE_PROJECT;
+  constexpr bool EARLY = C::FEW && f * sizeof(cpx<T>) <= 64 && NFC == 1 && MC != MODE_NL && MC != MODE_PROJECT;
   const bool tt = pencil_tile_truncated<T, TX>(a, x0, ky);  // N = 0 on the whole tile
   // the state vanishes there too: nothing to do (NL and PROJECT write their zeros)
   if (tt && a.cut && mode != MODE_NL && mode != MODE_PROJECT &&
@@ -754,8 +752,8 @@ __device__ __forceinline__ void pencil_tile(const PencilArgs<T>& a, int tile_id,
 }
 
 // EP: the one-input variant that also stores the tile's energy sums (a.epart non-null)
-// MC: the stage mode at compile time (the Rogallo stages) or -1 (a.mode); V: tile variant
-template <typename T, int N, int NFC, int NOC, bool EP = false, int MC = -1, int V = 0>
+// MC: the stage mode; V: tile variant
+template <typename T, int N, int NFC, int NOC, bool EP, int MC, int V = 0>
 __global__ void __launch_bounds__(K2Cfg<T, N, V>::NTP, NFC == 2 ? K2Cfg<T, N, V>::MINB_P2 : K2Cfg<T, N, V>::MINB_P)
     k2_pencil(PencilArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
