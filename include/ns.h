@@ -279,9 +279,10 @@ int ns_batch_grid(ns_batch* b);
 /* Schedule: gran tiles per work-list ticket of the persistent launch (the ticket, the
  * bounded wait and the completion fence are paid once per gran tiles) and ctas_per_sm CTAs
  * per SM (0: as many as fit); gran 0 selects the grid schedule (ctas_per_sm unused).  The
- * first ns_batch_step tunes both on the ensemble (each candidate times one step; the
- * members' states, times and step counters are saved before and restored after) unless
- * ns_batch_set_schedule was called, NS_BATCH_SCHEDULE="g,q" is set or NS_AUTOTUNE=0.
+ * first ns_batch_step tunes both on the ensemble (each candidate times up to two steps after
+ * as many untimed ones; the members' states, times and step counters are saved before and
+ * restored after) unless ns_batch_set_schedule was called, NS_BATCH_SCHEDULE="g,q" is set or
+ * NS_AUTOTUNE=0.
  * Results do not depend on the schedule.  NS_ERR_INVALID_ARG for gran < 0 or ctas_per_sm < 0. */
 int ns_batch_set_schedule(ns_batch* b, int gran, int ctas_per_sm);
 int ns_batch_schedule(ns_batch* b, int* gran, int* ctas_per_sm);

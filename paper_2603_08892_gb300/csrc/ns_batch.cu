@@ -16,14 +16,17 @@ int batch_step_any(ns_batch* b, const double* dt, int nsteps) {
   return b->precision == NS_FP32 ? batch_step_t<float>(b, dt, nsteps) : ns_batch_step_f64(b, dt, nsteps);
 }
 
-// Schedule tuner of the persistent launch: the work-list granularity (tiles per ticket) and
-// the CTAs per SM are timed on this ensemble, four steps per candidate after an untimed call (the
-// time of a single step is mostly that of the call, which favours the one launch of the persistent
-// schedule: six members of 64^3 take 157 us per step with it and 75 with grid launches);
-// the members' states, times and step counters are saved before and restored after, so the
-// tuning leaves the simulation unchanged.  NS_BATCH_SCHEDULE="gran,ctas_per_sm" forces a
+// Schedule tuner: the grid schedule, and the persistent launch with its work-list granularity
+// (tiles per ticket) and CTAs per SM, are timed on this ensemble over two steps (one, where the call
+// has no more: the time of a single step is mostly that of the call, which favours the one launch of
+// the persistent schedule), each after an untimed call of as many, so that its graph exists when it is
+// timed.  A candidate whose untimed call takes more than twice the best time (and 1 ms, for what a
+// first call does once) is not timed, and when the plain persistent launch is one, its other forms are
+// not tried.  First call of 64 members (16 each of 32, 64, 96, 128 FP32), ten steps: 70 ms, 197 with
+// four timed steps of every candidate.  The members' states, times and step counters are saved before and restored
+// after, so the tuning leaves the simulation unchanged.  NS_BATCH_SCHEDULE="gran,ctas_per_sm" forces a
 // schedule; NS_AUTOTUNE=0 keeps the default (1 tile per ticket, as many CTAs as fit).
-int batch_tune(ns_batch* b, const double* dt) {
+int batch_tune(ns_batch* b, const double* dt, int nsteps) {
   b->tuned = true;
   if (const char* f = std::getenv("NS_BATCH_SCHEDULE")) {
     int g = 1, q = 0;
@@ -71,27 +74,35 @@ int batch_tune(ns_batch* b, const double* dt) {
     else
       maxq = ns_batch_max_ctas_f64();  // (the FP64 kernel lives in its own translation unit)
   }
-  for (int g : {0, 1, 4}) {  // 0: the grid schedule (one launch per pass and size class)
-    for (int q : {0, 1}) {
-      if (q == 1 && (maxq <= 1 || g != 1)) continue;
-      b->gran = g;
-      b->per_sm_req = q;
-      rc = batch_step_any(b, dt, 1);  // untimed (graph capture)
-      if (rc != NS_OK) break;
-      cudaEventRecord(e0, b->st);
-      rc = batch_step_any(b, dt, 4);
-      cudaEventRecord(e1, b->st);
-      if (rc != NS_OK) break;
-      cudaEventSynchronize(e1);
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (ms < best) {
-        best = ms;
-        bg = g;
-        bq = q;
-      }
-    }
+  const int nt = nsteps < 2 ? nsteps : 2;
+  auto timed = [&](int steps, float* ms) {  // one call, from an idle stream
+    cudaEventRecord(e0, b->st);
+    const int r = batch_step_any(b, dt, steps);
+    cudaEventRecord(e1, b->st);
+    if (r != NS_OK) return r;
+    cudaEventSynchronize(e1);
+    *ms = 0.f;
+    cudaEventElapsedTime(ms, e0, e1);
+    return r;
+  };
+  const int cand[4][2] = {{0, 0}, {1, 0}, {1, 1}, {4, 0}};  // gran 0: the grid schedule (one launch per pass and size class)
+  for (int i = 0; i < 4 && rc == NS_OK; ++i) {
+    if (cand[i][1] == 1 && maxq <= 1) continue;
+    b->gran = cand[i][0];
+    b->per_sm_req = cand[i][1];
+    float first = 0.f, ms = 0.f;
+    rc = timed(b->gran == 0 ? 1 : nt, &first);  // (the grid schedule has no graph)
     if (rc != NS_OK) break;
+    if (i > 0 && first > 2.f * best + 1.f) {
+      if (i == 1) break;
+      continue;
+    }
+    rc = timed(nt, &ms);
+    if (rc == NS_OK && ms < best) {
+      best = ms;
+      bg = cand[i][0];
+      bq = cand[i][1];
+    }
   }
   for (int m = 0; m < n; ++m) {
     cudaMemcpyAsync(cb[m].state, save + off[m], bytes[m], cudaMemcpyDeviceToDevice, b->st);
@@ -206,7 +217,7 @@ int ns_batch_step(ns_batch* b, const double* dt, int nsteps) {
   for (int i = 0; i < b->count; ++i)
     if (!(dt[i] > 0.0) || !std::isfinite(dt[i])) return NS_ERR_INVALID_ARG;
   if (!b->tuned) {
-    const int rc = batch_tune(b, dt);
+    const int rc = batch_tune(b, dt, nsteps);
     if (rc != NS_OK) return rc;
   }
   return batch_step_any(b, dt, nsteps);
