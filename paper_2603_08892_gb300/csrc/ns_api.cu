@@ -1074,8 +1074,8 @@ struct Solver : SolverBase {
 
   // ---- autotuner of the plane-group size of the slab pass ------------------------------
   // Candidates G (planes per group of the scratch) with one or two streams are timed on the
-  // slab pass with CUDA events; the fastest is kept and cached in a JSON file keyed by device,
-  // N, precision and the slab tiles.  Results do not depend on G or on the streams (every
+  // slab pass of a truncated state with CUDA events; the fastest is kept and cached in a JSON file keyed
+  // by device, N, precision, the slab tiles and the share of the columns that is kept.  Results do not depend on G or on the streams (every
   // plane is transformed the same way).  NS_AUTOTUNE=0 disables it; NS_AUTOTUNE_CACHE sets the
   // cache file; NS_SLAB_PLANES=g forces a group size, NS_SLAB_STREAMS=1|2 the stream count,
   // NS_SLAB_PIPE=1 the pipeline (ring NS_PIPE_RING, lag NS_PIPE_LAG) and =0 excludes it;
@@ -1096,6 +1096,12 @@ struct Solver : SolverBase {
     if (use2)  // the slab kernels' tiles and thread counts: a change of kernels re-tunes
       k += "|" + std::to_string(k2.TYI) + "," + std::to_string(k2.NTYI) + "," + std::to_string(k2.TY) +
            "," + std::to_string(k2.NTY) + "," + std::to_string(k2.RX) + "," + std::to_string(k2.NTX);
+    if (cut_on()) {  // the work of a pass goes with the columns that are kept: their share, in sixteenths
+      size_t kept = 0;
+      for (int iy = 0; iy < N; ++iy)
+        for (int k = 0; k < M && column_kept(c->p.truncation, c->K2max, c->Kimax, -1, k, iy < M ? iy : iy - N); ++k) ++kept;
+      k += "|k" + std::to_string((16 * kept + (size_t)N * M / 2) / ((size_t)N * M));
+    }
     for (auto& ch : k)
       if (ch == '"' || ch == '\\') ch = '_';
     return k;
@@ -1209,7 +1215,7 @@ struct Solver : SolverBase {
     if (Gmax <= 1 || N < 128) return;  // small grids: one group holds every plane
     const bool can_alt = use2 && k2.has_alt && !(fv && *fv);
     const std::string path = cache_path(),
-                      key = tune_key() + (can_pipe ? "|g5p" : "|g5") + (can_cl ? "c" + std::to_string(k2.CLS) : "") +
+                      key = tune_key() + (can_pipe ? "|g6p" : "|g6") + (can_cl ? "c" + std::to_string(k2.CLS) : "") +
                             (can_alt ? "|v" + std::to_string(k2.alt.TX) + "," + std::to_string(k2.alt.TYI) + "," +
                                            std::to_string(k2.alt.TY)
                                      : "");
@@ -1235,22 +1241,52 @@ struct Solver : SolverBase {
       for (int v = 0; v < 2; ++v) cand.push_back({1 + v, 3});
     if (cand.empty()) return;
     CUDA_TRY(cudaMemsetAsync(mixed[0], 0, 5 * F1 * sizeof(cpx<T>), st));
+    CUDA_TRY(cudaMemsetAsync(acc, 0, 3 * F1 * sizeof(cpx<T>), st));
+    CUDA_TRY(cudaMemsetAsync(Ft[0], 0, 3 * F1 * sizeof(cpx<T>), st));
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
     const bool pon = prof.on;
     prof.on = false;
-    float best = 1e30f;
-    std::pair<int, int> bestc = {G, 0};
-    for (const auto& cm : cand) {
-      set_mode(cm.first, cm.second);
-      slab(mixed[0], Ft[0]);  // warm-up
+    // ms of 8 passes after an untimed one, on zero fields and under the flag of a truncated state
+    auto time8 = [&](auto&& pass) {
+      pass(0);
       CUDA_TRY(cudaEventRecord(e0, st));
-      for (int r = 0; r < 8; ++r) slab(mixed[0], Ft[0]);
+      for (int r = 0; r < 8; ++r) pass(r);
       CUDA_TRY(cudaEventRecord(e1, st));
       CUDA_TRY(cudaEventSynchronize(e1));
       float ms = 0;
       CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
+      return ms;
+    };
+    auto time_slab = [&]() { return time8([&](int) { slab(mixed[0], Ft[0], false, cut_clean()); }); };
+    // both Rogallo stages on the work buffers (acc as the state, Ft[0] as the input, mixed[0] as the
+    // output; all recomputed before any step uses them)
+    auto time_pencil = [&]() {
+      return time8([&](int r) {
+        PencilArgs<T> a = pencil_args((r & 1) ? MODE_ROG_2 : MODE_ROG_1);
+        a.shell = nullptr;
+        a.state = acc;
+        a.nF = 1; a.F[0] = Ft[0]; a.wF[0] = (T)1;
+        a.nOut = 1; a.out[0] = mixed[0];
+        a.cut = cut_clean();
+        pencil(a);
+      });
+    };
+    // the cluster pass keeps the fields apart and every column: the pencil is slower beside it, so
+    // where it is a candidate the pencil counts (as many pencil as slab passes a step)
+    float pencil_ms[2] = {0.f, 0.f};
+    if (can_cl) {
+      set_mode(cand[0].first, cand[0].second);
+      pencil_ms[0] = time_pencil();
+      set_mode(1, 3);
+      pencil_ms[1] = time_pencil();
+    }
+    float best = 1e30f;
+    std::pair<int, int> bestc = {G, 0};
+    for (const auto& cm : cand) {
+      set_mode(cm.first, cm.second);
+      const float ms = time_slab() + pencil_ms[clus];
       if (ms < best) {
         best = ms;
         bestc = cm;
@@ -1263,16 +1299,6 @@ struct Solver : SolverBase {
     // the compiled tile alternatives, one kernel family at a time: the slab kernels in the
     // chosen slab mode (three-kernel modes only), the pencil on the Rogallo stages
     if (can_alt) {
-      auto time_slab = [&]() {
-        slab(mixed[0], Ft[0]);
-        CUDA_TRY(cudaEventRecord(e0, st));
-        for (int r = 0; r < 8; ++r) slab(mixed[0], Ft[0]);
-        CUDA_TRY(cudaEventRecord(e1, st));
-        CUDA_TRY(cudaEventSynchronize(e1));
-        float ms = 0;
-        CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-        return ms;
-      };
       if (!pipe && !clus) {
         float base = time_slab();
         for (int bit : {2, 8}) {
@@ -1282,29 +1308,6 @@ struct Solver : SolverBase {
           else vsel ^= bit;
         }
       }
-      // pencil: both Rogallo stages on the work buffers (acc as the state, Ft[0] as the input,
-      // mixed[0] as the output; all recomputed before any step uses them), zero inputs
-      CUDA_TRY(cudaMemsetAsync(acc, 0, 3 * F1 * sizeof(cpx<T>), st));
-      CUDA_TRY(cudaMemsetAsync(Ft[0], 0, 3 * F1 * sizeof(cpx<T>), st));
-      cpx<T>* pout = mixed[0];
-      auto time_pencil = [&]() {
-        PencilArgs<T> a = pencil_args(MODE_ROG_1);
-        a.shell = nullptr;
-        a.state = acc;
-        a.nF = 1; a.F[0] = Ft[0]; a.wF[0] = (T)1;
-        a.nOut = 1; a.out[0] = pout;
-        pencil(a);
-        CUDA_TRY(cudaEventRecord(e0, st));
-        for (int r = 0; r < 8; ++r) {
-          a.mode = (r & 1) ? MODE_ROG_2 : MODE_ROG_1;
-          pencil(a);
-        }
-        CUDA_TRY(cudaEventRecord(e1, st));
-        CUDA_TRY(cudaEventSynchronize(e1));
-        float ms = 0;
-        CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-        return ms;
-      };
       const float pbest = time_pencil();
       vsel ^= 1;
       if (!(time_pencil() < pbest)) vsel ^= 1;
