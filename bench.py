@@ -9,8 +9,9 @@ Workload (timed `--steps` steps, one JSON line on rank 0):
   that t = 9 lands on a step, shifts from splitmix64 seed 12345.
   Comparison leg: RK4 + 2/3 spherical truncation at 384^3 (kmax = 128, same dt rule).
 
-Per step the state (201 MB) and the moved data (2.95 GB by the two-pass byte model) are
-larger than the 129 MB L2, so no L2 flush is needed between steps.
+Per step the state (201 MB) and the moved data (2.33 GB by the two-pass byte model, in the
+columns inside the truncation) are larger than the 129 MB L2, so no L2 flush is needed
+between steps.
 
 --impl reference times the FP64 CPU oracle on the host cores on the same workload (a
 bounded number of whole steps).  Under torchrun (N > 1) every rank runs an independent
@@ -84,7 +85,7 @@ def peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("ns_fft.cuh", "ns_kernels.cuh", "ns_fft2.cuh", "ns_kernels2.cuh"):
+    for f in ("ns_fft.cuh", "ns_kernels.cuh", "ns_fft2.cuh", "ns_fft3.cuh", "ns_kernels2.cuh"):
         with open(os.path.join(ROOT, "paper_2603_08892_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -100,6 +101,15 @@ def ncu_traffic(kernel):
         return d["kernels"][kernel]["dram_bytes_per_launch_full_size"]
     except Exception:
         return None
+
+
+def kept_columns(N, kmax):
+    """Share of the (kx, ky) columns that hold modes of the spherical truncation |k| < kmax: the
+    passes of a truncated state read and write no others."""
+    kept = 0
+    for ky in range(-(N // 2), N // 2):
+        kept += sum(1 for kx in range(N // 2) if kx * kx + ky * ky < kmax * kmax)
+    return kept / (N * (N // 2))
 
 
 class Clocks:
@@ -451,7 +461,6 @@ def main():
     barrier(world)
 
     C = N_PS ** 3 * 4.0
-    model_bytes = s.model_bytes_per_step()
     value = world * K / (ms_max / 1000.0)
     ms_step = ms_max / K
     hbm, peak_kind = peaks()
@@ -460,13 +469,16 @@ def main():
     # kernels per plane group (y inverse, x rows, y forward) whose algorithmic traffic is the
     # 5 mixed fields read (5C) and the 3 transformed products written (3C), 8C per pass; its
     # scratch is an implementation choice (L2 or HBM by group size) and shows in the measured
-    # ncu traffic, not in the model.
+    # ncu traffic, not in the model.  Both in the columns inside the truncation, the only ones
+    # that the passes touch (0.789 of them at kmax = N/2).
+    kept = kept_columns(N_PS, KMAX)
+    model_bytes = s.model_bytes_per_step() * kept
     nchunks = (K + 255) // 256
     # every pencil pass of a step reads Ft and the state and writes the state and the mixed
     # fields of the next evaluation (the last one prepares the next step): 14C per launch
     units = {
-        "k_pencil": (14.0 * C, prof["k_pencil"][0], prof["k_pencil"][1]),
-        "slab_pass": (8.0 * C, prof["slab_pass"][0], prof["slab_pass"][1]),
+        "k_pencil": (14.0 * C * kept, prof["k_pencil"][0], prof["k_pencil"][1]),
+        "slab_pass": (8.0 * C * kept, prof["slab_pass"][0], prof["slab_pass"][1]),
     }
     roof_units = {}
     for name, (nbytes, tot_ms, n) in units.items():
@@ -498,7 +510,7 @@ def main():
             "units": roof_units, "pass_ms_per_step": pass_ms, "pass_time_shares": pass_shares,
             "kernel_event_ms_per_step_overlapping": kernel_ms,
             "slab_groups_per_pass": prof["k_yinv"][2] / max(1, prof["slab_pass"][2]),
-            "step_model_bytes": model_bytes,
+            "kept_columns": kept, "step_model_bytes": model_bytes,
             "step_frac": (model_bytes / (ms_step / 1000.0) / 1e9) / hbm}
 
     # secondary roofline: FP32 CUDA-core arithmetic, 130 N^3 log2 N flop per RK2-family step
@@ -519,7 +531,7 @@ def main():
         "data": "synthetic (Taylor-Green initial field, Eq. T-G-init; no dataset)",
         "config": {"workload": WORKLOAD, "N": N_PS, "kmax": KMAX, "nu": NU, "dt": dt,
                    "parallelism": "replicas" if world > 1 else "single GPU",
-                   "l2": "no flush: state 201 MB and 2.95 GB moved per step exceed the 129 MB L2"},
+                   "l2": "no flush: state 201 MB and 2.33 GB moved per step exceed the 129 MB L2"},
         "gcells_per_s": value * N_PS ** 3 / 1e9,
         "sim_time_per_s": value * dt / world,
         "energy_at_end": E, "dissipation_at_end": eps,
@@ -537,7 +549,7 @@ def main():
         Kr = max(3, args.rk4_steps)
         ms4 = reduce_max(timed_steps(ns, r, dt4, Kr, stream), world)
         rate4 = world * Kr / (ms4 / 1000.0)
-        mb4 = r.model_bytes_per_step()
+        mb4 = r.model_bytes_per_step() * kept_columns(N_RK4, KMAX)
         line["rk4_two_thirds"] = {
             "N": N_RK4, "kmax": KMAX, "dt": dt4, "steps": Kr, "steps_per_s": rate4,
             "gcells_per_s": rate4 * N_RK4 ** 3 / 1e9, "sim_time_per_s": rate4 * dt4 / world,
@@ -573,14 +585,14 @@ def main():
         msb = reduce_max(e0.elapsed_time(e1), world)
         Eb, _ = b.energy()
         gran, qsm = b.schedule()
-        model = sum(44.0 * n ** 3 * 4.0 for n in Ns)
+        model = sum(44.0 * n ** 3 * 4.0 * kept_columns(n, n / 2.0) for n in Ns)
         line["batched_ensemble"] = {
             "members": len(Ns), "sizes": "16 x {32, 64, 96, 128}", "steps": Kb,
             "member_steps_per_s": world * len(Ns) * Kb / (msb / 1000.0),
             "ensemble_steps_per_s": world * Kb / (msb / 1000.0), "ms_per_step": msb / Kb,
             "schedule": {"kind": "grid" if gran == 0 else "persistent", "tiles_per_ticket": gran,
                          "ctas_per_sm": qsm},
-            "launches_per_call": 4 * (2 + 9 * Kb) if gran == 0 else 1,
+            "launches_per_call": 1 + (4 * (2 + 9 * Kb) if gran == 0 else 1),
             "persistent_ctas": b.grid() if gran != 0 else None,
             "gcells_per_s": world * sum(n ** 3 for n in Ns) * Kb / (msb / 1000.0) / 1e9,
             "model_bytes_per_step": model,
