@@ -98,9 +98,9 @@ struct DFT<T, 9> {
 };
 
 // ---- radix plans ------------------------------------------------------------------------
-// The plans list their radices in descending order: the first stage's butterflies are the
-// widest, so the set of f elements j + (N/f) r of one of them is also what K = f / l butterflies
-// of the last stage (radix l, where l divides f) hold together: p = j + (N/f) i, i < K, element
+// No radix of a plan exceeds the first (f).  Where the last one (l) divides it, as in every plan of
+// radix_plan (those of cplan need not: 8.2.3 at 48), the set of f elements j + (N/f) r of a first-stage
+// butterfly is also what K = f / l last-stage butterflies hold together: p = j + (N/f) i, i < K, element
 // p + (N/l) r = j + (N/f) (i + K r).  A thread that runs those K butterflies at the end of one
 // transform has in registers what the first stage of the next one (same plan) reads.
 constexpr int kRadices[] = {16, 12, 9, 8, 6, 4, 3, 2};
@@ -136,7 +136,7 @@ __host__ __device__ constexpr CPlan radix_plan(int n, int cap) {
 }
 // FP32 transforms of 24 points and more keep the plans of cplan (radix cap mr), so that results
 // recorded in FP64 from FP32 runs (energies, spectra, fields) stay the same to the last bit;
-// FP64 ones, whose arithmetic bounds them, take the plan with the fewest stages.
+// FP64 ones, whose arithmetic bounds them, take the plan with the fewest stages of radices <= cap64.
 template <typename T>
 __host__ __device__ constexpr CPlan fplan(int n, int mr, int cap64) {
   return sizeof(T) == 4 && n >= 24 ? cplan(n, mr) : radix_plan(n, sizeof(T) == 4 ? 8 : cap64);

@@ -202,9 +202,9 @@ __device__ __forceinline__ cpx<T> phase3(const cpx<T>* tab, int N, int ix, int i
 
 // Run-time sizes: one block per ky row and TX columns.  The z transforms' first stages read global
 // memory (or form the shifted values) and their last ones write it: only the stages between them
-// go through shared memory.  216^3 FP32, one in and one out: 394 us a launch, 834 before.  A step of 216^3 (all
-// run-time kernels): 6180 us with run-time divisions, six-tile y passes and 15 values a thread, 3240
-// now; issue-bound (index arithmetic, radix-8 and radix-3 stages).
+// go through shared memory.  Bound by issue (index arithmetic, radix-8 and radix-3 stages).  216^3 FP32,
+// one in and one out: 394 us a launch, 834 with the tiles loaded and stored whole; a step 3240 us, 6180
+// with that, run-time divisions, six-tile y passes and 15 values a thread.
 template <typename T>
 __global__ void __launch_bounds__(384, sizeof(T) == 4 ? 2 : 1) k_pencil(const __grid_constant__ PencilArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -425,8 +425,8 @@ __device__ void block_max3(T m0, T m1, T m2, T* scratch, void* umax) {
 // Inverse y transforms of one field per block: the velocity, or omega = i k x u formed from the
 // mixed fields as they are read.  grid (M/TY, G, fields).  One field per block reads some mixed
 // fields twice (from L2) and needs one tile of shared memory instead of six, so that enough blocks
-// are resident to cover the loads: 216^3 FP32, per 100 planes: 160 us, 400 to 435 before (8 warps an SM).  The
-// products are fused in writing: the compiler merges the branches' subtractions otherwise.
+// are resident to cover the loads: 216^3 FP32, per 100 planes: 160 us, 400 to 435 with six tiles (8 warps
+// an SM).  The products are fused in writing: the compiler merges the branches' subtractions otherwise.
 template <typename T>
 __global__ void __launch_bounds__(384, sizeof(T) == 4 ? 2 : 1) k_yinv(const __grid_constant__ SlabArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

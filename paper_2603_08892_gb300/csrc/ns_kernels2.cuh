@@ -4,10 +4,10 @@
 // for the data layout): k2_pencil = z transforms + spectral stage of Sec. 4 / 6.1,
 // k2_yinv / k2_xrow / k2_yfwd = slab pass (y transforms, x rows with u x omega), and
 // k2_slabpipe = the slab pass as one persistent pipelined launch.  What changes is how the
-// transforms run: tiles are staged with cp.async, the first FFT stage reads the staged tile
-// or global memory and the last one writes global memory or applies the spectral factors,
-// every index is a compile-time expression, and the butterflies are radix 8 or 16 in
-// registers (per kernel, K2Cfg).
+// transforms run: the first stage's inputs and the last stage's outputs are in registers, which
+// global memory or a pointwise operation fills and takes (ns_fft3.cuh), the stages between them go
+// through shared memory, every index is a compile-time expression, and the butterflies are of
+// radix 2 to 16 (per kernel and size, K2Cfg).
 #pragma once
 
 #include "ns_fft3.cuh"
@@ -103,15 +103,6 @@ struct MemCG {
 // the half length m within the cap, else half (down to minw), else the default.
 __host__ __device__ constexpr int alt_width(int w, int m, int cap, int minw) {
   return (m % (2 * w) == 0 && 2 * w <= cap) ? 2 * w : ((w / 2 >= minw && m % (w / 2) == 0) ? w / 2 : w);
-}
-
-// rows of an x-row tile of `per` threads per row: the smallest even number that gives at least
-// 128 threads (64 up to N = 64, where blocks are few), halved while three lines per row pass 52 KB
-__host__ __device__ constexpr int x_rows(int per, int n, int line_bytes) {
-  int r = 2;
-  while (r * per < (n <= 64 ? 64 : 128)) r += 2;
-  while (r % 4 == 0 && 3 * r * line_bytes > 52 * 1024) r /= 2;
-  return r;
 }
 
 // columns of a tile of `per` threads per column: 64-byte rows (128 bytes for an interleaved pair),
