@@ -578,12 +578,12 @@ struct Solver : SolverBase {
     return k;
   }
   // Whether columns are left out at all (with the launch that looks at the state, where needed): from
-  // 20 MB of state on.  Below, the fields stay in L2 and the launches are short.  Measured, steps with
-  // all columns and without, us: FP32 96^3 (11 MB) 397 and 401 at C_t = 1, 380 and 381 at 2/3; 128^3
-  // (25 MB) 619 and 625 at 1 (three grids at once: 808 and 788), 592 and 573 at 0.8, 590 and 470 at 2/3;
-  // 192^3 (85 MB) 2200 and 2110 at 1; FP64 64^3 (6 MB) 2318 and 2333 at 2/3; 96^3 (21 MB) 5381 and
-  // 5091 at 2/3.
-  bool cut_on() const { return use2 && !clus && 3 * F1 * sizeof(cpx<T>) >= 20000000; }
+  // 5 MB of state on.  Below, the fields stay in L2 even with several grids stepping, and the launches
+  // are short.  Measured, two steps from a shared state, us, with all columns and without, one grid and
+  // three at once: 64^3 FP32 (3 MB) 147 and 153, 57.9 and 58.4 at C_t = 0.6; 48^3 FP64 (3 MB) 442 and 449,
+  // 304 and 305 at 1; 64^3 FP64 (6 MB) 698 and 693, 486 and 434 at 0.6, 777 and 784, 583 and 578 at 1;
+  // 96^3 FP32 (11 MB) 206 and 201, 127 and 104 at 0.6, 207 and 218, 140 and 139 at 1.
+  bool cut_on() const { return use2 && !clus && 3 * F1 * sizeof(cpx<T>) >= 5000000; }
   void cut_check() {
     cut_mix = cut_cur;
     if (!cut_on() || (cut_cur && !state_shared)) return;

@@ -1,4 +1,4 @@
-"""Column skipping where it is used (from 20 MB of state on), FP32 as well as FP64.
+"""Column skipping where it is used (from 5 MB of state on), FP32 as well as FP64.
 
 The state is looked at only where something may have written it, once per look; and steps of states
 with modes outside the truncation, among them states written through the device address between two
